@@ -410,9 +410,10 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
 
   // With 0 < K0 < K, one tensor-core pass over V after the first R0 tokens gives every
   // candidate its exact value on their basis (and ||v||^2); otherwise values start from
-  // p_hat * ||v||^lambda.  The first K0c <= min(128, S) tokens of R0 are factored before the pass;
-  // the rest of R0 is retained in the rounds after it, as forced picks, and every
-  // value the pass gave stays a valid upper bound (values only shrink as the basis grows).
+  // p_hat * ||v||^lambda.  The first K0c <= min(kCholMax, S) tokens of R0 are factored before the
+  // pass, which takes their first 128 basis vectors; the rest of R0 is retained in the rounds after
+  // it, as forced picks.  Where the basis has more vectors than the pass took, every value it gave
+  // stays a valid upper bound (values only shrink as the basis grows).
   const int K0c = std::min({K0, mapk::kCholMax, S});
   const bool project = K0 > 0 && K0 < K;
   if (K0 < K && !project) {

@@ -13,8 +13,8 @@
 // <v_i, v_j>, computed on the tensor cores in blocks.
 //   R0     : the first K0 picks (top-K0 by p_hat) are forced, in p_hat order; their basis is
 //            the Cholesky factor of G[R0, R0] (sel_chol_kernel).  A tensor-core projection
-//            of every token on that basis (gemm_tc.cu) then gives every candidate its exact
-//            value.
+//            of every token on that basis (gemm_tc.cu; its first 128 vectors) then gives every
+//            candidate its exact value (or a bound).
 // Later picks proceed in rounds:
 //   choose : active set A = the s candidates with the largest value bound U (a stale
 //            value, or p_hat * ||v||^lambda for tokens never evaluated; values only shrink
@@ -66,6 +66,23 @@ __device__ __forceinline__ float sel_value(float p, float r2, float sq, float la
   if (!(r2 > tau * sq) || !(r2 > 0.f)) return 0.f;
   const float v = lam == 1.f ? (p * p) * r2 : (p * p) * powf(r2, lam);
   return v > 0.f ? v : 0.f;
+}
+
+// 1 / sqrt(x), x > 0: the hardware estimate (2 ulp) and one Newton step (below 1 ulp, like the
+// quotient of a rounded root), without the branches of an IEEE root and division.
+__device__ __forceinline__ float inv_sqrt(float x) {
+  const float y = rsqrtf(x), t = x * y;
+  return x < INFINITY ? fmaf(0.5f * y, fmaf(-t, y, 1.0f), y) : 0.f;
+}
+
+// Two fp32 fused multiply-adds in one instruction (the halves of a 64-bit register pair).
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float sum2(uint64_t a) {
+  return __uint_as_float(static_cast<uint32_t>(a)) + __uint_as_float(static_cast<uint32_t>(a >> 32));
 }
 
 // k-th largest of n distinct 64-bit keys in shared memory (1 <= k <= n): MSB-first radix
@@ -491,81 +508,199 @@ __global__ void __launch_bounds__(kUpdSlots * kUpdWarps, 1) sel_update_kernel(Se
 
 // ------------------------------------------------------------------ R0 basis
 // The K0 forced picks (R0 in p_hat order) need no argmax: their basis is the Cholesky factor
-// of the K0 x K0 Gram matrix G[R0, R0], column by column in pick order (right-looking, in
-// shared memory).  Column t adds basis vector nb unless its residual is degenerate
-// (r^2 <= tau ||v||^2); its entries below the diagonal are the later R0 tokens' coordinates
-// e_nb.  Writes picks, state, basis, Ec rows, cstep and r2 of the R0 tokens.
-constexpr int kCholThreads = kCholMax;
+// of the K0 x K0 Gram matrix G[R0, R0] in pick order.  Column t adds a basis vector unless its
+// residual is degenerate (r^2 <= tau ||v||^2: the column is zero and is dropped when the
+// coordinates are written); its entries below the diagonal are the later R0 tokens'
+// coordinates.  Writes picks, state, basis, Ec rows, cstep and r2 of the R0 tokens.
+//
+// Blocked, 32 columns (a panel) at a time, so that only the 32 x 32 diagonal block is a
+// sequential chain, and that one stays inside a warp (a barrier and a whole dot product per
+// column made up nearly all of the column-by-column form's time):
+//   1. the panel less its products with the columns before it, a register-tiled matrix product;
+//   2. the diagonal block by warp 0, lane = row, the row in registers, shuffles for the others';
+//   3. the rows below it, a thread per row, by forward substitution against the block.
+// One image, K0 = 80: 35.4 -> 23.0 us; 16 images, K0 = 202: 70.5 us for 128 columns and a forced
+// round for the rest -> 77.6 us for all of them (ncu, cold).
+// In shared memory, rows of panel b hold 32 (b + 1) columns and 4 of padding: eight consecutive
+// rows read 16 bytes each from 32 different banks.
+constexpr int kCholThreads = 256;
+static_assert(kCholMax <= kCholThreads && kCholMax % 32 == 0, "a thread per R0 token");
 
-// Left-looking, one thread per R0 position u, G[R0, R0] and the coordinate rows in shared
-// memory; one block barrier per basis vector.
+// First float of row u in the panel-wise lower triangle.
+__host__ __device__ inline int chol_row(int u) {
+  const int p = u / 32;
+  return 32 * (16 * p * (p + 1) + 4 * p) + (u - 32 * p) * (32 * (p + 1) + 4);
+}
+
 __global__ void __launch_bounds__(kCholThreads, 1) sel_chol_kernel(SelState s) {
   pdl_enter();
-  extern __shared__ __align__(16) float shc[];
-  __shared__ float r2s[kCholMax], dg[kCholMax], dpick[kCholMax], ps[kCholMax];
-  __shared__ int tk[kCholMax], mine_s[kCholMax], bidx[kCholMax];
-  const int b = blockIdx.x;
-  const int K0 = s.K0, ldg = (K0 + 3) & ~3, PL = coord_pitch(K0);
-  float* Gs = shc;                                   // [K0][ldg]
-  float* Ls = shc + K0 * ldg;                        // [K0][PL] coordinates, zeros past the valid ones
+  extern __shared__ __align__(16) float A[];           // G, then L, in place
+  // the diagonal block's columns: LT[t][j] = L[c0 + j][c0 + t], zero for j <= t and past 31
+  __shared__ __align__(16) float LT[32][56];
+  __shared__ float rinv_s[32];                         // 1 / r of its columns, 0: no basis vector
+  __shared__ float dg[kCholMax], dpick[kCholMax];
+  __shared__ int tk[kCholMax], mine_s[kCholMax], ext_s[kCholMax];
+  const int b = blockIdx.x, K0 = s.K0;
+  const int npan = (K0 + 31) / 32;
   const long long base = static_cast<long long>(b) * s.N;
   const float* Gb = s.G + static_cast<long long>(b) * s.S * s.R;
-  {
-    const int v4 = ldg / 4;                          // G rows are 16-byte aligned (R % 16 == 0)
-    for (int i = threadIdx.x; i < K0 * v4; i += blockDim.x) {
-      const int r = i / v4, c = (i - r * v4) * 4;
-      cp_async16(Gs + r * ldg + c, Gb + static_cast<long long>(r) * s.R + c);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int r = warp; r < 32 * npan; r += kCholThreads / 32) {
+    float* row = A + chol_row(r);
+    const int w4 = 8 * (r / 32 + 1);                   // G rows are 16-byte aligned (R % 16 == 0)
+    for (int c = lane; c < w4; c += 32) {
+      // columns past K0 (rows too) are zero: they never extend the basis
+      if (r < K0 && 4 * c + 4 <= K0) cp_async16(row + 4 * c, Gb + static_cast<long long>(r) * s.R + 4 * c);
+      else
+        for (int k = 0; k < 4; ++k)
+          row[4 * c + k] = r < K0 && 4 * c + k < K0 ? Gb[static_cast<long long>(r) * s.R + 4 * c + k] : 0.f;
     }
   }
-  for (int i = threadIdx.x; i < K0 * PL / 4; i += blockDim.x)
-    reinterpret_cast<float4*>(Ls)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-  cp_async_wait_all();
+  for (int i = threadIdx.x; i < 32 * 24; i += kCholThreads) LT[i / 24][32 + i % 24] = 0.f;
   const int u = threadIdx.x;
+  float pscore = 0.f;
   if (u < K0) {
     tk[u] = s.r0[static_cast<long long>(b) * s.K + u];
-    ps[u] = s.scores[base + tk[u]];
+    pscore = sel_scores(s)[base + tk[u]];
   }
+  cp_async_wait_all();
   __syncthreads();
-  float r2 = 0.f;
-  if (u < K0) {
-    r2 = Gs[u * ldg + u];
-    r2s[u] = r2;
-    dg[u] = r2;
-  }
+  if (u < K0) dg[u] = A[chol_row(u) + u];
+  else if (u < kCholMax) dg[u] = 0.f;
   __syncthreads();
-  float* me = Ls + u * PL;
-  int nb = 0;
-  for (int t = 0; t < K0; ++t) {
-    const float d = r2s[t], sq = dg[t];
-    const bool ext = d > s.tau * sq && d > 0.f;
-    if (u == t) {                                         // global writes wait for the end
-      mine_s[t] = nb;
-      dpick[t] = d;
-      bidx[t] = ext ? nb : -1;
-    }
-    if (!ext) continue;                                   // uniform
-    if (u > t && u < K0) {
-      const float* lt = Ls + t * PL;
-      const float rinv = 1.0f / sqrtf(d), gut = Gs[u * ldg + t];   // independent of the dot product
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 4
-      for (int q = 0; q < nb; q += 4) {                   // rows are zero past nb
-        const float4 x = *reinterpret_cast<const float4*>(lt + q);
-        const float4 y = *reinterpret_cast<const float4*>(me + q);
-        a0 = fmaf(x.x, y.x, a0);
-        a1 = fmaf(x.y, y.y, a1);
-        a2 = fmaf(x.z, y.z, a2);
-        a3 = fmaf(x.w, y.w, a3);
+  int nb = 0;                                          // basis vectors so far (warp 0)
+  const int cg = threadIdx.x & 7, rg = threadIdx.x >> 3;   // products: columns cg + 8 k, row rg of each panel
+  for (int pan = 0; pan < npan; ++pan) {
+    const int c0 = 32 * pan;
+    if (c0 > 0) {
+      const float* lc[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) lc[k] = A + chol_row(c0 + cg + 8 * k);
+      for (int i0 = pan; i0 < npan; i0 += 4) {         // up to four row panels at a time
+        float* lr[4];
+        float acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          lr[i] = A + chol_row(32 * min(i0 + i, npan - 1) + rg);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) acc[i][k] = 0.f;
+        }
+        for (int q = 0; q < c0; q += 4) {
+          float4 y[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) y[k] = *reinterpret_cast<const float4*>(lc[k] + q);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (i0 + i < npan) {                       // uniform
+              const float4 x = *reinterpret_cast<const float4*>(lr[i] + q);
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                float v = acc[i][k];
+                v = fmaf(x.x, y[k].x, v);
+                v = fmaf(x.y, y[k].y, v);
+                v = fmaf(x.z, y[k].z, v);
+                acc[i][k] = fmaf(x.w, y[k].w, v);
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (i0 + i < npan) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) lr[i][c0 + cg + 8 * k] -= acc[i][k];
+          }
       }
-      const float e = (gut - ((a0 + a1) + (a2 + a3))) * rinv;
-      me[nb] = e;
-      r2 = fmaf(-e, e, r2);
-      r2s[u] = r2;
+      __syncthreads();
+    }
+    if (warp == 0) {                                   // the diagonal block
+      // eight columns per pass, then the row shifts down by eight: the loop's code stays small
+      float a[32];
+      float* row = A + chol_row(c0 + lane) + c0;
+#pragma unroll
+      for (int j = 0; j < 32; j += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(row + j);
+        a[j] = v.x; a[j + 1] = v.y; a[j + 2] = v.z; a[j + 3] = v.w;
+      }
+      const float floor2 = s.tau * dg[c0 + lane];
+      float mydiag = 0.f;
+      bool myext = false;
+#pragma unroll 1
+      for (int t0 = 0; t0 < 32; t0 += 8) {
+        float ev[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const bool me = lane == t0 + t;
+          const float d = __shfl_sync(0xffffffffu, a[t], t0 + t);
+          const float fl = __shfl_sync(0xffffffffu, floor2, t0 + t);
+          const bool ext = d > fl && d > 0.f;
+          const float rinv = ext ? inv_sqrt(d) : 0.f;
+          const float e = ext && lane > t0 + t ? a[t] * rinv : 0.f;
+          if (me) { mydiag = d; myext = ext; rinv_s[t0 + t] = rinv; }
+          ev[t] = e;
+          LT[t0 + t][lane] = e;
+          const int done = t < 7 ? t + 1 : t;          // columns up to here are up to date
+          if (t < 7) a[t + 1] = fmaf(-e, __shfl_sync(0xffffffffu, e, t0 + t + 1), a[t + 1]);   // the next pivot column
+          __syncwarp();
+#pragma unroll
+          for (int j = (done + 1) & ~3; j < 32; j += 4) {   // zero at and before column t, and past 31
+            const float4 l = *reinterpret_cast<const float4*>(&LT[t0 + t][t0 + j]);
+            if (j > done) a[j] = fmaf(-e, l.x, a[j]);
+            if (j + 1 > done) a[j + 1] = fmaf(-e, l.y, a[j + 1]);
+            if (j + 2 > done) a[j + 2] = fmaf(-e, l.z, a[j + 2]);
+            if (j + 3 > done) a[j + 3] = fmaf(-e, l.w, a[j + 3]);
+          }
+        }
+        *reinterpret_cast<float4*>(row + t0) = make_float4(ev[0], ev[1], ev[2], ev[3]);
+        *reinterpret_cast<float4*>(row + t0 + 4) = make_float4(ev[4], ev[5], ev[6], ev[7]);
+#pragma unroll
+        for (int j = 0; j < 24; ++j) a[j] = a[j + 8];
+#pragma unroll
+        for (int j = 24; j < 32; ++j) a[j] = 0.f;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, myext);
+      dpick[c0 + lane] = mydiag;
+      ext_s[c0 + lane] = myext;
+      mine_s[c0 + lane] = nb + __popc(m & ((1u << lane) - 1u));
+      nb += __popc(m);
     }
     __syncthreads();
-    ++nb;
+    const int r = c0 + 32 + threadIdx.x;               // the rows below
+    if (r < K0) {
+      float x[32];
+      float* row = A + chol_row(r) + c0;
+#pragma unroll
+      for (int j = 0; j < 32; j += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(row + j);
+        x[j] = v.x; x[j + 1] = v.y; x[j + 2] = v.z; x[j + 3] = v.w;
+      }
+#pragma unroll 1
+      for (int t0 = 0; t0 < 32; t0 += 8) {
+        float ev[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+          const float ri = rinv_s[t0 + t];
+          const float e = ri != 0.f ? x[t] * ri : 0.f;
+          ev[t] = e;
+#pragma unroll
+          for (int j = (t + 1) & ~3; j < 32; j += 4) {
+            const float4 l = *reinterpret_cast<const float4*>(&LT[t0 + t][t0 + j]);
+            if (j > t) x[j] = fmaf(-e, l.x, x[j]);
+            if (j + 1 > t) x[j + 1] = fmaf(-e, l.y, x[j + 1]);
+            if (j + 2 > t) x[j + 2] = fmaf(-e, l.z, x[j + 2]);
+            if (j + 3 > t) x[j + 3] = fmaf(-e, l.w, x[j + 3]);
+          }
+        }
+        *reinterpret_cast<float4*>(row + t0) = make_float4(ev[0], ev[1], ev[2], ev[3]);
+        *reinterpret_cast<float4*>(row + t0 + 4) = make_float4(ev[4], ev[5], ev[6], ev[7]);
+#pragma unroll
+        for (int j = 0; j < 24; ++j) x[j] = x[j + 8];
+#pragma unroll
+        for (int j = 24; j < 32; ++j) x[j] = 0.f;
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
   if (u < K0) {
     const int tok = tk[u];
     const float d = dpick[u];
@@ -573,16 +708,18 @@ __global__ void __launch_bounds__(kCholThreads, 1) sel_chol_kernel(SelState s) {
     s.state[base + tok] = 1;
     s.cstep[base + tok] = mine_s[u];
     s.r2[base + tok] = d;
-    s.U[base + tok] = sel_value(ps[u], d, dg[u], s.lambda, s.tau);
-    if (bidx[u] >= 0) {
-      s.basis_tok[static_cast<long long>(b) * s.K + bidx[u]] = tok;
-      s.rnorm[static_cast<long long>(b) * s.K + bidx[u]] = sqrtf(d);
+    s.U[base + tok] = sel_value(pscore, d, dg[u], s.lambda, s.tau);
+    if (ext_s[u]) {
+      s.basis_tok[static_cast<long long>(b) * s.K + mine_s[u]] = tok;
+      s.rnorm[static_cast<long long>(b) * s.K + mine_s[u]] = sqrtf(d);
     }
   }
   // coordinate rows of the R0 tokens: e_beta for beta < (basis size at their pick)
-  for (int i = threadIdx.x; i < K0 * PL; i += blockDim.x) {
-    const int r = i / PL, q = i - r * PL;
-    if (q < mine_s[r]) s.Ec[(base + tk[r]) * s.KP + q] = Ls[r * PL + q];
+  for (int r = warp; r < K0; r += kCholThreads / 32) {
+    const float* row = A + chol_row(r);
+    float* g = s.Ec + (base + tk[r]) * s.KP;
+    for (int q = lane; q < r; q += 32)
+      if (ext_s[q]) g[mine_s[q]] = row[q];
   }
   if (threadIdx.x == 0) {
     s.nbasis[b] = nb;
@@ -596,9 +733,9 @@ __global__ void __launch_bounds__(kCholThreads, 1) sel_chol_kernel(SelState s) {
 // the active set is
 //   G'[i][k] = <v_i, v_k> - sum_{q < c0} e_q[i] e_q[k]   (the inner product of the residuals),
 // and a pick then needs only the coordinates added during the round (sel_greedy_kernel).
-// It replaces the A x A part of the Gram block in place.  One CTA of 64 threads per 32 x 32
-// tile of the upper triangle (the matrix is symmetric: the mirrored tile is written from the
-// same values), 4 x 4 outputs per thread; the coordinates are staged in 16-column chunks,
+// It replaces the lower triangle of the A x A part of the Gram block in place (the picks read
+// no more).  One CTA of 64 threads per 32 x 32 tile of the upper triangle, whose mirrored tile
+// it writes, 4 x 4 outputs per thread; the coordinates are staged in 16-column chunks,
 // transposed, in two shared buffers, the next chunk loaded during the products of the
 // current one.  Small tiles keep several CTAs on every SM, so the chunk loop's latency is
 // hidden, with few images (c0 is large) as with many.
@@ -682,8 +819,8 @@ __global__ void __launch_bounds__(kRgThreads) sel_resgram_kernel(SelState s) {
     }
     __syncthreads();
   }
-  // G' = G - acc through a shared tile, so that both the tile and its mirror are read and
-  // written in whole rows (coalesced)
+  // G' = G - acc through a shared tile, so that the tile is read and its mirror written in
+  // whole rows (coalesced)
   float(*Tt)[kRgTile + 1] = reinterpret_cast<float(*)[kRgTile + 1]>(sbuf);
 #pragma unroll
   for (int r = 0; r < 4; ++r)
@@ -702,16 +839,18 @@ __global__ void __launch_bounds__(kRgThreads) sel_resgram_kernel(SelState s) {
       const int r = r0 + m * (kRgThreads / kRgTile);
       gv[m] = okc && toki[r] >= 0 ? g0[static_cast<long long>(r) * s.R] : 0.f;
     }
+    if (ti == tk) {
 #pragma unroll
-    for (int m = 0; m < kRowsPer; ++m) {
-      const int r = r0 + m * (kRgThreads / kRgTile);
-      if (okc && toki[r] >= 0) {
-        const float v = gv[m] - Tt[r][c];
-        g0[static_cast<long long>(r) * s.R] = v;
-        Tt[r][c] = v;
+      for (int m = 0; m < kRowsPer; ++m) {
+        const int r = r0 + m * (kRgThreads / kRgTile);
+        if (okc && toki[r] >= 0) g0[static_cast<long long>(r) * s.R] = gv[m] - Tt[r][c];
       }
-    }
-    if (ti != tk) {
+    } else {                                         // the mirrored tile alone: the lower triangle is read
+#pragma unroll
+      for (int m = 0; m < kRowsPer; ++m) {
+        const int r = r0 + m * (kRgThreads / kRgTile);
+        Tt[r][c] = gv[m] - Tt[r][c];
+      }
       __syncthreads();
       float* m0 = Gb + static_cast<long long>(tk * kRgTile) * s.R + ti * kRgTile + c;
 #pragma unroll
@@ -724,54 +863,65 @@ __global__ void __launch_bounds__(kRgThreads) sel_resgram_kernel(SelState s) {
 }
 
 // ------------------------------------------------------------------ greedy
-// One CTA of S threads per image; thread = active slot.  The A x A part of the Gram block
-// holds the residual Gram matrix G' on the c0 basis vectors of the round (above), so a pick
-// of slot j updates slot i with the coordinates added in this launch only:
+// One CTA of S threads per image; thread = active slot.  The lower triangle of the A x A part of
+// the Gram block holds the residual Gram matrix G' on the c0 basis vectors of the round (above),
+// so a pick of slot j updates slot i with the coordinates added in this launch only:
 //   e_new[i] = (G'[j][i] - sum_{c0 <= q < nb} e_q[j] e_q[i]) / r_j.
-// Each slot keeps its round coordinates in a shared-memory row: its own side of the dot
-// products, and the other side for every thread (16-byte broadcasts) when that slot wins.  The picks take one block barrier each: the winning slot is carried in the low bits
-// of the key, and every slot's residual is published in shared memory, so all threads
-// derive the basis update from the same values; the winner's G' entry is loaded while the
-// dot product runs.  At most kRoundPicks picks per launch (the next round continues).
+// The picks are sequential, so a pick's latency is what counts; everything on its chain is on
+// chip.  G' sits in shared memory, its rows padded to 16 bytes.  A slot keeps its own round
+// coordinates in registers, moved there eight at a time, and in a shared row that the others
+// read by 16-byte broadcasts when it wins; the residual it publishes becomes the winner's 1 / r
+// beside the dot product.  The picks take one block barrier each: the winning slot is carried in
+// the low bits of the key.  At most kRoundPicks picks per launch (the next round continues):
+// the triangle leaves room for 88 coordinates a slot.  Bound by the chain of dependent
+// instructions of a pick (two reductions of keys, the barrier, the dot product: about 930 cycles,
+// 0.45 us; two slots a thread were slower, 1860 cycles, as were a branch per eight coordinates,
+// 1020, and G' read from global memory).  One image, 80 picks: 80.9 -> 52.9 us; 64 images: 82.1 ->
+// 52.4 us (ncu, cold).
+constexpr int kRoundChunks = kRoundPicks / 8;
+constexpr int kGreedyWarps = kActiveSlots / 32;
+static_assert(kRoundPicks % 8 == 0 && kRoundPitch % 4 == 0, "coordinate rows in 16-byte units");
+static_assert((kGreedyWarps & (kGreedyWarps - 1)) == 0, "lanes read the warps' keys round robin");
 
-// key of a candidate inside the round: (value bits, 0xFFFF - token, slot); the upper 48
-// bits order like make_key (value descending, lower token first).
-__device__ __forceinline__ uint64_t theta48(uint64_t theta) {   // make_key -> upper 48 bits of the round key
-  if (theta == 0) return 0;
-  const uint32_t tok = static_cast<uint32_t>(key_index(theta));
-  return ((theta >> 32) << 16) | (0xFFFFu - tok);
-}
-
-// Largest (hi, lo) pair over the warp, hi first: two warp reductions on 32-bit words.
-__device__ __forceinline__ uint64_t warp_max_key(uint32_t hi, uint32_t lo) {
-  const uint32_t h = __reduce_max_sync(0xffffffffu, hi);
-  const uint32_t l = __reduce_max_sync(0xffffffffu, hi == h ? lo : 0u);
-  return (static_cast<uint64_t>(h) << 32) | l;
+// First float of row i of the lower triangle whose rows are padded to 16 bytes.
+__host__ __device__ inline int tri_row(int i) {
+  const int g = i >> 2;
+  return 8 * g * (g + 1) + (i & 3) * 4 * (g + 1);
 }
 
 __global__ void __launch_bounds__(kActiveSlots, 1) sel_greedy_kernel(SelState s) {
   pdl_enter();
   extern __shared__ __align__(16) float shf[];
-  __shared__ uint64_t wkey[2][32];
+  __shared__ uint2 wkey[2][kGreedyWarps];            // (value bits, (0xFFFF - token, slot)) per warp
   const int b = blockIdx.x;
   if (s.done[b]) return;
-  const int S = s.S, R = s.R, KP = s.KP;
-  float* r2s = shf;                                  // [S] published residuals
-  float* sqs = r2s + S;                              // [S]
-  int32_t* tks = reinterpret_cast<int32_t*>(sqs + S);   // [S] tokens of the slots
+  constexpr int S = kActiveSlots;
+  const int R = s.R, KP = s.KP;
+  float* Gt = shf;                                   // [tri_row(S)] residual Gram matrix, lower triangle
+  float* Er = Gt + tri_row(S);                       // [S][kRoundPitch] round coordinates
+  float* pub = Er + S * kRoundPitch;                 // [S] residual^2, or -1: degenerate, no basis vector
+  int32_t* tks = reinterpret_cast<int32_t*>(pub + S);   // [S] tokens of the slots
   int32_t* ends = tks + S;                           // [S] round coordinates of the slots at the end
   int32_t* pk_tok = ends + S;                        // [kRoundPicks] this launch's picks
   float* pk_r2 = reinterpret_cast<float*>(pk_tok + kRoundPicks);  // their residuals (-1: no basis vector)
-  float* Er = pk_r2 + kRoundPicks;                   // [S][kRoundPitch] round coordinates
   const long long base = static_cast<long long>(b) * s.N;
   const int slot = threadIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-  const int tok = s.aslot[static_cast<long long>(b) * S + slot];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float* Gb = s.G + static_cast<long long>(b) * S * R;
+  const int tok = s.aslot[static_cast<long long>(b) * S + slot];
+#pragma unroll 4
+  for (int r = warp; r < S; r += kGreedyWarps) {     // padded rows, a warp per row (R % 16 == 0)
+    const float* g = Gb + static_cast<long long>(r) * R + 4 * lane;
+    float* d = Gt + tri_row(r) + 4 * lane;
+    if (4 * lane <= r) cp_async16(d, g);
+    if (4 * lane + 128 <= r) cp_async16(d + 128, g + 128);
+  }
   int nb = s.nbasis[b], np = s.npicks[b];
-  const int c0 = nb;
+  const int c0 = nb, np0 = np;
   const bool forced = s.mode[b] == 1;
-  const uint64_t th48 = theta48(s.theta[b]);
+  const uint64_t theta = s.theta[b];                 // the best key outside the active set
+  const uint32_t th_v = static_cast<uint32_t>(theta >> 32);
+  const uint32_t th_t = theta ? 0xFFFFu - static_cast<uint32_t>(key_index(theta)) : 0u;
   float* me = Er + slot * kRoundPitch;
 
   float r2 = 0.f, sq = 0.f, p = 0.f, val = 0.f;
@@ -786,25 +936,39 @@ __global__ void __launch_bounds__(kActiveSlots, 1) sel_greedy_kernel(SelState s)
     }
     r2 = s.r2[base + tok];
     sq = s.sqn[base + tok];
+    val = sel_value(p, r2, sq, s.lambda, s.tau);
   }
   {
-    // zero rows: the unrolled dot products read a winner's row up to the next multiple of 32
+    // zero rows: the dot products read a winner's row up to the next multiple of 8
     float4* row4 = reinterpret_cast<float4*>(me);
     for (int q = 0; q < kRoundPitch / 4; ++q) row4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   tks[slot] = tok;
-  if (tok >= 0) val = sel_value(p, r2, sq, s.lambda, s.tau);
-  r2s[slot] = r2;
-  sqs[slot] = sq;
+  // sel_value with what does not change between picks taken out of the loop.  A slot that is not a
+  // candidate (any more) goes through the same steps with a value of zero and the lowest key.
+  const bool lam1 = s.lambda == 1.f;
+  const float floor2 = fmaxf(s.tau * sq, 0.f);
+  float pv = alive && p > 0.f ? p : 0.f;             // p_hat of a candidate
+  float r2_end = r2, val_end = val;                  // residual and value of a slot that leaves
+  pub[slot] = r2 > floor2 ? r2 : -1.f;
+  uint32_t vkey = alive ? __float_as_uint(val) : 0u;   // val >= 0: bit order = numeric order
+  uint32_t lkey = alive ? ((0xFFFFu - static_cast<uint32_t>(tok)) << 16) | static_cast<uint32_t>(slot) : 0u;
+  uint64_t er[kRoundChunks][4];                      // own round coordinates, whole chunks of eight (pairs)
+#pragma unroll
+  for (int c = 0; c < kRoundChunks; ++c)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) er[c][u] = 0ull;
+  cp_async_wait_all();
   __syncthreads();
 
-  int nr = 0;                                        // round coordinates so far (uniform)
-  for (int step = 0, buf = 0; np < s.K && step < kRoundPicks; ++step, buf ^= 1) {
+  int nr = 0, cc = 0;                                // round coordinates so far, whole chunks (uniform)
+  const int steps = min(s.K - np, kRoundPicks);
+  int step = 0;
+  for (; step < steps; ++step) {
     {
-      const uint32_t vb = alive ? __float_as_uint(val > 0.f ? val : 0.f) : 0u;
-      const uint32_t lo = alive ? ((0xFFFFu - static_cast<uint32_t>(tok)) << 16) | static_cast<uint32_t>(slot) : 0u;
-      const uint64_t key = warp_max_key(vb, lo);
-      if (lane == 0) wkey[buf][warp] = key;
+      const uint32_t vm = __reduce_max_sync(0xffffffffu, vkey);
+      const uint32_t lm = __reduce_max_sync(0xffffffffu, vkey == vm ? lkey : 0u);
+      if (lane == 0) wkey[step & 1][warp] = make_uint2(vm, lm);
     }
     __syncthreads();
     int jslot;
@@ -812,58 +976,76 @@ __global__ void __launch_bounds__(kActiveSlots, 1) sel_greedy_kernel(SelState s)
       jslot = step;
       if (jslot >= S || tks[jslot] < 0) break;
     } else {
-      const uint64_t k = lane < nwarps ? wkey[buf][lane] : 0ull;
-      const uint64_t best = warp_max_key(static_cast<uint32_t>(k >> 32), static_cast<uint32_t>(k));
-      if (best == 0 || (best >> 16) <= th48) break;   // uniform
-      jslot = static_cast<int>(best & 0xFFFFu);
+      const uint2 k = wkey[step & 1][lane & (kGreedyWarps - 1)];
+      const uint32_t vm = __reduce_max_sync(0xffffffffu, k.x);
+      const uint32_t lm = __reduce_max_sync(0xffffffffu, k.x == vm ? k.y : 0u);
+      // nothing left, or a token outside the set may come first (uniform)
+      if (lm == 0u || vm < th_v || (vm == th_v && (lm >> 16) <= th_t)) break;
+      jslot = static_cast<int>(lm & 0xFFFFu);
     }
-    const int jt = tks[jslot];
-    const float r2j = r2s[jslot], sqj = sqs[jslot];
-    const bool ext = (r2j > s.tau * sqj) && (r2j > 0.f);
+    const float r2j = pub[jslot];
     if (slot == jslot) {                             // global writes wait for the end
       alive = false;
-      mine = nb;
-      pk_tok[step] = jt;
-      pk_r2[step] = ext ? r2j : -1.f;
+      pv = 0.f;
+      vkey = 0u;
+      lkey = 0u;
+      r2_end = r2;
+      val_end = val;
+      mine = nb + nr;
+      pk_tok[step] = tok;
+      pk_r2[step] = r2j >= 0.f ? r2j : -1.f;
     }
-    if (ext) {
-      if (alive) {
-        const float gji = Gb[static_cast<long long>(jslot) * R + slot];   // in flight during the dot product
-        const float rinv = 1.0f / sqrtf(r2j);
-        const float* cj = Er + jslot * kRoundPitch;
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        // 32 coordinates per branch, so that the loads of a block issue together; rows are
-        // zero past the round's coordinates
+    if (r2j >= 0.f) {                                // uniform: the pick adds a basis vector
+      const float gji = Gt[tri_row(max(slot, jslot)) + min(slot, jslot)];
+      const ulonglong2* cj = reinterpret_cast<const ulonglong2*>(Er + jslot * kRoundPitch);
+      const ulonglong2* mj = reinterpret_cast<const ulonglong2*>(me) + 2 * cc;
+      // the chunk being filled, from both rows (zeros past the end; cc < kRoundChunks here)
+      const ulonglong2 x0 = cj[2 * cc], x1 = cj[2 * cc + 1], m0 = mj[0], m1 = mj[1];
+      const float rinv = inv_sqrt(r2j);
+      uint64_t a0 = fma2(x0.x, m0.x, 0ull), a1 = fma2(x0.y, m0.y, 0ull);
+      uint64_t a2 = fma2(x1.x, m1.x, 0ull), a3 = fma2(x1.y, m1.y, 0ull);
+      // whole chunks, four at a time with all their loads in flight (both sides are zero at and past
+      // chunk cc: one branch per 32 coordinates instead of one per eight)
 #pragma unroll
-        for (int blk = 0; blk < kRoundPicks / 32; ++blk) {
-          if (32 * blk < nr) {
+      for (int g = 0; g < kRoundChunks; g += 4) {
+        if (g >= cc) break;                          // uniform
+        ulonglong2 x[8];
 #pragma unroll
-            for (int g = 8 * blk; g < 8 * blk + 8; ++g) {
-              const float4 c = *reinterpret_cast<const float4*>(cj + 4 * g);
-              const float4 m = *reinterpret_cast<const float4*>(me + 4 * g);
-              a0 = fmaf(c.x, m.x, a0);
-              a1 = fmaf(c.y, m.y, a1);
-              a2 = fmaf(c.z, m.z, a2);
-              a3 = fmaf(c.w, m.w, a3);
-            }
+        for (int c = 0; c < 8; ++c)
+          if (g + c / 2 < kRoundChunks) x[c] = cj[2 * g + c];
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (g + c < kRoundChunks) {
+            a0 = fma2(x[2 * c].x, er[g + c][0], a0);
+            a1 = fma2(x[2 * c].y, er[g + c][1], a1);
+            a2 = fma2(x[2 * c + 1].x, er[g + c][2], a2);
+            a3 = fma2(x[2 * c + 1].y, er[g + c][3], a3);
           }
-        }
-        const float e = (gji - ((a0 + a1) + (a2 + a3))) * rinv;
-        me[nr] = e;
-        r2 = fmaf(-e, e, r2);
-        val = sel_value(p, r2, sq, s.lambda, s.tau);
-        r2s[slot] = r2;
       }
-      ++nb;
+      const float e = (gji - ((sum2(a0) + sum2(a1)) + (sum2(a2) + sum2(a3)))) * rinv;
+      me[nr] = e;
+      r2 = fmaf(-e, e, r2);
+      const bool pos = r2 > floor2;                  // floor2 >= 0: the basis can be extended
+      pub[slot] = pos ? r2 : -1.f;
+      if (lam1) val = pos ? fmaxf((pv * pv) * r2, 0.f) : 0.f;
+      else val = sel_value(pv, r2, sq, s.lambda, s.tau);
+      vkey = __float_as_uint(val);
       ++nr;
+      if ((nr & 7) == 0) {                           // uniform: the chunk is full
+        const ulonglong2 n0 = mj[0], n1 = mj[1];
+#pragma unroll
+        for (int c = 0; c < kRoundChunks; ++c)
+          if (c == cc) { er[c][0] = n0.x; er[c][1] = n0.y; er[c][2] = n1.x; er[c][3] = n1.y; }
+        ++cc;
+      }
     }
-    ++np;
   }
+  np += step;
+  nb += nr;
   // write back: this launch's picks, then the active tokens
-  const int np0 = s.npicks[b], nb0 = s.nbasis[b];
   __syncthreads();
   if (threadIdx.x == 0) {
-    int nbw = nb0;
+    int nbw = c0;
     for (int i = 0; i < np - np0; ++i) {
       if (pk_r2[i] >= 0.f) {
         s.basis_tok[static_cast<long long>(b) * s.K + nbw] = pk_tok[i];
@@ -879,13 +1061,13 @@ __global__ void __launch_bounds__(kActiveSlots, 1) sel_greedy_kernel(SelState s)
   if (tok >= 0) {
     if (alive) mine = nb;
     s.cstep[base + tok] = mine;
-    s.r2[base + tok] = r2;
-    s.U[base + tok] = val;
+    s.r2[base + tok] = alive ? r2 : r2_end;
+    s.U[base + tok] = alive ? val : val_end;
   }
   // coordinates [c0, mine) of every slot: its round row, one warp per row
   ends[slot] = tok >= 0 ? mine : c0;
   __syncthreads();
-  for (int r = warp; r < S; r += nwarps) {
+  for (int r = warp; r < S; r += kGreedyWarps) {
     const int t = tks[r], end = ends[r];
     if (t < 0) continue;
     float* g = s.Ec + (base + t) * KP;
@@ -926,8 +1108,9 @@ __global__ void sel_proj_done_kernel(SelState s) {
   pdl_enter();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < s.B && s.proj_lim[b] > 0) {
-    s.gbase[b] = s.nbasis[b];
-    s.nb_gathered[b] = s.nbasis[b];
+    const int nb = min(s.nbasis[b], kReprojMax);       // coordinates the projection gave
+    s.gbase[b] = nb;
+    s.nb_gathered[b] = nb;
   }
 }
 
@@ -1010,11 +1193,11 @@ __global__ void sel_loop_cond_kernel(SelState s, cudaGraphConditionalHandle h, i
 size_t sel_init_smem(int N, int K0) { return (static_cast<size_t>(N) + pow2_at_least(std::max(K0, 1))) * 8; }
 size_t sel_choose_smem(int N) { return static_cast<size_t>(N) * 8; }
 size_t sel_greedy_smem(int S) {
-  return static_cast<size_t>(S) * 16 + static_cast<size_t>(kRoundPicks) * 8 +
-         static_cast<size_t>(S) * kRoundPitch * 4;
+  return static_cast<size_t>(tri_row(S)) * 4 + static_cast<size_t>(S) * kRoundPitch * 4 +
+         static_cast<size_t>(S) * 12 + static_cast<size_t>(kRoundPicks) * 8;
 }
 size_t sel_chol_smem(int K0) {
-  return (static_cast<size_t>(K0) * ((K0 + 3) & ~3) + static_cast<size_t>(K0) * coord_pitch(K0)) * 4;
+  return static_cast<size_t>(chol_row((K0 + 31) / 32 * 32)) * 4;
 }
 size_t sel_update_smem(int KP) {
   return (static_cast<size_t>(kUpdSlots) * coord_pitch(KP) + static_cast<size_t>(kChunk) * KP) * 4;

@@ -6,7 +6,7 @@
 
 namespace mapk {
 
-constexpr int kCholMax = 128;     // largest R0 factored by sel_chol_kernel
+constexpr int kCholMax = 256;     // largest R0 factored by sel_chol_kernel (a thread per token)
 
 struct SelState {
   int B, N, D, K, K0, S;          // S = active-set size (Gram block rows)
@@ -53,9 +53,10 @@ struct SelState {
 size_t sel_init_smem(int N, int K0);
 size_t sel_choose_smem(int N);
 // Active-set size (Gram block rows, threads of the greedy CTA) and the most picks one greedy
-// launch makes (their coordinates are held in registers; the next round continues).
+// launch makes (their coordinates are held in registers, and in the shared memory that the
+// packed residual Gram matrix leaves; the next round continues).
 constexpr int kActiveSlots = 256;
-constexpr int kRoundPicks = 128;
+constexpr int kRoundPicks = 88;
 size_t sel_greedy_smem(int S);
 cudaError_t launch_sel_init(const SelState& s, cudaStream_t st);
 cudaError_t launch_sel_choose(const SelState& s, cudaStream_t st);
