@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/map_gb300.h"
@@ -40,7 +41,7 @@ struct map_ctx {
   // [hi | hi | lo] of W_Q W_T2 / W_K W_V2 ([dp, 3 Dh]) and fp32 biases W_Q b_T2 / W_K b_V2
   void* wqt = nullptr; void* wkv = nullptr; float* bqt = nullptr; float* bkv = nullptr;
   DevBuf rope;  int rope_rows = 0;
-  DevBuf h1, kb, th1, qb, stats, qoff, post, sqn, pmean, snv, dist, dsa, dsb, dsc;
+  DevBuf h1, kb, th1, qb, stats, qoff, post, sqn, pmean, snv, dist;
   // selection
   DevBuf sU, sr2, scstep, sstate, sEc, spicks, sr0, sbt, srn, ssmall, stheta, saslot, sVg, sG;
   // map_prune staging
@@ -874,139 +875,163 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
   const long long D = g.D, Dh = g.Dh, dp = g.dp, Tv = static_cast<long long>(B) * N, Tt = total_m;
   CU_TRY(cudaSetDevice(c->device));
   MAP_TRY(ensure_rope(c, g.rope_on ? N + max_m + 1 : 1));
-  // question offsets and positions N + m (as for map_score), image of every question row
+  // the staged rows are 64 to a block of the elementwise kernels' grids
+  if ((std::max(Tv, Tt) + 31) / 32 > 65535) return MAP_EUNSUPPORTED;
+  // question offsets and positions N + m (as for map_score)
   MAP_TRY(ensure(c->qoff, static_cast<size_t>(3 * B + 1) * 4));
   MAP_TRY(ensure(c->post, static_cast<size_t>(total_m) * 4));
   std::vector<long long> offs(B);
-  std::vector<int32_t> row_img(static_cast<size_t>(total_m));
+  long long prows = 0;                               // question rows, each image's padded to 64
   {
     long long acc = 0;
     for (int b = 0; b < B; ++b) {
       offs[b] = acc;
-      for (int m = 0; m < lens[b]; ++m) row_img[static_cast<size_t>(acc + m)] = b;
       acc += lens[b];
+      prows += (lens[b] + 63) / 64 * 64;
     }
   }
   int32_t* qo = static_cast<int32_t*>(c->qoff.p);
+  int32_t* d_len = qo + (B + 1);
   int32_t* post = static_cast<int32_t*>(c->post.p);
-  CU_TRY(mapk::launch_query_meta(lens, offs.data(), B, N, qo, qo + (B + 1), post, nullptr, nullptr, st));
-  // fp32 workspace (the features and weights stay bf16: the tensor-core GEMMs read them as exact
-  // operands; only the biases are needed in fp32)
-  const int nblk = (N + 255) / 256;
+  long long launches = (B + 1023) / 1024;
+  CU_TRY(mapk::launch_query_meta(lens, offs.data(), B, N, qo, d_len, post, nullptr, nullptr, st));
+
+  const int nblk = (N + 255) / 256, iN = N, iD = g.D, iDh = g.Dh, idp = g.dp;
   const long long Np = (N + 3) / 4 * 4;              // logits row stride: 16-byte aligned rows
-  const int bias_idx[4] = {1, 3, 6, 8};
-  const long long floats = 4 * Dh + 5 * (Tv + Tt) * Dh + 4 * (Tv + Tt) * dp + Tt * Np + 2LL * B * N +
-                           static_cast<long long>(B) * nblk + total_m + 64 * Dh + 64 * 16;
-  MAP_TRY(ensure(c->dist, static_cast<size_t>(floats) * 4));
-  float* base = static_cast<float*>(c->dist.p);
-  auto take = [&](long long n) { float* p = base; base += ((n + 15) / 16) * 16; return p; };
-  float* Wb[10] = {};
-  for (int i : bias_idx) Wb[i] = take(Dh);
-  float *z1v = take(Tv * Dh), *h1v = take(Tv * Dh), *h2v = take(Tv * Dh), *dh2v = take(Tv * Dh), *dh1v = take(Tv * Dh);
-  float *z1t = take(Tt * Dh), *h1t = take(Tt * Dh), *h2t = take(Tt * Dh), *dh2t = take(Tt * Dh), *dh1t = take(Tt * Dh);
-  float *kp = take(Tv * dp), *kk = take(Tv * dp), *dk = take(Tv * dp), *dkp = take(Tv * dp);
-  float *qp = take(Tt * dp), *qq = take(Tt * dp), *dq = take(Tt * dp), *dqp = take(Tt * dp);
-  float* S = take(Tt * Np);
-  float *p_hat = take(static_cast<long long>(B) * N), *gb = take(static_cast<long long>(B) * N);
-  float* part = take(static_cast<long long>(B) * nblk);
-  int32_t* d_row_img = reinterpret_cast<int32_t*>(take(total_m));
-  float* colpart = take(64 * Dh);                    // partial column sums of the bias gradients
+  const int Nk = (N + 63) / 64 * 64;                 // columns of a staged logits term
   const float rs = 1.0f / std::sqrt(static_cast<float>(dp));
-  // Every contraction of the step, in order: C = alpha A(M x K) B(K x N) with A(i, k) = ta ? A[k lda
-  // + i] : A[i lda + k], B(k, j) = tb ? B[j ldb + k] : B[k ldb + j]; bf16 operands are exact.
-  struct Mm { bool ta, tb; long long M, N, K; float alpha; const void* A; bool abf; long long lda;
-              const void* Bm; bool bbf; long long ldb; float* C; long long ldc; };
-  std::vector<Mm> fwd, mid, bwd;
-  auto branch_fwd = [&](const void* X, long long T, int i1, float* z1, float* h1, float* h2, int ip, float* pre) {
-    fwd.push_back({false, true, T, Dh, D, 1.f, X, true, D, c->w[i1], true, D, z1, Dh});
-    fwd.push_back({false, true, T, Dh, Dh, 1.f, h1, false, Dh, c->w[i1 + 2], true, Dh, h2, Dh});
-    fwd.push_back({false, true, T, dp, Dh, 1.f, h2, false, Dh, c->w[ip], true, Dh, pre, dp});
+  const float2* tab = static_cast<const float2*>(c->rope.p);
+  // One modality: its rows, weights (first index, projection), buffers and stream.
+  struct Branch {
+    long long T; const void* X; int i1, ip; cudaStream_t st;
+    const int32_t* pos; int pos_mod;
+    const void* xa;                                  // the features, 16-byte aligned
+    float *z1, *raw, *pre, *part, *ws;
+    uint16_t *h1, *h2, *dpre, *dh2, *dh1;
+    long long ws_floats;
   };
-  branch_fwd(vis_feats, Tv, 5, z1v, h1v, h2v, 9, kp);
-  branch_fwd(text_feats, Tt, 0, z1t, h1t, h2t, 4, qp);
-  for (int b = 0; b < B; ++b)     // Eq. 3 logits per image, then (after the loss) dq and dk
-    mid.push_back({false, true, lens[b], N, dp, rs, qq + offs[b] * dp, false, dp, kk + b * N * dp, false, dp,
-                   S + offs[b] * Np, Np});
-  for (int b = 0; b < B; ++b) {
-    mid.push_back({false, false, lens[b], dp, N, rs, S + offs[b] * Np, false, Np, kk + b * N * dp, false, dp,
-                   dq + offs[b] * dp, dp});
-    mid.push_back({true, false, N, dp, lens[b], rs, S + offs[b] * Np, false, Np, qq + offs[b] * dp, false, dp,
-                   dk + b * N * dp, dp});
+  Branch br[2] = {};
+  br[0].T = Tv; br[0].X = vis_feats; br[0].i1 = 5; br[0].ip = 9; br[0].st = st;
+  br[0].pos = nullptr; br[0].pos_mod = g.rope_on ? N : 1;
+  br[1].T = Tt; br[1].X = text_feats; br[1].i1 = 0; br[1].ip = 4; br[1].st = st;
+  br[1].pos = g.rope_on ? post : nullptr; br[1].pos_mod = 1;
+  const int ks_dq = mapk::tc_ksplit(max_m, idp, iN, 6, c->num_sms);
+  auto slices = [&](long long M, int Nn, long long K, int products) {
+    return mapk::tc_ksplit(static_cast<int>(M), Nn, static_cast<int>(K), products, c->num_sms);
+  };
+  for (Branch& x : br) {                             // K slices of the branch's contractions
+    const int T = static_cast<int>(x.T);
+    auto need = [&](long long M, int Nn, long long K, int products) {
+      const int ks = slices(M, Nn, K, products);
+      if (ks > 1) x.ws_floats = std::max(x.ws_floats, ks * M * ((Nn + 3) / 4 * 4));
+    };
+    need(T, iDh, D, 1); need(T, iDh, Dh, 3); need(T, idp, Dh, 3);
+    need(dp, iDh, T, 6); need(T, iDh, dp, 3); need(Dh, iDh, T, 6); need(T, iDh, Dh, 3); need(Dh, iD, T, 3);
   }
-  auto branch_bwd = [&](long long T, float* dpre, const void* X, int i1, const float* h1, const float* h2, float* dh2,
-                        float* dh1, int ip) {
-    bwd.push_back({true, false, dp, Dh, T, 1.f, dpre, false, dp, h2, false, Dh, gout[ip], Dh});
-    bwd.push_back({false, false, T, Dh, dp, 1.f, dpre, false, dp, c->w[ip], true, Dh, dh2, Dh});
-    bwd.push_back({true, false, Dh, Dh, T, 1.f, dh2, false, Dh, h1, false, Dh, gout[i1 + 2], Dh});
-    bwd.push_back({false, false, T, Dh, Dh, 1.f, dh2, false, Dh, c->w[i1 + 2], true, Dh, dh1, Dh});
-    bwd.push_back({true, false, Dh, D, T, 1.f, dh1, false, Dh, X, true, D, gout[i1], D});
-  };
-  branch_bwd(Tv, dkp, vis_feats, 5, h1v, h2v, dh2v, dh1v, 9);
-  branch_bwd(Tt, dqp, text_feats, 0, h1t, h2t, dh2t, dh1t, 4);
-  // staging buffers for the split-bf16 operands: the largest any contraction needs
-  size_t wa = 0, wb = 0, wc = 0;
-  for (const auto* list : {&fwd, &mid, &bwd})
-    for (const Mm& m : *list) {
-      size_t a = 0, bb = 0, cc = 0;
-      mapk::tc_matmul_ws(static_cast<int>(m.M), static_cast<int>(m.N), static_cast<int>(m.K), m.alpha, m.abf, m.bbf,
-                         c->num_sms, &a, &bb, &cc);
-      wa = std::max(wa, a);
-      wb = std::max(wb, bb);
-      wc = std::max(wc, cc);
+  // workspace: carved twice, first for its size
+  float *S = nullptr, *dq = nullptr, *dk = nullptr, *p_hat = nullptr, *gb = nullptr, *part = nullptr,
+        *ws_dq = nullptr;
+  uint16_t *kk = nullptr, *qq = nullptr, *dl = nullptr;
+  int32_t *poff = nullptr, *prow = nullptr, *img = nullptr;
+  size_t used = 0;
+  auto carve_all = [&](char* base) {
+    used = 0;
+    auto take = [&](auto*& p, long long n) {
+      using T = std::remove_reference_t<decltype(*p)>;
+      p = reinterpret_cast<T*>(base + used);
+      used += (static_cast<size_t>(n) * sizeof(T) + 255) / 256 * 256;
+    };
+    for (Branch& x : br) {
+      take(x.z1, x.T * Dh); take(x.raw, x.T * Dh); take(x.pre, x.T * dp);
+      take(x.part, (x.T + 63) / 64 * Dh); take(x.ws, x.ws_floats);
+      take(x.h1, x.T * 3 * Dh); take(x.h2, x.T * 3 * Dh); take(x.dh2, x.T * 3 * Dh); take(x.dh1, x.T * 3 * Dh);
+      take(x.dpre, x.T * 3 * dp);
+      uint16_t* xc = nullptr;
+      x.xa = x.X;
+      if (!aligned16(x.X)) { take(xc, x.T * D); x.xa = xc; }
     }
-  MAP_TRY(ensure(c->dsa, wa * 2));
-  MAP_TRY(ensure(c->dsb, wb * 2));
-  MAP_TRY(ensure(c->dsc, std::max<size_t>(wc, 4) * 4));
-  long long mm_launches = 0;
-  auto run_mm = [&](const Mm& m) -> int {
-    cudaError_t e = mapk::launch_tc_matmul(m.ta, m.tb, static_cast<int>(m.M), static_cast<int>(m.N),
-                                           static_cast<int>(m.K), m.alpha, m.A, m.abf, m.lda, m.Bm, m.bbf, m.ldb,
-                                           m.C, m.ldc, c->dsa.p, c->dsb.p, static_cast<float*>(c->dsc.p), c->num_sms,
-                                           c->status, c->wait_ns, st, &mm_launches);
+    take(kk, Tv * 3 * dp); take(qq, prows * 3 * dp);
+    take(S, prows * Np); take(dl, prows * 3 * Nk);
+    take(dq, prows * dp); take(ws_dq, ks_dq > 1 ? static_cast<long long>(ks_dq) * prows * dp : 0); take(dk, Tv * dp);
+    take(p_hat, static_cast<long long>(B) * N); take(gb, static_cast<long long>(B) * N);
+    take(part, static_cast<long long>(B) * nblk);
+    take(poff, B); take(prow, total_m); take(img, prows);
+  };
+  carve_all(nullptr);
+  MAP_TRY(ensure(c->dist, used));
+  carve_all(static_cast<char*>(c->dist.p));
+
+  using mapk::TcBatch; using mapk::TcOperand; using mapk::TcResult;
+  auto split = [](const uint16_t* p, long long rows, int cols, int mn) { return TcOperand{p, rows, 3 * cols, cols, mn}; };
+  auto exact = [](const void* p, long long rows, int cols, int mn) { return TcOperand{p, rows, cols, 0, mn}; };
+  auto mm = [&](long long M, int Nn, long long K, const TcOperand& A, const TcOperand& Bo, const TcBatch& bt, int ks,
+                bool add, float* C, long long ldc, float* ws, cudaStream_t s, TcResult* res) -> int {
+    cudaError_t e = mapk::launch_tc_matmul(static_cast<int>(M), Nn, static_cast<int>(K), A, Bo, bt, ks, add, C, ldc, ws,
+                                           c->num_sms, c->status, c->wait_ns, s, &launches, res);
     if (e == cudaErrorInvalidValue) return MAP_EUNSUPPORTED;
     return cuda_err(e);
   };
-  CU_TRY(mapk::launch_put_ints(row_img.data(), static_cast<int>(total_m), d_row_img, st));
-  for (int i : bias_idx) CU_TRY(mapk::launch_bf16_to_f32(c->w[i], Dh, Wb[i], st));
-  const float2* tab = static_cast<const float2*>(c->rope.p);
+  ++launches;
+  CU_TRY(mapk::launch_distill_meta(d_len, qo, B, poff, prow, img, st));
   // forward: z1 = X W1^T + b1, h1 = GELU(z1), h2 = h1 W2^T + b2, projection, RoPE
-  auto fwd_tail = [&](int j, long long T, int i1, float* z1, float* h1, float* h2, float* pre, float* post_rope,
-                      const int32_t* pos, int pos_mod) -> int {
-    MAP_TRY(run_mm(fwd[j]));
-    CU_TRY(mapk::launch_bias_gelu(z1, Wb[i1 + 1], T, Dh, h1, st));
-    MAP_TRY(run_mm(fwd[j + 1]));
-    CU_TRY(mapk::launch_bias_add(h2, Wb[i1 + 3], T, Dh, st));
-    MAP_TRY(run_mm(fwd[j + 2]));
-    CU_TRY(mapk::launch_rope_f32(false, pre, T, dp, tab, c->rope_rows, pos, pos_mod, post_rope, st));
+  auto forward = [&](const Branch& x, float scale, uint16_t* out, const int32_t* out_map) -> int {
+    TcResult r;
+    if (x.xa != x.X)
+      CU_TRY(cudaMemcpyAsync(const_cast<void*>(x.xa), x.X, static_cast<size_t>(x.T) * D * 2, cudaMemcpyDeviceToDevice, x.st));
+    MAP_TRY(mm(x.T, iDh, D, exact(x.xa, x.T, iD, 0), exact(c->w[x.i1], Dh, iD, 0), TcBatch{}, slices(x.T, iDh, D, 1),
+               false, x.raw, Dh, x.ws, x.st, &r));
+    CU_TRY(mapk::launch_act_split(true, r, c->w[x.i1 + 1], x.T, iDh, x.z1, x.h1, x.st));
+    MAP_TRY(mm(x.T, iDh, Dh, split(x.h1, x.T, iDh, 0), exact(c->w[x.i1 + 2], Dh, iDh, 0), TcBatch{},
+               slices(x.T, iDh, Dh, 3), false, x.raw, Dh, x.ws, x.st, &r));
+    CU_TRY(mapk::launch_act_split(false, r, c->w[x.i1 + 3], x.T, iDh, nullptr, x.h2, x.st));
+    MAP_TRY(mm(x.T, idp, Dh, split(x.h2, x.T, iDh, 0), exact(c->w[x.ip], dp, iDh, 0), TcBatch{},
+               slices(x.T, idp, Dh, 3), false, x.pre, dp, x.ws, x.st, &r));
+    CU_TRY(mapk::launch_rope_split(false, r, nullptr, x.T, idp, tab, c->rope_rows, x.pos, x.pos_mod, scale, out,
+                                   out_map, x.st));
+    launches += 3;
     return MAP_OK;
   };
-  MAP_TRY(fwd_tail(0, Tv, 5, z1v, h1v, h2v, kp, kk, nullptr, g.rope_on ? N : 1));
-  MAP_TRY(fwd_tail(3, Tt, 0, z1t, h1t, h2t, qp, qq, g.rope_on ? post : nullptr, 1));
-  // Eq. 3 logits per image, softmax, KL, and dL/dlogits
-  for (int b = 0; b < B; ++b) MAP_TRY(run_mm(mid[b]));
-  CU_TRY(mapk::launch_distill_loss_grad(S, Np, total_m, qo, d_row_img, teacher, B, N, p_hat, gb, part, loss, st));
-  for (size_t j = B; j < mid.size(); ++j) MAP_TRY(run_mm(mid[j]));
-  // backward through RoPE, the projection and the MLP of each branch
-  auto bwd_tail = [&](int j, float* dpost, long long T, const int32_t* pos, int pos_mod, float* dpre, const float* z1,
-                      float* dh2, float* dh1, int i1) -> int {
-    CU_TRY(mapk::launch_rope_f32(true, dpost, T, dp, tab, c->rope_rows, pos, pos_mod, dpre, st));
-    MAP_TRY(run_mm(bwd[j]));                         // dW_p
-    MAP_TRY(run_mm(bwd[j + 1]));                     // dh2
-    MAP_TRY(run_mm(bwd[j + 2]));                     // dW2
-    CU_TRY(mapk::launch_colsum(dh2, T, Dh, colpart, gout[i1 + 3], st));
-    MAP_TRY(run_mm(bwd[j + 3]));                     // dh1
-    CU_TRY(mapk::launch_gelu_back(dh1, z1, T * Dh, st));
-    MAP_TRY(run_mm(bwd[j + 4]));                     // dW1
-    CU_TRY(mapk::launch_colsum(dh1, T, Dh, colpart, gout[i1 + 1], st));
+  // backward through RoPE, the projection and the MLP
+  auto backward = [&](const Branch& x, const TcResult& dpost, const int32_t* in_map, float scale) -> int {
+    TcResult r;
+    CU_TRY(mapk::launch_rope_split(true, dpost, in_map, x.T, idp, tab, c->rope_rows, x.pos, x.pos_mod, scale, x.dpre,
+                                   nullptr, x.st));
+    MAP_TRY(mm(dp, iDh, x.T, split(x.dpre, x.T, idp, 1), split(x.h2, x.T, iDh, 1), TcBatch{}, slices(dp, iDh, x.T, 6),
+               true, gout[x.ip], Dh, x.ws, x.st, nullptr));                                          // dW_p
+    MAP_TRY(mm(x.T, iDh, dp, split(x.dpre, x.T, idp, 0), exact(c->w[x.ip], dp, iDh, 1), TcBatch{},
+               slices(x.T, iDh, dp, 3), false, x.raw, Dh, x.ws, x.st, &r));                          // dh2
+    CU_TRY(mapk::launch_back_split(r, nullptr, x.T, iDh, x.dh2, x.part, gout[x.i1 + 3], x.st));
+    MAP_TRY(mm(Dh, iDh, x.T, split(x.dh2, x.T, iDh, 1), split(x.h1, x.T, iDh, 1), TcBatch{}, slices(Dh, iDh, x.T, 6),
+               true, gout[x.i1 + 2], Dh, x.ws, x.st, nullptr));                                      // dW2
+    MAP_TRY(mm(x.T, iDh, Dh, split(x.dh2, x.T, iDh, 0), exact(c->w[x.i1 + 2], Dh, iDh, 1), TcBatch{},
+               slices(x.T, iDh, Dh, 3), false, x.raw, Dh, x.ws, x.st, &r));                          // dh1
+    CU_TRY(mapk::launch_back_split(r, x.z1, x.T, iDh, x.dh1, x.part, gout[x.i1 + 1], x.st));
+    MAP_TRY(mm(Dh, iD, x.T, split(x.dh1, x.T, iDh, 1), exact(x.xa, x.T, iD, 1), TcBatch{}, slices(Dh, iD, x.T, 3), true,
+               gout[x.i1], D, x.ws, x.st, nullptr));                                                 // dW1
+    launches += 5;
     return MAP_OK;
   };
-  MAP_TRY(bwd_tail(0, dk, Tv, nullptr, g.rope_on ? N : 1, dkp, z1v, dh2v, dh1v, 5));
-  MAP_TRY(bwd_tail(5, dq, Tt, g.rope_on ? post : nullptr, 1, dqp, z1t, dh2t, dh1t, 0));
-  // query metadata, question-row images, 4 bias conversions, the contractions (the GEMM, its
-  // operand stagings and the sum of its K slices, as counted by the launcher), 2 x 3 forward
-  // elementwise, 4 loss / softmax-backward kernels, 2 x 6 backward elementwise (RoPE transpose,
-  // GELU', two column sums of two launches each)
-  c->counters.launches += (B + 1023) / 1024 + (total_m + 2047) / 2048 + 4 + mm_launches + 6 + 4 + 12;
+  MAP_TRY(forward(br[0], 1.f, kk, nullptr));
+  MAP_TRY(forward(br[1], rs, qq, prow));
+  CU_TRY(mapk::launch_zero_pad_rows(qq, 3 * idp, img, prows, br[1].st));
+  // Eq. 3 logits (q k / sqrt(dp), the scale is in q) of every image, softmax, KL, and dL/dlogits
+  TcBatch lb;
+  lb.n = B; lb.a_off = poff; lb.b_rows = iN; lb.m_count = d_len; lb.c_rows = prows;
+  MAP_TRY(mm(max_m, iN, dp, split(qq, prows, idp, 0), split(kk, Tv, idp, 0), lb, 1, false, S, Np, nullptr, st, nullptr));
+  CU_TRY(mapk::launch_distill_loss_grad(S, Np, prows, d_len, poff, img, teacher, B, N, p_hat, gb, part, loss, dl, Nk, st));
+  launches += 5;
+  // dk = dl^T q per image (K = its question rows, padded with zeros), dq = dl k (K = its tokens)
+  TcResult rk, rq;
+  TcBatch kb;
+  kb.n = B; kb.a_off = poff; kb.b_off = poff; kb.k_count = d_len; kb.c_stride = static_cast<long long>(N) * dp;
+  kb.c_rows = Tv;
+  MAP_TRY(mm(N, idp, max_m, split(dl, prows, Nk, 1), split(qq, prows, idp, 1), kb, 1, false, dk, dp, nullptr, br[0].st, &rk));
+  TcBatch qb;
+  qb.n = B; qb.a_off = poff; qb.b_rows = iN; qb.m_count = d_len; qb.c_rows = prows;
+  MAP_TRY(mm(max_m, idp, N, split(dl, prows, Nk, 0), split(kk, Tv, idp, 1), qb, ks_dq, false, dq, dp, ws_dq, br[1].st, &rq));
+  MAP_TRY(backward(br[0], rk, nullptr, 1.f));
+  MAP_TRY(backward(br[1], rq, prow, rs));
+  c->counters.launches += launches;
   return MAP_OK;
 }
 
@@ -1034,7 +1059,7 @@ void map_destroy(map_ctx* ctx) {
   for (void* p : {ctx->wqt, ctx->wkv, static_cast<void*>(ctx->bqt), static_cast<void*>(ctx->bkv)})
     if (p) cudaFree(p);
   DevBuf* bufs[] = {&ctx->rope, &ctx->h1, &ctx->kb, &ctx->th1, &ctx->qb, &ctx->stats,
-                    &ctx->qoff, &ctx->post, &ctx->sqn, &ctx->pmean, &ctx->snv, &ctx->dist, &ctx->dsa, &ctx->dsb, &ctx->dsc, &ctx->sU, &ctx->sr2, &ctx->scstep, &ctx->sstate,
+                    &ctx->qoff, &ctx->post, &ctx->sqn, &ctx->pmean, &ctx->snv, &ctx->dist, &ctx->sU, &ctx->sr2, &ctx->scstep, &ctx->sstate,
                     &ctx->sEc, &ctx->spicks, &ctx->sr0, &ctx->sbt, &ctx->srn, &ctx->ssmall, &ctx->stheta,
                     &ctx->saslot, &ctx->sVg, &ctx->sG, &ctx->pvis, &ctx->ptext, &ctx->pout, &ctx->pkeep,
                     &ctx->pscores};

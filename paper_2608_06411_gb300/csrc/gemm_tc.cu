@@ -49,13 +49,14 @@ struct KArgs {
   const int* col_count;
   int b_base;
   ProjArgs proj;
-  int a_kwrap, b_kwrap;
+  int a_kwrap;
   int split3;
   const float* biasf;
   const int* blist; const int* bcount;
   const int* m_limit;
   unsigned long long wait_ns;   // limit of the role waits (the drain waits keep kWaitLimitNs)
   int ksplit; long long c_split_stride;   // EPI_F32 split-K: partial sums per K slice
+  GemmProducts pr;                         // EPI_F32: products of column segments (pr.n > 0)
   int sym;                                 // B is A: the diagonal tile reads its A stage as B
   int n_outer;                             // unit order: column tiles outermost
 };
@@ -196,16 +197,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int n_tiles = (a.N + BN - 1) / BN;
   const int nbatch = a.blist ? min(a.batch, *a.bcount) : a.batch;
   const int total = nbatch * m_units * n_tiles * a.ksplit;
-  const int KB = a.K / kBK;
+  constexpr bool PRODUCTS = EPI == EPI_F32;       // the epilogue of the segmented products
+  // K blocks of one product of image c.b
+  auto product_kblocks = [&](const TileCoord& c) {
+    return a.pr.k_count ? (__ldg(a.pr.k_count + c.b) + kBK - 1) / kBK : a.pr.kblocks;
+  };
   // K blocks of a unit's slice (the whole K without split-K)
   auto kb_range = [&](const TileCoord& c, int& kb0, int& kb1) {
+    int KB = a.K / kBK;
+    if constexpr (PRODUCTS) {
+      if (a.pr.n > 0) KB = a.pr.n * product_kblocks(c);
+    }
     kb0 = c.ks * KB / a.ksplit;
     kb1 = (c.ks + 1) * KB / a.ksplit;
   };
   // K block kb -> (A column, B column)
   auto kcols = [&](int kb, int& ac, int& bc) {
     if (a.split3) {
-      const int nbk = KB / 3;
+      const int nbk = a.K / kBK / 3;
       if (kb < 2 * nbk) {
         const int j = kb >> 1;
         ac = j * kBK;
@@ -215,7 +224,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
     } else {
       ac = a.a_kwrap > 0 ? (kb * kBK) % a.a_kwrap : kb * kBK;
-      bc = a.b_kwrap > 0 ? (kb * kBK) % a.b_kwrap : kb * kBK;
+      bc = kb * kBK;
     }
   };
 
@@ -247,6 +256,60 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int kstep = alias ? 2 : 1;           // alias: two K blocks per stage (A and B buffers)
         int kb0, kb1;
         kb_range(c, kb0, kb1);
+        if constexpr (PRODUCTS) {
+          if (a.pr.n > 0) {
+            // K block k0 of product p: segment p of each operand, K-major (one box of rows) or
+            // MN-major (boxes of 64 columns by 64 K rows: the operand's rows are its K index).  One
+            // thread issues every load, so what a K block does not change is kept out of its loop.
+            const GemmProducts& q = a.pr;
+            constexpr int BR = CG2 ? BN / 2 : BN;
+            const int nkb = product_kblocks(c);
+            const int n0 = c.n_blk * BN + (CG2 ? static_cast<int>(crank) * BR : 0), m0 = c.m_blk * kBM;
+            const int arb = q.a_off ? __ldg(q.a_off + c.b) : c.b * a.a_row_stride;
+            const int brb = q.b_off ? __ldg(q.b_off + c.b) : c.b * a.b_row_stride;
+            const bool amn = q.a_mn != 0, bmn = q.b_mn != 0;
+            int p = kb0 / nkb, j = kb0 - p * nkb;
+            int aseg = q.a_seg[p], bseg = q.b_seg[p];
+            const uint32_t fb0 = CG2 ? mapa_u32(full, 0) : 0u;
+            for (int kb = kb0; kb < kb1; ++kb) {
+              if (!mbar_wait(&empty[stage], phase ^ 1, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
+              const uint32_t fb = fb0 + stage * 8;
+              if constexpr (CG2) {
+                if (crank == 0) mbar_arrive_expect_tx(&full[stage], 2 * S::STAGE_BYTES);
+              } else {
+                mbar_arrive_expect_tx(&full[stage], S::STAGE_BYTES);
+              }
+              auto load = [&](uint8_t* dst, const CUtensorMap* tm, int x, int y) {
+                if constexpr (CG2) tma_load_2d_cg2(dst, tm, fb, x, y);
+                else tma_load_2d(dst, tm, &full[stage], x, y);
+              };
+              uint8_t* da = sA + stage * S::A_BYTES;
+              uint8_t* db = sB + stage * S::B_BYTES;
+              const int k0 = j * kBK;
+              if (amn) {
+#pragma unroll
+                for (int h = 0; h < kBM; h += 64) load(da + h * 128, &tmA, aseg + m0 + h, arb + k0);
+              } else {
+                load(da, &tmA, aseg + k0, arb + m0);
+              }
+              if (bmn) {
+#pragma unroll
+                for (int h = 0; h < BR; h += 64) load(db + h * 128, &tmB, bseg + n0 + h, brb + k0);
+              } else {
+                load(db, &tmB, bseg + k0, brb + n0);
+              }
+              last_par[stage] = static_cast<int>(phase);
+              if (++stage == STAGES) { stage = 0; phase ^= 1; }
+              if (++j == nkb && kb + 1 < kb1) {
+                j = 0;
+                ++p;
+                aseg = q.a_seg[p];
+                bseg = q.b_seg[p];
+              }
+            }
+            continue;
+          }
+        }
         for (int kb = kb0; kb < kb1; kb += kstep) {
           if (!mbar_wait(&empty[stage], phase ^ 1, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
           int ac, bc;
@@ -286,6 +349,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // ---------------------------------------------------------------- MMA issuer (CG2: leader)
       uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
       bool issued = false, ok = true;
+      // products: descriptors without their address (shared memory addresses are below 2^18), and
+      // their step per 16 K: 32 bytes along a K-major row, 16 rows of 128 bytes of an MN-major box
+      const bool amn = PRODUCTS && a.pr.a_mn, bmn = PRODUCTS && a.pr.b_mn;
+      const uint64_t adesc0 = amn ? desc_sw128_mn(0) : desc_sw128(0), bdesc0 = bmn ? desc_sw128_mn(0) : desc_sw128(0);
+      const uint32_t astep = (amn ? 2048 : 32) >> 4, bstep = (bmn ? 2048 : 32) >> 4;
+      const uint32_t pid = IDESC | (amn ? 1u << 15 : 0u) | (bmn ? 1u << 16 : 0u);
       for (int t = unit0; t < total && ok; t += units_step) {
         TileCoord c = tile_coord<PAIR>(a, t, nbatch, m_units, n_tiles, BN, crank);
         if (c.skip) continue;
@@ -301,7 +370,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           tc_fence_after();
           const uint32_t a0 = smem_u32(sA + stage * S::A_BYTES);
           const uint32_t b0 = alias ? a0 : smem_u32(sB + stage * S::B_BYTES);
-          if (alias) {
+          if (PRODUCTS && a.pr.n > 0) {
+#pragma unroll
+            for (int k = 0; k < kBK / 16; ++k) {
+              const uint64_t da = adesc0 + (a0 >> 4) + k * astep, db = bdesc0 + (b0 >> 4) + k * bstep;
+              if constexpr (CG2) umma_bf16_cg2(d_tmem, da, db, pid, (kb != kb0 || k != 0));
+              else umma_bf16(d_tmem, da, db, pid, (kb != kb0 || k != 0));
+            }
+            if constexpr (CG2) umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
+            else umma_commit(&empty[stage]);
+          } else if (alias) {
             // each buffer is both operands of its K block (the tile's B rows are its A rows)
             const uint32_t a1 = smem_u32(sB + stage * S::B_BYTES);
             const int n2 = kb + 1 < kb1 ? 2 : 1;
@@ -703,7 +781,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           pj.cstep[tok] = nb0;
         }
       } else if constexpr (EPI == EPI_F32) {
-        float* out = reinterpret_cast<float*>(a.C) + crow + col0 + c.ks * a.c_split_stride;
+        // products with per-image A rows write C at the same rows
+        const long long orow = a.pr.n > 0 && a.pr.a_off && !a.pr.a_mn
+                                   ? (__ldg(a.pr.a_off + c.b) + static_cast<long long>(row)) * a.ldc : crow;
+        float* out = reinterpret_cast<float*>(a.C) + orow + col0 + c.ks * a.c_split_stride;
 #pragma unroll 1
         for (int ch = 0; ch < BN / 32; ++ch) {
           uint32_t r[32];
@@ -864,8 +945,11 @@ template <int BN, int STAGES, int EPI, bool PAIR = false>
 cudaError_t run(const GemmDesc& d, const KArgs& ka, int num_sms, cudaStream_t st) {
   using S = Smem<BN, STAGES, EPI, PAIR>;
   CUtensorMap ta, tb;
-  if (!make_map(&ta, d.A, d.a_rows_total, d.a_kwrap > 0 ? d.a_kwrap : d.K, kBM)) return cudaErrorInvalidValue;
-  if (!make_map(&tb, d.B, d.b_rows_total, d.b_kwrap > 0 ? d.b_kwrap : d.K, PAIR ? BN / 2 : BN))
+  const bool prod = d.pr.n > 0;
+  const int acols = prod ? d.pr.a_cols : (d.a_kwrap > 0 ? d.a_kwrap : d.K);
+  const int bcols = prod ? d.pr.b_cols : d.K;
+  if (!make_map(&ta, d.A, d.a_rows_total, acols, prod && d.pr.a_mn ? 64 : kBM)) return cudaErrorInvalidValue;
+  if (!make_map(&tb, d.B, d.b_rows_total, bcols, prod && d.pr.b_mn ? 64 : (PAIR ? BN / 2 : BN)))
     return cudaErrorInvalidValue;
   CUtensorMap tc = ta;
   if constexpr (S::TSTORE) {       // output [rows, ldc] bf16, 32x32 boxes, 64-byte swizzle
@@ -921,8 +1005,6 @@ cudaError_t run(const GemmDesc& d, const KArgs& ka, int num_sms, cudaStream_t st
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
   if (d.K <= 0 || d.K % kBK != 0 || d.M < 0 || d.N <= 0 || d.batch <= 0) return cudaErrorInvalidValue;
   if (d.a_kwrap < 0 || d.a_kwrap % kBK != 0 || d.a_kwrap > d.K) return cudaErrorInvalidValue;
-  if (d.b_kwrap < 0 || d.b_kwrap % kBK != 0 || d.b_kwrap > d.K || (d.b_kwrap > 0 && d.split3))
-    return cudaErrorInvalidValue;
   if (d.split3 && (d.K % (3 * kBK) != 0 || d.a_kwrap != 2 * (d.K / 3))) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(d.A) | reinterpret_cast<uintptr_t>(d.B)) & 15) return cudaErrorInvalidValue;
   if (d.M == 0) return cudaSuccess;
@@ -949,7 +1031,7 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
   ka.split_kind = d.split_kind; ka.scale = d.scale; ka.aux = d.aux; ka.b_off = d.b_off;
   ka.stats = d.stats; ka.stat_ld = d.stat_ld; ka.col_count = d.col_count;
   ka.b_base = d.b_base; ka.proj = d.proj;
-  ka.a_kwrap = d.a_kwrap; ka.b_kwrap = d.b_kwrap; ka.biasf = d.biasf; ka.split3 = d.split3;
+  ka.a_kwrap = d.a_kwrap; ka.biasf = d.biasf; ka.split3 = d.split3;
   ka.blist = d.blist; ka.bcount = d.blist ? d.bcount : nullptr;
   ka.m_limit = d.m_limit;
   ka.wait_ns = d.wait_ns > 0 ? static_cast<unsigned long long>(d.wait_ns) : kWaitLimitNs;
@@ -959,8 +1041,18 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
   ka.ksplit = d.ksplit; ka.c_split_stride = d.c_split_stride;
   if (d.blist && !d.bcount) return cudaErrorInvalidValue;
   if (d.sym && (d.A != d.B || d.a_row_stride != d.b_row_stride || d.a_rows_total != d.b_rows_total || d.b_off ||
-                d.a_kwrap || d.b_kwrap || d.split3))
+                d.a_kwrap || d.split3 || d.pr.n))
     return cudaErrorInvalidValue;
+  ka.pr = d.pr;
+  if (d.pr.n) {      // segments start at whole boxes; K is the products' K blocks side by side
+    const GemmProducts& q = d.pr;
+    if (d.epi != EPI_F32 || q.n < 0 || q.n > kMaxProducts || d.a_kwrap || d.split3 || d.b_off || d.b_base ||
+        q.kblocks <= 0 || d.K != q.n * q.kblocks * kBK || q.a_cols % 8 != 0 || q.b_cols % 8 != 0)
+      return cudaErrorInvalidValue;
+    for (int i = 0; i < q.n; ++i)
+      if (q.a_seg[i] < 0 || q.a_seg[i] % kBK != 0 || q.b_seg[i] < 0 || q.b_seg[i] % kBK != 0)
+        return cudaErrorInvalidValue;
+  }
   ka.sym = d.sym;
   ka.n_outer = d.n_outer;
   switch (d.epi) {

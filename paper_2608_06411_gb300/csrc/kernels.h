@@ -36,6 +36,22 @@ struct ProjArgs {
   float* r2; float* U; float* sqn; int32_t* cstep;   // [B, N] outputs
 };
 
+// EPI_F32 as a sum of products of column segments: C = sum_p A_p B_p^T, where A_p (B_p) is the
+// operand's array from column a_seg[p] (b_seg[p]) on.  An array of a_cols columns (row stride too)
+// is K-major (its rows are the operand's rows, K runs along a row) or, with a_mn, MN-major (its
+// rows are the K index, the operand's rows run along a row): no operand is transposed in memory.
+// Batched: an operand's array rows of entry b start at a_off[b] (device) or b * a_row_stride,
+// likewise B's; K per entry is k_count[b] (device; rows past it up to the next multiple of 64 must
+// be zero in one operand) or 64 * kblocks.  With a_off and a K-major A, C has A's rows.
+constexpr int kMaxProducts = 6;
+struct GemmProducts {
+  int n;                       // 0: a plain product
+  int kblocks;                 // 64-wide K blocks of one product (the most over the batch)
+  int a_seg[kMaxProducts], b_seg[kMaxProducts];
+  int a_mn, b_mn, a_cols, b_cols;
+  const int* a_off; const int* b_off; const int* k_count;
+};
+
 // Batched C = epi(A @ B^T): A rows [batch][a_row_stride] x K, B rows [batch][b_row_stride] x K
 // (both bf16, K contiguous, tightly packed 2D arrays of a_rows_total / b_rows_total rows).
 struct GemmDesc {
@@ -65,8 +81,6 @@ struct GemmDesc {
   // A has a_kwrap columns; its K coordinate wraps (k mod a_kwrap), so a K-segment of A can
   // be read twice against different B segments (0: A has K columns)
   int a_kwrap = 0;
-  // B has b_kwrap columns and its K coordinate wraps likewise (0: B has K columns)
-  int b_kwrap = 0;
   // split3 = 1 (with K = 3 Dh, A = [hi | lo] and B = [W_hi | W_hi | W_lo]): K blocks are taken
   // as (hi_j, W_hi_j), (hi_j, W_lo_j) for every j, then (lo_j, W_hi_j), so each block of A_hi
   // is read twice back to back (the second time from L2)
@@ -91,6 +105,7 @@ struct GemmDesc {
   // EPI_F32 split-K: ksplit K slices, each unit one slice of a tile, slice s writing its partial
   // sum at C + s * c_split_stride (elements, a multiple of 4); the caller adds the slices
   int ksplit = 1; long long c_split_stride = 0;
+  GemmProducts pr{};
 };
 
 // Returns cudaSuccess, or an error for an unsupported shape (cudaErrorInvalidValue).
@@ -140,37 +155,60 @@ cudaError_t launch_assemble(const void* V, const int32_t* idx, const void* T, co
                             cudaStream_t st);
 
 // ------------------------------------------------------------------ distillation step (fp32)
-// C[i, j] = alpha sum_k A(i, k) B(k, j) on the tcgen05 GEMM, fp32 in (or bf16: a_bf16 / b_bf16)
-// and fp32 out; row-major, A(i, k) = ta ? A[k lda + i] : A[i lda + k], B(k, j) = tb ? B[j ldb + k]
-// : B[k ldb + j].  fp32 operands are staged as three bf16 terms (split-bf16 products to fp32
-// accuracy, see distill.cu) in wsA / wsB, of at least the element counts tc_matmul_ws returns; C must be
-// 16-byte aligned with ldc % 4 == 0.  Deterministic (fixed summation order).
-// wsC: K-slice partial sums when the output has too few tiles to fill the GPU.  A bf16 operand
-// that is K-major, dense and 64-aligned is read in place.  *launches (if given) counts the
-// kernels launched.
-void tc_matmul_ws(int M, int N, int K, float alpha, bool a_bf16, bool b_bf16, int num_sms, size_t* a_elems,
-                  size_t* b_elems, size_t* c_elems);
-cudaError_t launch_tc_matmul(bool ta, bool tb, int M, int N, int K, float alpha, const void* A, bool a_bf16,
-                             long long lda, const void* B, bool b_bf16, long long ldb, float* C, long long ldc,
-                             void* wsA, void* wsB, float* wsC, int num_sms, int* status, long long wait_ns,
-                             cudaStream_t st, long long* launches);
-cudaError_t launch_bf16_to_f32(const void* x, long long n, float* y, cudaStream_t st);
-// z += b (per column); h = GELU(z)
-cudaError_t launch_bias_gelu(float* z, const float* b, long long rows, int cols, float* h, cudaStream_t st);
-cudaError_t launch_bias_add(float* x, const float* b, long long rows, int cols, cudaStream_t st);
-// RoPE (or its transpose when backward) on [rows, d] fp32 rows; positions pos[r] or r % pos_mod.
-cudaError_t launch_rope_f32(bool backward, const float* x, long long rows, int d, const float2* tab, int ld,
-                            const int32_t* pos, int pos_mod, float* y, cudaStream_t st);
-// S [total_m, N] logits of all images' question rows (row stride ld; image b: rows qoff[b] ..
-// qoff[b+1]) -> softmax, p_hat [B, N], g = dL/dp_hat, *loss = mean_b D_KL(teacher_b || p_hat_b),
-// then S is overwritten with dL/dlogits.  row_img [total_m]: image of each row; part: B * ceil(N/256)
-// floats.
-cudaError_t launch_distill_loss_grad(float* S, long long ld, long long total_m, const int32_t* qoff,
-                                     const int32_t* row_img, const float* teacher, int B, int N, float* p_hat,
-                                     float* g, float* part, float* loss, cudaStream_t st);
-// dh *= GELU'(z)
-cudaError_t launch_gelu_back(float* dh, const float* z, long long n, cudaStream_t st);
-// out[c] = sum_r X[r, c], in a fixed order; part: 64 * cols floats of workspace
-cudaError_t launch_colsum(const float* X, long long rows, int cols, float* part, float* out, cudaStream_t st);
+// A bf16 operand of a contraction: element (i, k) = p[i * cols + k] (mn = 0) or p[k * cols + i]
+// (mn = 1), `rows` array rows.  seg > 0: an fp32 operand as three bf16 terms hi, mid, lo at columns
+// 0, seg and 2 seg (split-bf16 products to fp32 accuracy, see distill.cu); 0: exact bf16.
+struct TcOperand {
+  const void* p; long long rows; int cols; int seg; int mn;
+};
+// Result of a contraction before its K slices are added: sum over s < ks of p[s * stride + row * ld
+// + col] (ks = 1: the result itself).
+struct TcResult {
+  const float* p; int ks; long long stride; long long ld;
+};
+// Batch of a contraction (device arrays; batch 1: none), as in GemmProducts / GemmDesc.
+struct TcBatch {
+  int n = 1;
+  const int* a_off = nullptr; int a_rows = 0;        // array rows of A per entry
+  const int* b_off = nullptr; int b_rows = 0;
+  const int* m_count = nullptr;                      // rows of C per entry
+  const int* k_count = nullptr;
+  long long c_stride = 0;                            // C elements per entry (without a_off)
+  long long c_rows = 0;                              // rows of C over the whole batch
+};
+// K slices launch_tc_matmul takes for an M x N output over K, and the floats its slices need.
+int tc_ksplit(int M, int N, int K, int products, int num_sms);
+int tc_products(bool a_split, bool b_split);
+// C[i, j] = sum_k A(i, k) B(j, k) on the tcgen05 GEMM, fp32 out, deterministic (fixed order).  With
+// one K slice the result is in C (16-byte aligned, ldc % 4 == 0); with more, the slices are in wsC
+// and, with add = true, their sum in C (else the consumer adds them).
+cudaError_t launch_tc_matmul(int M, int N, int K, const TcOperand& A, const TcOperand& B, const TcBatch& batch,
+                             int ksplit, bool add, float* C, long long ldc, float* wsC, int num_sms, int* status,
+                             long long wait_ns, cudaStream_t st, long long* launches, TcResult* res);
+// Rows of the padded question layout (each image's rows start at a multiple of 64): poff[b], the
+// padded row of every question row, and the image of every padded row (-1: padding).
+cudaError_t launch_distill_meta(const int32_t* len, const int32_t* off, int B, int32_t* poff, int32_t* prow,
+                                int32_t* img, cudaStream_t st);
+// x = GELU(in + bias) (gelu: in + bias goes to z) or in + bias, as three bf16 terms [rows, 3 cols].
+cudaError_t launch_act_split(bool gelu, const TcResult& in, const void* bias, long long rows, int cols, float* z,
+                             void* dst, cudaStream_t st);
+// x = in * GELU'(z) (z given) or in, as three bf16 terms, and its column sums (part: kColRows-row
+// partial sums, ceil(rows / 64) * cols floats).
+cudaError_t launch_back_split(const TcResult& in, const float* z, long long rows, int cols, void* dst, float* part,
+                              float* colsum, cudaStream_t st);
+// RoPE (or its transpose) of in [rows, d] times scale, as three bf16 terms at row in_map / out_map
+// (nullptr: the row itself).  Position pos[r] or r % pos_mod.
+cudaError_t launch_rope_split(bool backward, const TcResult& in, const int32_t* in_map, long long rows, int d,
+                              const float2* tab, int ld, const int32_t* pos, int pos_mod, float scale, void* dst,
+                              const int32_t* out_map, cudaStream_t st);
+// S [padded rows, ld] logits -> p_hat [B, N], g = dL/dp_hat, *loss = mean_b D_KL(teacher_b ||
+// p_hat_b), and dL/dlogits as three bf16 terms [padded rows, 3 seg] (zero in padding rows and past
+// column N).  part: B * ceil(N / 256) floats.  S is overwritten.
+cudaError_t launch_distill_loss_grad(float* S, long long ld, long long prows, const int32_t* len,
+                                     const int32_t* poff, const int32_t* img, const float* teacher, int B, int N,
+                                     float* p_hat, float* g, float* part, float* loss, void* dst, int seg,
+                                     cudaStream_t st);
+// Zeroes the padding rows of a [padded rows, cols] bf16 array.
+cudaError_t launch_zero_pad_rows(void* x, int cols, const int32_t* img, long long prows, cudaStream_t st);
 
 }  // namespace mapk

@@ -75,3 +75,28 @@ def test_distill_is_deterministic():
 def test_distill_llava_next_shape():
     """Full predictor widths (D = 4096, Dh = 1024, dp = 128), two N = 2880 images."""
     _check(W.PredictorDims(), W.WORKLOADS["c1"], 2, 2880, np.array([64, 23], np.int32), 14)
+
+
+@pytest.mark.parametrize("dp,N,lens", [(64, 64, [1]), (128, 65, [64, 1]), (64, 127, [65, 63, 2]), (128, 300, [129, 3])])
+def test_distill_edges_of_the_padded_question_rows(dp, N, lens):
+    """Question lengths around the 64 rows each image is padded to (and past one 128-row tile),
+    token counts around the 64-column blocks of the staged logits; the usual bounds."""
+    _check(W.PredictorDims(D=256, Dh=256, dp=dp), W.WORKLOADS["c0"], len(lens), N, np.array(lens, np.int32), 15)
+
+
+def test_distill_takes_features_at_any_even_address():
+    dims, lens = W.PredictorDims(D=256, Dh=256, dp=64), [7, 30]
+    ctx, vis, text, teacher, loss, grads = _check(dims, W.WORKLOADS["c0"], 2, 130, np.array(lens, np.int32), 16)
+
+    def shifted(a):                                    # the same values two bytes past a 16-byte boundary
+        flat = dev_bits(a).reshape(-1)
+        buf = torch.empty(flat.numel() + 8, dtype=torch.int16, device=DEV)
+        buf[1:1 + flat.numel()] = flat
+        return buf[1:1 + flat.numel()].view(a.shape)
+
+    loss2, grads2 = ctx.distill_grad(shifted(text), shifted(vis), lens, torch.from_numpy(teacher).to(DEV))
+    torch.cuda.synchronize()
+    ctx.check()
+    assert torch.equal(loss2, loss)
+    for name in DO.WEIGHT_NAMES:
+        assert torch.equal(grads2[name], grads[name]), name
