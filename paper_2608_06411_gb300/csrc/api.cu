@@ -180,6 +180,14 @@ int gemm(map_ctx* c, const GemmDesc& d, cudaStream_t st) {
   return cuda_err(e);
 }
 
+// The second stream of the question branch and its fork and join events.
+int ensure_aux(map_ctx* c) {
+  if (!c->s_aux) CU_TRY(cudaStreamCreateWithFlags(&c->s_aux, cudaStreamNonBlocking));
+  if (!c->ev_fork) CU_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+  if (!c->ev_join) CU_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+  return MAP_OK;
+}
+
 GemmDesc linear_desc(map_ctx* c, const void* x, long long rows, int K, const void* w, int Nout, const void* bias,
                      void* y, int epi) {
   GemmDesc d{};
@@ -274,9 +282,7 @@ int score_impl(map_ctx* c, const void* text, const void* vis, const int32_t* len
   MAP_TRY(ensure(c->qb, static_cast<size_t>(total_m) * dp3 * 2));
   // The two branches are independent until Eq. 3: the question branch runs on a second stream
   // (it fills SMs that a small batch's visual GEMMs leave idle), joined before the logits.
-  if (!c->s_aux) CU_TRY(cudaStreamCreateWithFlags(&c->s_aux, cudaStreamNonBlocking));
-  if (!c->ev_fork) CU_TRY(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-  if (!c->ev_join) CU_TRY(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+  MAP_TRY(ensure_aux(c));
   CU_TRY(cudaEventRecord(c->ev_fork, st));
   CU_TRY(cudaStreamWaitEvent(c->s_aux, c->ev_fork, 0));
   MAP_TRY(predictor_branch(c, text, total_m, c->w[0], c->w[1], c->wqt, c->bqt, c->th1, c->qb.p, 1,
@@ -901,6 +907,14 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
   const int Nk = (N + 63) / 64 * 64;                 // columns of a staged logits term
   const float rs = 1.0f / std::sqrt(static_cast<float>(dp));
   const float2* tab = static_cast<const float2*>(c->rope.p);
+  // The modalities meet only in Eq. 3 and its gradient: the question branch, a chain of launches
+  // too small to fill the GPU, runs on a second stream beside the visual one, forward and backward
+  // (4 samples of 2880 tokens: 922 -> 805 us, 2 of 576: 374 -> 253 us).
+  MAP_TRY(ensure_aux(c));
+  auto after = [&](cudaStream_t first, cudaStream_t then, cudaEvent_t e) -> int {
+    CU_TRY(cudaEventRecord(e, first));
+    return cuda_err(cudaStreamWaitEvent(then, e, 0));
+  };
   // One modality: its rows, weights (first index, projection), buffers and stream.
   struct Branch {
     long long T; const void* X; int i1, ip; cudaStream_t st;
@@ -913,7 +927,7 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
   Branch br[2] = {};
   br[0].T = Tv; br[0].X = vis_feats; br[0].i1 = 5; br[0].ip = 9; br[0].st = st;
   br[0].pos = nullptr; br[0].pos_mod = g.rope_on ? N : 1;
-  br[1].T = Tt; br[1].X = text_feats; br[1].i1 = 0; br[1].ip = 4; br[1].st = st;
+  br[1].T = Tt; br[1].X = text_feats; br[1].i1 = 0; br[1].ip = 4; br[1].st = c->s_aux;
   br[1].pos = g.rope_on ? post : nullptr; br[1].pos_mod = 1;
   const int ks_dq = mapk::tc_ksplit(max_m, idp, iN, 6, c->num_sms);
   auto slices = [&](long long M, int Nn, long long K, int products) {
@@ -1011,26 +1025,38 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
     launches += 5;
     return MAP_OK;
   };
-  MAP_TRY(forward(br[0], 1.f, kk, nullptr));
-  MAP_TRY(forward(br[1], rs, qq, prow));
-  CU_TRY(mapk::launch_zero_pad_rows(qq, 3 * idp, img, prows, br[1].st));
-  // Eq. 3 logits (q k / sqrt(dp), the scale is in q) of every image, softmax, KL, and dL/dlogits
-  TcBatch lb;
-  lb.n = B; lb.a_off = poff; lb.b_rows = iN; lb.m_count = d_len; lb.c_rows = prows;
-  MAP_TRY(mm(max_m, iN, dp, split(qq, prows, idp, 0), split(kk, Tv, idp, 0), lb, 1, false, S, Np, nullptr, st, nullptr));
-  CU_TRY(mapk::launch_distill_loss_grad(S, Np, prows, d_len, poff, img, teacher, B, N, p_hat, gb, part, loss, dl, Nk, st));
-  launches += 5;
-  // dk = dl^T q per image (K = its question rows, padded with zeros), dq = dl k (K = its tokens)
-  TcResult rk, rq;
-  TcBatch kb;
-  kb.n = B; kb.a_off = poff; kb.b_off = poff; kb.k_count = d_len; kb.c_stride = static_cast<long long>(N) * dp;
-  kb.c_rows = Tv;
-  MAP_TRY(mm(N, idp, max_m, split(dl, prows, Nk, 1), split(qq, prows, idp, 1), kb, 1, false, dk, dp, nullptr, br[0].st, &rk));
-  TcBatch qb;
-  qb.n = B; qb.a_off = poff; qb.b_rows = iN; qb.m_count = d_len; qb.c_rows = prows;
-  MAP_TRY(mm(max_m, idp, N, split(dl, prows, Nk, 0), split(kk, Tv, idp, 1), qb, ks_dq, false, dq, dp, ws_dq, br[1].st, &rq));
-  MAP_TRY(backward(br[0], rk, nullptr, 1.f));
-  MAP_TRY(backward(br[1], rq, prow, rs));
+  auto step = [&]() -> int {
+    MAP_TRY(after(st, c->s_aux, c->ev_fork));
+    MAP_TRY(forward(br[1], rs, qq, prow));
+    CU_TRY(mapk::launch_zero_pad_rows(qq, 3 * idp, img, prows, br[1].st));
+    MAP_TRY(forward(br[0], 1.f, kk, nullptr));
+    MAP_TRY(after(c->s_aux, st, c->ev_join));
+    // Eq. 3 logits (q k / sqrt(dp), the scale is in q) of every image, softmax, KL, and dL/dlogits
+    TcBatch lb;
+    lb.n = B; lb.a_off = poff; lb.b_rows = iN; lb.m_count = d_len; lb.c_rows = prows;
+    MAP_TRY(mm(max_m, iN, dp, split(qq, prows, idp, 0), split(kk, Tv, idp, 0), lb, 1, false, S, Np, nullptr, st, nullptr));
+    CU_TRY(mapk::launch_distill_loss_grad(S, Np, prows, d_len, poff, img, teacher, B, N, p_hat, gb, part, loss, dl, Nk, st));
+    launches += 5;
+    // dk = dl^T q per image (K = its question rows, padded with zeros), dq = dl k (K = its tokens)
+    TcResult rk, rq;
+    TcBatch kb;
+    kb.n = B; kb.a_off = poff; kb.b_off = poff; kb.k_count = d_len; kb.c_stride = static_cast<long long>(N) * dp;
+    kb.c_rows = Tv;
+    MAP_TRY(mm(N, idp, max_m, split(dl, prows, Nk, 1), split(qq, prows, idp, 1), kb, 1, false, dk, dp, nullptr, br[0].st, &rk));
+    MAP_TRY(after(st, c->s_aux, c->ev_fork));
+    TcBatch qb;
+    qb.n = B; qb.a_off = poff; qb.b_rows = iN; qb.m_count = d_len; qb.c_rows = prows;
+    MAP_TRY(mm(max_m, idp, N, split(dl, prows, Nk, 0), split(kk, Tv, idp, 1), qb, ks_dq, false, dq, dp, ws_dq, br[1].st, &rq));
+    MAP_TRY(backward(br[1], rq, prow, rs));
+    MAP_TRY(backward(br[0], rk, nullptr, 1.f));
+    MAP_TRY(after(c->s_aux, st, c->ev_join));
+    return MAP_OK;
+  };
+  const int rc = step();
+  if (rc != MAP_OK) {                                // what the second stream still runs comes first
+    after(c->s_aux, st, c->ev_join);
+    return rc;
+  }
   c->counters.launches += launches;
   return MAP_OK;
 }
