@@ -6,12 +6,17 @@
 //
 // The work is one streaming read of the attention maps (hundreds of MB per sample for a
 // 7B backbone), so it is HBM-bound; two launches:
-//   1. qcts_colsum_kernel: Eq. 1 column sums.  A cluster of 8 CTAs splits the rows (head,
-//      question token) of one (sample, layer, 512-column tile); each thread owns 8 adjacent
-//      columns (one 16-byte load per row) and one of 4 row phases, with 8 rows in flight.
-//      The 32 partial sums per column are added in a fixed order through distributed
-//      shared memory (each CTA of the cluster finishes 1/8 of the columns), so results do
-//      not depend on scheduling and no global scratch or atomics are needed.
+//   1. qcts_colsum_kernel: Eq. 1 column sums.  One CTA sums all rows (head, question token) of one
+//      (sample, layer) over a tile of 64 columns: a thread owns 8 adjacent columns (one aligned
+//      16-byte load per row, whatever N is) and one of 32 row phases, with 8 rows in flight, the
+//      last ones too.  The 32 partial sums per column are added in a fixed order through shared
+//      memory, so results do not depend on scheduling and no global scratch, atomics or other CTAs
+//      are needed.  (Clusters of 8 CTAs splitting a tile's rows and adding through distributed
+//      shared memory spent that time loading nothing, and narrower loads where N is not a multiple of 8
+//      had a quarter or less of the bytes in flight: 2 samples of 2880 tokens, 32 x 32 maps, 205 ->
+//      175 us per call, the time the measured copy rate takes; 4 of 576: 62 -> 35 us; N = 2881: 399 -> 87 us.)
+//      Samples with the most rows come first in the grid, so that the last CTAs to run
+//      are short.
 //   2. qcts_finish_kernel: one CTA per (sample, layer): l1 normalisation of both aggregates
 //      in place and the divergence; the last CTA of each sample to finish takes the argmax
 //      over layers (ties to the lower layer) and copies p^{l*}.
@@ -27,143 +32,132 @@
 namespace mapk {
 namespace {
 
-constexpr int kThreads = 256;
-constexpr int kColGroups = 64;                  // threads across the columns of a tile
-constexpr int kPhases = kThreads / kColGroups;  // threads down the rows
-constexpr int kCluster = 8;                     // CTAs splitting the rows of one tile
+constexpr int kTile = 64;                       // columns per tile
+constexpr int kPhases = 32;                     // threads down the rows
 constexpr int kUnroll = 8;                      // rows in flight per thread
+constexpr int kFinishThreads = 1024;
+static_assert(kFinishThreads == 32 * 32, "a warp adds the warps' sums");
 constexpr int kMaxSamples = 1024;               // samples per launch (kernel-parameter table)
 
 struct QctsMeta {
   int b0, count;       // global index of the first sample of this launch, samples in it
   int L, H, N, m_ref;
   int32_t lens[kMaxSamples];
+  int32_t order[kMaxSamples];    // samples of this launch, most rows first
   long long row0[kMaxSamples];   // first row (of N elements) of each sample's question block
 };
 
-template <int VEC> struct Load;
-template <> struct Load<8> {
-  using T = uint4;
-  static __device__ __forceinline__ T get(const uint16_t* p) { return __ldcs(reinterpret_cast<const uint4*>(p)); }
-  static __device__ __forceinline__ void add(const T& u, float* acc) {
-    acc[0] += __uint_as_float(u.x << 16);
-    acc[1] += __uint_as_float(u.x & 0xFFFF0000u);
-    acc[2] += __uint_as_float(u.y << 16);
-    acc[3] += __uint_as_float(u.y & 0xFFFF0000u);
-    acc[4] += __uint_as_float(u.z << 16);
-    acc[5] += __uint_as_float(u.z & 0xFFFF0000u);
-    acc[6] += __uint_as_float(u.w << 16);
-    acc[7] += __uint_as_float(u.w & 0xFFFF0000u);
-  }
-};
-template <> struct Load<2> {
-  using T = unsigned int;
-  static __device__ __forceinline__ T get(const uint16_t* p) {
-    return __ldcs(reinterpret_cast<const unsigned int*>(p));
-  }
-  static __device__ __forceinline__ void add(const T& u, float* acc) {
-    acc[0] += __uint_as_float(u << 16);
-    acc[1] += __uint_as_float(u & 0xFFFF0000u);
-  }
-};
-template <> struct Load<1> {
-  using T = unsigned short;
-  static __device__ __forceinline__ T get(const uint16_t* p) { return __ldcs(p); }
-  static __device__ __forceinline__ void add(const T& u, float* acc) {
-    acc[0] += __uint_as_float(static_cast<uint32_t>(u) << 16);
-  }
-};
+__device__ __forceinline__ float low_bf16(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float high_bf16(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
-// acc += rows p, p + stride, ... (n of them), kUnroll loads issued before their adds.
-template <int VEC>
-__device__ __forceinline__ void add_rows(const uint16_t* p, long long stride, long long n, float* acc) {
-  using L = Load<VEC>;
-  long long i = 0;
-  for (; i + kUnroll <= n; i += kUnroll) {
-    typename L::T x[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) x[u] = L::get(p + u * stride);
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) L::add(x[u], acc);
-    p += kUnroll * stride;
-  }
-  for (; i < n; ++i, p += stride) L::add(L::get(p), acc);
+// acc[0], acc[1] += the two columns of one 32-bit word of eight rows, added as a tree.
+__device__ __forceinline__ void add_words(const uint32_t (&w)[kUnroll], float* acc) {
+  static_assert(kUnroll == 8, "a tree of eight rows");
+  acc[0] += ((low_bf16(w[0]) + low_bf16(w[1])) + (low_bf16(w[2]) + low_bf16(w[3]))) +
+            ((low_bf16(w[4]) + low_bf16(w[5])) + (low_bf16(w[6]) + low_bf16(w[7])));
+  acc[1] += ((high_bf16(w[0]) + high_bf16(w[1])) + (high_bf16(w[2]) + high_bf16(w[3]))) +
+            ((high_bf16(w[4]) + high_bf16(w[5])) + (high_bf16(w[6]) + high_bf16(w[7])));
 }
 
-__device__ __forceinline__ float ld_shared_cluster_f32(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-  return v;
+// acc[v] += element v of the 16-byte chunks at p, p + step, ... (n of them), kUnroll loads issued
+// before their adds; the last, incomplete batch is loaded under predicates (a zero added for a
+// missing row), not row by row.  A chunk that reaches outside [lo, hi), the array (only its first
+// or last one can), is read element by element.
+__device__ __forceinline__ void add_rows(const uint16_t* p, long long step, long long n, const uint16_t* lo,
+                                         const uint16_t* hi, float* acc) {
+  auto by_element = [&](const uint16_t* q) {
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+      if (q + v >= lo && q + v < hi) acc[v] += __uint_as_float(static_cast<uint32_t>(q[v]) << 16);
+  };
+  if (n > 0 && p < lo) {
+    by_element(p);
+    p += step;
+    --n;
+  }
+  const bool last = n > 0 && p + (n - 1) * step + 8 > hi;
+  if (last) --n;
+  for (long long i = 0; i < n; i += kUnroll, p += kUnroll * step) {
+    uint4 x[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u)
+      x[u] = i + u < n ? __ldcs(reinterpret_cast<const uint4*>(p + u * step)) : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t w0[8] = {x[0].x, x[1].x, x[2].x, x[3].x, x[4].x, x[5].x, x[6].x, x[7].x};
+    const uint32_t w1[8] = {x[0].y, x[1].y, x[2].y, x[3].y, x[4].y, x[5].y, x[6].y, x[7].y};
+    const uint32_t w2[8] = {x[0].z, x[1].z, x[2].z, x[3].z, x[4].z, x[5].z, x[6].z, x[7].z};
+    const uint32_t w3[8] = {x[0].w, x[1].w, x[2].w, x[3].w, x[4].w, x[5].w, x[6].w, x[7].w};
+    add_words(w0, acc);
+    add_words(w1, acc + 2);
+    add_words(w2, acc + 4);
+    add_words(w3, acc + 6);
+    if (i + kUnroll >= n) {                     // p: the row after the last one
+      p += (n - i) * step;
+      break;
+    }
+  }
+  if (last) by_element(p);
 }
 
 // Eq. 1 for one (sample, layer, column tile): a[n] = 1/(H M) sum_{h, m} A[h, m, n] for the
 // question (into a_out) and 1/(H M_ref) sum for the reference question (into aref_out).
-// Grid (kCluster, column tiles, samples * L); cluster (kCluster, 1, 1).  No thread returns
-// before the two cluster barriers.
-template <int VEC>
-__global__ void __launch_bounds__(kThreads, 3) qcts_colsum_kernel(const __grid_constant__ QctsMeta m,
+// Grid (column tiles, L, samples).
+// Rows start at any even address (N need not be a multiple of 8), so the aligned chunks of a row
+// start up to 7 columns before the tile: by the same amount in every 32nd row, i.e. in all rows of
+// a thread.  GROUPS = 8 chunks cover the tile when rows are aligned (N % 8 == 0 and both arrays on
+// 16 bytes), 9 otherwise; the sums of columns outside the tile are dropped.
+template <int GROUPS>
+__global__ void __launch_bounds__(GROUPS * kPhases, 4) qcts_colsum_kernel(const __grid_constant__ QctsMeta m,
                                                                const uint16_t* __restrict__ attn,
+                                                               const uint16_t* __restrict__ attn_end,
                                                                const uint16_t* __restrict__ ref,
+                                                               const uint16_t* __restrict__ ref_end,
                                                                float* __restrict__ a_out,
                                                                float* __restrict__ aref_out,
                                                                int32_t* __restrict__ teacher) {
-  constexpr int W = kColGroups * VEC;       // columns per tile
-  constexpr int kPer = W / kCluster;        // columns each CTA finishes
-  __shared__ float part[2][kPhases][W];
+  __shared__ float part[2][kPhases][kTile];
   pdl_enter();
-  const int rank = static_cast<int>(cluster_ctarank());
-  const int tile = blockIdx.y;
-  const int bl = blockIdx.z / m.L, l = blockIdx.z - bl * m.L;
+  const int tile = blockIdx.x, l = blockIdx.y, bl = m.order[blockIdx.z];
   const long long b = m.b0 + bl;
   const int N = m.N;
-  const int cg = threadIdx.x % kColGroups, ph = threadIdx.x / kColGroups;
-  const long long col = static_cast<long long>(tile) * W + cg * VEC;
-  if (rank == 0 && tile == 0 && l == 0 && threadIdx.x == 0) teacher[b] = 0;   // finish-kernel counter
+  const int cg = threadIdx.x % GROUPS, ph = threadIdx.x / GROUPS;
+  const int c0 = tile * kTile;
+  if (tile == 0 && l == 0 && threadIdx.x == 0) teacher[b] = 0;   // finish-kernel counter
 
-  float acc_q[VEC], acc_r[VEC];
+  const long long Rq = static_cast<long long>(m.H) * m.lens[bl], Rr = static_cast<long long>(m.H) * m.m_ref;
+  const long long step = static_cast<long long>(kPhases) * N;
 #pragma unroll
-  for (int v = 0; v < VEC; ++v) acc_q[v] = acc_r[v] = 0.f;
-  if (col < N) {   // N % VEC == 0: the whole group is inside the row
-    const long long Rq = static_cast<long long>(m.H) * m.lens[bl];
-    const long long q_begin = Rq * rank / kCluster, q_end = Rq * (rank + 1) / kCluster;
-    const long long nq = q_end - q_begin - ph > 0 ? (q_end - q_begin - ph + kPhases - 1) / kPhases : 0;
-    const uint16_t* pq = attn + (m.row0[bl] + l * Rq + q_begin + ph) * N + col;
-    add_rows<VEC>(pq, static_cast<long long>(kPhases) * N, nq, acc_q);
-
-    const long long Rr = static_cast<long long>(m.H) * m.m_ref;
-    const long long r_begin = Rr * rank / kCluster, r_end = Rr * (rank + 1) / kCluster;
-    const long long nr = r_end - r_begin - ph > 0 ? (r_end - r_begin - ph + kPhases - 1) / kPhases : 0;
-    const uint16_t* pr = ref + ((b * m.L + l) * Rr + r_begin + ph) * N + col;
-    add_rows<VEC>(pr, static_cast<long long>(kPhases) * N, nr, acc_r);
-  }
+  for (int which = 1; which >= 0; --which) {    // the reference's few rows, then the question's
+    const long long R = which ? Rr : Rq;
+    const uint16_t* row = which ? ref + ((b * m.L + l) * Rr + ph) * N : attn + (m.row0[bl] + l * Rq + ph) * N;
+    const int s = GROUPS == 8 ? 0 : static_cast<int>((reinterpret_cast<uintptr_t>(row + c0) >> 1) & 7u);
+    const int k0 = cg * 8 - s;                  // the chunk's first column, from the tile's
+    float acc[8];
 #pragma unroll
-  for (int v = 0; v < VEC; ++v) {
-    part[0][ph][cg * VEC + v] = acc_q[v];
-    part[1][ph][cg * VEC + v] = acc_r[v];
+    for (int v = 0; v < 8; ++v) acc[v] = 0.f;
+    if (c0 + k0 < N && k0 < kTile)
+      add_rows(row + c0 + k0, step, ph < R ? (R - ph + kPhases - 1) / kPhases : 0, which ? ref : attn,
+               which ? ref_end : attn_end, acc);
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+      if (GROUPS == 8 || (k0 + v >= 0 && k0 + v < kTile)) part[which][ph][k0 + v] = acc[v];
   }
-  cluster_sync();   // every CTA's partials are written
-
+  __syncthreads();
   const int Mb = m.lens[bl];
   const float scale_q = Mb > 0 ? 1.0f / (static_cast<float>(m.H) * static_cast<float>(Mb)) : 0.f;
   const float scale_r = 1.0f / (static_cast<float>(m.H) * static_cast<float>(m.m_ref));
-  for (int i = threadIdx.x; i < 2 * kPer; i += kThreads) {
-    const int which = i / kPer;
-    const int c = rank * kPer + (i - which * kPer);
+  for (int i = threadIdx.x; i < 2 * kTile; i += GROUPS * kPhases) {
+    const int which = i / kTile, c = i - which * kTile;
     float s = 0.f;
-    for (int src = 0; src < kCluster; ++src) {
 #pragma unroll
-      for (int p = 0; p < kPhases; ++p) s += ld_shared_cluster_f32(mapa_u32(&part[which][p][c], src));
-    }
-    const long long gcol = static_cast<long long>(tile) * W + c;
-    if (gcol < N) {
+    for (int p = 0; p < kPhases; ++p) s += part[which][p][c];
+    if (c0 + c < N) {
       float* out = which ? aref_out : a_out;
-      out[(b * m.L + l) * N + gcol] = s * (which ? scale_r : scale_q);
+      out[(b * m.L + l) * N + c0 + c] = s * (which ? scale_r : scale_q);
     }
   }
-  cluster_sync();   // no CTA leaves while a peer may still read its shared memory
 }
 
-// Deterministic block sum of two values (256 threads): warp trees, then warp 0 in order.
+// Deterministic block sum of two values (kFinishThreads threads): trees within and over the warps.
 __device__ __forceinline__ float2 block_sum2(float x, float y, float2* red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -173,16 +167,17 @@ __device__ __forceinline__ float2 block_sum2(float x, float y, float2* red) {
   const int w = threadIdx.x >> 5;
   if ((threadIdx.x & 31) == 0) red[w] = make_float2(x, y);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float2 s = red[0];
-    for (int i = 1; i < kThreads / 32; ++i) {
-      s.x += red[i].x;
-      s.y += red[i].y;
+  if (threadIdx.x < 32) {
+    float2 s = red[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
     }
-    red[kThreads / 32] = s;
+    if (threadIdx.x == 0) red[kFinishThreads / 32] = s;
   }
   __syncthreads();
-  const float2 r = red[kThreads / 32];
+  const float2 r = red[kFinishThreads / 32];
   __syncthreads();   // red may be reused
   return r;
 }
@@ -212,11 +207,11 @@ __device__ __forceinline__ float js_term(float pn, float qn) {
 // l* = argmax_l js (ties to the lower layer), writes it over the count and copies p^{l*} to
 // teacher_p.  V4: N % 4 == 0 and 16-byte aligned rows (float4 accesses).
 template <bool V4>
-__global__ void __launch_bounds__(kThreads) qcts_finish_kernel(int L, int N, int b0, float* __restrict__ p,
+__global__ void __launch_bounds__(kFinishThreads) qcts_finish_kernel(int L, int N, int b0, float* __restrict__ p,
                                                                float* __restrict__ pref, float* __restrict__ js,
                                                                int32_t* __restrict__ teacher,
                                                                float* __restrict__ teacher_p) {
-  __shared__ float2 red[kThreads / 32 + 1];
+  __shared__ float2 red[kFinishThreads / 32 + 1];
   __shared__ int last;
   pdl_enter();
   const long long b = b0 + blockIdx.y;
@@ -230,14 +225,14 @@ __global__ void __launch_bounds__(kThreads) qcts_finish_kernel(int L, int N, int
     float4* a4 = reinterpret_cast<float4*>(a);
     float4* r4 = reinterpret_cast<float4*>(r);
     float sa = 0.f, sr = 0.f;
-    for (int i = threadIdx.x; i < n4; i += kThreads) {
+    for (int i = threadIdx.x; i < n4; i += kFinishThreads) {
       const float4 x = a4[i], y = r4[i];
       sa += (x.x + x.y) + (x.z + x.w);
       sr += (y.x + y.y) + (y.z + y.w);
     }
     const float2 s = block_sum2(sa, sr, red);
     const bool ua = !(s.x > 0.f), ur = !(s.y > 0.f);
-    for (int i = threadIdx.x; i < n4; i += kThreads) {
+    for (int i = threadIdx.x; i < n4; i += kFinishThreads) {
       const float4 x = a4[i], y = r4[i];
       const float4 pn = ua ? make_float4(inv_n, inv_n, inv_n, inv_n)
                            : make_float4(x.x / s.x, x.y / s.x, x.z / s.x, x.w / s.x);
@@ -249,13 +244,13 @@ __global__ void __launch_bounds__(kThreads) qcts_finish_kernel(int L, int N, int
     }
   } else {
     float sa = 0.f, sr = 0.f;
-    for (int n = threadIdx.x; n < N; n += kThreads) {
+    for (int n = threadIdx.x; n < N; n += kFinishThreads) {
       sa += a[n];
       sr += r[n];
     }
     const float2 s = block_sum2(sa, sr, red);
     const bool ua = !(s.x > 0.f), ur = !(s.y > 0.f);
-    for (int n = threadIdx.x; n < N; n += kThreads) {
+    for (int n = threadIdx.x; n < N; n += kFinishThreads) {
       const float pn = ua ? inv_n : a[n] / s.x;
       const float qn = ur ? inv_n : r[n] / s.y;
       a[n] = pn;
@@ -301,37 +296,16 @@ __global__ void __launch_bounds__(kThreads) qcts_finish_kernel(int L, int N, int
   __syncthreads();
   if (teacher_p != nullptr) {
     const float* src = p + (b * L + best_l) * N;
-    for (int n = threadIdx.x; n < N; n += kThreads) teacher_p[b * N + n] = __ldcg(src + n);
+    for (int n = threadIdx.x; n < N; n += kFinishThreads) teacher_p[b * N + n] = __ldcg(src + n);
   }
 }
 
-template <typename... KParams, typename... Args>
-cudaError_t launch_cluster(void (*kern)(KParams...), dim3 grid, dim3 block, unsigned cx, cudaStream_t st,
-                           Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cx;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-}
-
-template <int VEC>
-cudaError_t launch_colsum(const QctsMeta& m, const void* attn, const void* ref, float* p, float* pref,
-                          int32_t* teacher, cudaStream_t st) {
-  constexpr int W = kColGroups * VEC;
-  const dim3 grid(kCluster, (m.N + W - 1) / W, m.count * m.L);
-  return launch_cluster(qcts_colsum_kernel<VEC>, grid, dim3(kThreads), kCluster, st, m,
-                        static_cast<const uint16_t*>(attn), static_cast<const uint16_t*>(ref), p, pref, teacher);
+template <int GROUPS>
+cudaError_t launch_colsum(const QctsMeta& m, const uint16_t* attn, const uint16_t* attn_end, const uint16_t* ref,
+                          const uint16_t* ref_end, float* p, float* pref, int32_t* teacher, cudaStream_t st) {
+  const dim3 grid((m.N + kTile - 1) / kTile, m.L, m.count);
+  return launch_k(qcts_colsum_kernel<GROUPS>, grid, dim3(GROUPS * kPhases), 0, st, m, attn, attn_end, ref, ref_end, p,
+                  pref, teacher);
 }
 
 }  // namespace
@@ -342,18 +316,22 @@ extern "C" int map_qcts(const void* attn, const int32_t* lens, const void* attn_
   using namespace mapk;
   if (!attn || !lens || !attn_ref || !p || !p_ref || !js || !teacher) return MAP_EINVAL;
   if (B < 1 || L < 1 || H < 1 || N < 1 || M_ref < 1) return MAP_EINVAL;
-  if (L > 65535 || (static_cast<long long>(N) + kColGroups - 1) / kColGroups > 65535) return MAP_EUNSUPPORTED;
+  if (L > 65535 || (static_cast<long long>(N) + 63) / 64 > 65535) return MAP_EUNSUPPORTED;
   for (int b = 0; b < B; ++b)
     if (lens[b] < 0) return MAP_EINVAL;
   const uintptr_t ua = reinterpret_cast<uintptr_t>(attn), ur = reinterpret_cast<uintptr_t>(attn_ref);
   if ((ua | ur) & 1u) return MAP_EINVAL;
-  int vec = 1;
-  if (N % 8 == 0 && ((ua | ur) & 15u) == 0) vec = 8;
-  else if (N % 2 == 0 && ((ua | ur) & 3u) == 0) vec = 2;
+  const bool aligned = N % 8 == 0 && ((ua | ur) & 15u) == 0;
+  long long rows = 0;                                          // of all question blocks
+  for (int b = 0; b < B; ++b) rows += static_cast<long long>(L) * H * lens[b];
+  const uint16_t* a16 = static_cast<const uint16_t*>(attn);
+  const uint16_t* r16 = static_cast<const uint16_t*>(attn_ref);
+  const uint16_t* a_end = a16 + rows * N;
+  const uint16_t* r_end = r16 + static_cast<long long>(B) * L * H * M_ref * N;
   const bool v4 = N % 4 == 0 && ((reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(p_ref)) & 15u) == 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-  // samples per launch: the parameter table and gridDim.z = samples * L
+  // samples per launch: the parameter table, and at most 65535 rows of the finish grid
   const int per_launch = std::max(1, std::min(kMaxSamples, 65535 / L));
   std::unique_ptr<QctsMeta> mp(new (std::nothrow) QctsMeta);   // ~12 KB, copied into the launch parameters
   if (!mp) return MAP_ENOMEM;
@@ -370,15 +348,16 @@ extern "C" int map_qcts(const void* attn, const int32_t* lens, const void* attn_
       m.lens[i] = lens[b0 + i];
       m.row0[i] = row;
       row += static_cast<long long>(L) * H * lens[b0 + i];
+      m.order[i] = i;
     }
-    cudaError_t e = vec == 8 ? launch_colsum<8>(m, attn, attn_ref, p, p_ref, teacher, st)
-                  : vec == 2 ? launch_colsum<2>(m, attn, attn_ref, p, p_ref, teacher, st)
-                             : launch_colsum<1>(m, attn, attn_ref, p, p_ref, teacher, st);
+    std::stable_sort(m.order, m.order + m.count, [&](int32_t x, int32_t y) { return m.lens[x] > m.lens[y]; });
+    cudaError_t e = aligned ? launch_colsum<8>(m, a16, a_end, r16, r_end, p, p_ref, teacher, st)
+                            : launch_colsum<9>(m, a16, a_end, r16, r_end, p, p_ref, teacher, st);
     if (e == cudaSuccess)
-      e = v4 ? launch_k(qcts_finish_kernel<true>, dim3(L, m.count), dim3(kThreads), 0, st, L, N, b0, p, p_ref, js,
+      e = v4 ? launch_k(qcts_finish_kernel<true>, dim3(L, m.count), dim3(kFinishThreads), 0, st, L, N, b0, p, p_ref, js,
                         teacher, teacher_p)
-             : launch_k(qcts_finish_kernel<false>, dim3(L, m.count), dim3(kThreads), 0, st, L, N, b0, p, p_ref,
-                        js, teacher, teacher_p);
+             : launch_k(qcts_finish_kernel<false>, dim3(L, m.count), dim3(kFinishThreads), 0, st, L, N, b0, p,
+                        p_ref, js, teacher, teacher_p);
     if (e != cudaSuccess) {
       cudaGetLastError();
       return e == cudaErrorInvalidValue ? MAP_EINVAL : MAP_ECUDA;

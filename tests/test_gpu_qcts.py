@@ -98,3 +98,22 @@ def test_qcts_many_layers_split_over_launches(mb):
     ref = W.f32_to_bf16_bits(rng.random((2, L, H, 1, N), dtype=np.float32))
     out = _run(mb, attn, lens, ref, L, H, N)
     _compare(Q.qcts_batch(attn, lens, ref, L, H, N), *out)
+
+
+@pytest.mark.parametrize("N,shift", [(63, 0), (65, 1), (64, 3), (71, 7), (8, 5)])
+def test_qcts_rows_at_any_even_address(mb, N, shift):
+    """Rows that start anywhere in a 16-byte chunk (odd N, arrays off their 16-byte boundary), the
+    first and last chunks reaching outside the arrays, tiles ending raggedly: as the oracle."""
+    w = W.AttentionWorkload("t3", 95, 2, 3, 2, 1, 24, 1, 9, 3)
+    lens = np.array([3, 40], np.int32)
+    attn, lens, ref = W.make_attention_batch(w, lens=lens, N=N)
+
+    def put(a):
+        flat = _dev(a).reshape(-1)
+        buf = torch.empty(flat.numel() + shift, dtype=flat.dtype, device=flat.device)
+        buf[shift:] = flat
+        return buf[shift:].view(a.shape)
+
+    out = mb.qcts(put(attn), lens, put(ref), w.L, w.H, N)
+    torch.cuda.synchronize()
+    _compare(Q.qcts_batch(attn, lens, ref, w.L, w.H, N), *[x.cpu().numpy() for x in out])
