@@ -19,7 +19,7 @@ using mapk::GemmDesc;
 namespace {
 
 constexpr int kMaxKDiverse = 768;   // k limit when the diversity term is on (the coordinate update
-                                    // stages 32 slot rows and 32 basis rows of k floats in shared memory)
+                                    // stages slot rows and 32 basis rows of k floats in shared memory)
 constexpr int kProjMaxBasis = 128;  // basis vectors one projection pass takes
 constexpr int kMaxK = 4096;
 constexpr int kMaxN = 16384;

@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kGatherThreads) sel_gather_kernel(SelState s) 
 // Per-slot coordinate rows in shared memory have a pitch of 4 (mod 8) floats, so that eight
 // lanes reading 16 bytes each from eight rows hit disjoint banks.
 constexpr int kChunk = 32;
-constexpr int kUpdSlots = 32;
+constexpr int kUpdSlots = 16;
 constexpr int kRoundPitch = kRoundPicks + 4;
 
 __host__ __device__ inline int coord_pitch(int KP) { return ((KP + 7) / 8) * 8 + 4; }
@@ -357,25 +357,31 @@ __host__ __device__ inline int coord_pitch(int KP) { return ((KP + 7) / 8) * 8 +
 // Brings every active token's coordinates up to the current basis (nb vectors) by forward
 // substitution before the picks:
 //   e_beta[i] = (G[j_beta, i] - sum_{beta' < beta} e_beta'[j_beta] e_beta'[i]) / r_beta,
-// 32 basis vectors (a chunk) at a time.  A CTA serves 32 slots, their coordinate rows in
-// shared memory.  For a chunk starting at b0 the products with the coordinates before it,
-// P[slot][row] = sum_{q < b0} e_q[slot] L[row][q] (L rows: the chunk's basis tokens' own
-// coordinate rows), form a 32 x 32 x b0 matrix product: each warp takes every fourth
-// 16-column block with 4 slots x 8 rows per thread (every loaded value feeds 4 or 8 FMAs).
-// Warp 0 then adds the four partial products and solves the chunk's 32 x 32 triangle
-// right-looking (lane = slot: each new coordinate is subtracted from the later ones at once,
-// so a step waits for one FMA), while warps 1-3 copy the next chunk's L rows, triangle,
-// Gram entries and basis norms into shared memory (cp.async), so that no chunk waits for a
-// global load.  An image's slots spread over S / 32 CTAs.  Writes Ec, r2 and cstep = nb.
-constexpr int kUpdWarps = 4;
+// 32 basis vectors (a chunk) at a time.  The slots are independent, the chunks are not: what
+// bounds it is a chunk's latency, so a CTA serves only 16 slots (16 CTAs an image), their
+// coordinate rows in shared memory.  For a chunk starting at b0 the products with the coordinates
+// before it, P[slot][row] = sum_{q < b0} e_q[slot] L[row][q] (L rows: the chunk's basis tokens' own
+// coordinate rows), form a 16 x 32 x b0 matrix product: each warp takes every eighth
+// 16-column block with 4 slots x 4 rows per thread, then each thread adds the eight partial
+// products of two entries.  Warp 0 solves the chunk's 32 x 32 triangle right-looking (lane = slot:
+// each new coordinate is subtracted from the later ones at once), dividing by the basis norm as a
+// product with its reciprocal and one correction step (the quotient to the last bit or nearly so,
+// without the division's chain in every step), while the other warps copy the next chunk's L rows,
+// triangle, Gram entries and basis norms into shared memory (cp.async), so that no chunk waits for
+// a global load.  Writes Ec, r2 and cstep = nb.
+// 200 vectors 49 us -> 20 us, 600 vectors (19 chunks) about 180 -> 103 us with 32 slots and four
+// warps a CTA before; 8 slots a CTA were slower in a batch (16 images: the L rows are copied
+// twice as often).
+constexpr int kUpdWarps = 8;
 
-__global__ void __launch_bounds__(kUpdSlots * kUpdWarps, 1) sel_update_kernel(SelState s) {
+__global__ void __launch_bounds__(32 * kUpdWarps) sel_update_kernel(SelState s) {
   pdl_enter();
-  extern __shared__ __align__(16) float shu[];           // [32][P] slot rows, then [32][KP] L rows
+  extern __shared__ __align__(16) float shu[];           // [kUpdSlots][P] slot rows, then [32][P] L rows
   __shared__ float Lt[2][kChunk][kChunk + 1];            // a chunk's triangle L[i][b0 + q], q < i
   __shared__ float gsm[2][kUpdSlots][kChunk + 1];        // its Gram entries G[slot][b0 + i]
   __shared__ float rn[2][kChunk];                        // its basis norms
   __shared__ float part[kUpdWarps][kUpdSlots][kChunk + 1];
+  static_assert(kUpdSlots * kChunk == 2 * 32 * kUpdWarps, "two entries of a chunk per thread");
   __shared__ int tok_s[kUpdSlots], c0_s[kUpdSlots];
   const int b = blockIdx.y;
   if (s.done[b]) return;
@@ -402,7 +408,7 @@ __global__ void __launch_bounds__(kUpdSlots * kUpdWarps, 1) sel_update_kernel(Se
     const int nch = min(nb, c + kChunk) - c, v4 = c / 4;
     for (int e = t0; e < nch * v4; e += stride) {    // L rows, columns [0, c)
       const int row = e / v4, q = (e - row * v4) * 4;
-      cp_async16(Lb + row * KP + q, s.Ec + (base + __ldg(btok_g + c + row)) * KP + q);
+      cp_async16(Lb + row * P + q, s.Ec + (base + __ldg(btok_g + c + row)) * KP + q);
     }
     for (int e = t0; e < nch * kChunk; e += stride) {   // the triangle: row i, columns c .. c + i - 1
       const int i = e / kChunk, q = e - i * kChunk;
@@ -424,33 +430,33 @@ __global__ void __launch_bounds__(kUpdSlots * kUpdWarps, 1) sel_update_kernel(Se
   }
   const int first = (cmin / kChunk) * kChunk;
   stage(first, 0, threadIdx.x, blockDim.x);
-  const int mtok = tok_s[lane], mc0 = c0_s[lane];    // warp 0: this lane's slot
+  const int mtok = lane < kUpdSlots ? tok_s[lane] : -1, mc0 = lane < kUpdSlots ? c0_s[lane] : nb;   // warp 0: this lane's slot
   float r2 = warp == 0 && mtok >= 0 ? s.r2[base + mtok] : 0.f;
-  const int sg = lane >> 2, rg = lane & 3;           // products: slots 4 sg + 0..3, rows rg + 4 j
+  const int sg = lane >> 3, rg = lane & 7;           // products: slots 4 sg + 0..3, rows rg + 8 j
   int buf = 0;
   for (int b0 = first; b0 < nb; b0 += kChunk, buf ^= 1) {
     const int nch = min(nb, b0 + kChunk) - b0;
     cp_async_wait_all();                             // this chunk's copies (and the slot rows)
     __syncthreads();
-    float acc[4][8];
+    float acc[4][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[u][j] = 0.f;
+      for (int j = 0; j < 4; ++j) acc[u][j] = 0.f;
     for (int qa = 16 * warp; qa < b0; qa += 16 * kUpdWarps) {   // whole 16-column blocks (b0 % 32 == 0)
 #pragma unroll
       for (int q4 = 0; q4 < 16; q4 += 4) {
-        float4 m[4], l[8];
+        float4 m[4], l[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) m[u] = *reinterpret_cast<const float4*>(shu + (4 * sg + u) * P + qa + q4);
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-          l[j] = rg + 4 * j < nch ? *reinterpret_cast<const float4*>(Lb + (rg + 4 * j) * KP + qa + q4)
+        for (int j = 0; j < 4; ++j)
+          l[j] = rg + 8 * j < nch ? *reinterpret_cast<const float4*>(Lb + (rg + 8 * j) * P + qa + q4)
                                   : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
+          for (int j = 0; j < 4; ++j) {
             float t = acc[u][j];
             t = fmaf(m[u].x, l[j].x, t);
             t = fmaf(m[u].y, l[j].y, t);
@@ -462,29 +468,39 @@ __global__ void __launch_bounds__(kUpdSlots * kUpdWarps, 1) sel_update_kernel(Se
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-      for (int j = 0; j < 8; ++j) part[warp][4 * sg + u][rg + 4 * j] = acc[u][j];
+      for (int j = 0; j < 4; ++j) part[warp][4 * sg + u][rg + 8 * j] = acc[u][j];
     __syncthreads();                                 // products done: Lb is free
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {                    // a thread reads and writes its own entries only
+      const int sl = warp + kUpdWarps * h;
+      part[0][sl][lane] =
+          gsm[buf][sl][lane] - (((part[0][sl][lane] + part[1][sl][lane]) + (part[2][sl][lane] + part[3][sl][lane])) +
+                                ((part[4][sl][lane] + part[5][sl][lane]) + (part[6][sl][lane] + part[7][sl][lane])));
+    }
+    __syncthreads();
     if (warp != 0) {
       if (b0 + kChunk < nb) stage(b0 + kChunk, buf ^ 1, threadIdx.x - 32, blockDim.x - 32);
-    } else if (mtok >= 0) {
+    } else {
+      const float my_rn = lane < nch ? rn[buf][lane] : 1.f, my_inv = 1.0f / my_rn;
       float* me = shu + lane * P;
       float av[kChunk];
 #pragma unroll
-      for (int i = 0; i < kChunk; ++i)
-        av[i] = (i < nch && b0 + i >= mc0)
-                    ? gsm[buf][lane][i] - ((part[0][lane][i] + part[1][lane][i]) + (part[2][lane][i] + part[3][lane][i]))
-                    : 0.f;
+      for (int i = 0; i < kChunk; ++i) av[i] = mtok >= 0 && i < nch && b0 + i >= mc0 ? part[0][lane][i] : 0.f;
 #pragma unroll
       for (int i = 0; i < kChunk; ++i) {
-        if (i < nch) {
+        const float ri = __shfl_sync(0xffffffffu, my_inv, i), rr = __shfl_sync(0xffffffffu, my_rn, i);
+        if (i < nch) {                               // uniform
           const int beta = b0 + i;
-          float ei;
-          if (beta >= mc0) {
-            ei = av[i] / rn[buf][i];
-            me[beta] = ei;
-            r2 = fmaf(-ei, ei, r2);
-          } else {
-            ei = me[beta];
+          float ei = 0.f;
+          if (mtok >= 0) {
+            if (beta >= mc0) {
+              ei = av[i] * ri;
+              ei = fmaf(fmaf(-ei, rr, av[i]), ri, ei);
+              me[beta] = ei;
+              r2 = fmaf(-ei, ei, r2);
+            } else {
+              ei = me[beta];
+            }
           }
 #pragma unroll
           for (int j = i + 1; j < kChunk; ++j) av[j] = fmaf(-Lt[buf][j][i], ei, av[j]);
@@ -1200,7 +1216,7 @@ size_t sel_chol_smem(int K0) {
   return static_cast<size_t>(chol_row((K0 + 31) / 32 * 32)) * 4;
 }
 size_t sel_update_smem(int KP) {
-  return (static_cast<size_t>(kUpdSlots) * coord_pitch(KP) + static_cast<size_t>(kChunk) * KP) * 4;
+  return static_cast<size_t>(kUpdSlots + kChunk) * coord_pitch(KP) * 4;
 }
 
 cudaError_t launch_sel_init(const SelState& s, cudaStream_t st) {
@@ -1223,7 +1239,7 @@ cudaError_t launch_sel_greedy(const SelState& s, cudaStream_t st) {
   const size_t um = sel_update_smem(s.KP);
   cudaError_t e = cudaFuncSetAttribute(sel_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(um));
   if (e != cudaSuccess) return e;
-  e = launch_k(sel_update_kernel, dim3((s.S + kUpdSlots - 1) / kUpdSlots, s.B), dim3(kUpdSlots * kUpdWarps), um, st, s);
+  e = launch_k(sel_update_kernel, dim3((s.S + kUpdSlots - 1) / kUpdSlots, s.B), dim3(32 * kUpdWarps), um, st, s);
   if (e != cudaSuccess) return e;
   const int T = s.S / kRgTile;
   e = launch_k(sel_resgram_kernel, dim3(T * (T + 1) / 2, s.B), dim3(kRgThreads), 0, st, s);
