@@ -207,13 +207,14 @@ GemmDesc linear_desc(map_ctx* c, const void* x, long long rows, int K, const voi
 // the second layer and the projection are one folded matrix Wf = Wp W2 with bias Wp b2.
 int predictor_branch(map_ctx* c, const void* x, long long rows, const void* w1, const void* b1, const void* wf,
                      const float* bf, DevBuf& h1, void* out3, int split_kind, float scale, float* aux,
-                     const int* pos, int pos_mod, cudaStream_t st, int tid_l1, int tid_p) {
+                     const int* pos, int pos_mod, int tile_n, cudaStream_t st, int tid_l1, int tid_p) {
   const map_config& g = c->cfg;
   MAP_TRY(ensure(h1, static_cast<size_t>(rows) * g.Dh * 4));
   {
     Timed t(c, st, tid_l1);
     GemmDesc d = linear_desc(c, x, rows, g.D, w1, g.Dh, b1, h1.p, mapk::EPI_GELU_SPLIT);
     d.ldc = 2LL * g.Dh;
+    d.tile_n = tile_n;
     MAP_TRY(gemm(c, d, st));
   }
   {
@@ -283,14 +284,16 @@ int score_impl(map_ctx* c, const void* text, const void* vis, const int32_t* len
   // The two branches are independent until Eq. 3: the question branch runs on a second stream
   // (it fills SMs that a small batch's visual GEMMs leave idle), joined before the logits.
   MAP_TRY(ensure_aux(c));
+  int tile_v = 0, tile_t = 0;
+  mapk::predictor_tile_widths(static_cast<int>(vrows), static_cast<int>(total_m), g.Dh, g.D, c->num_sms, &tile_v, &tile_t);
   CU_TRY(cudaEventRecord(c->ev_fork, st));
   CU_TRY(cudaStreamWaitEvent(c->s_aux, c->ev_fork, 0));
   MAP_TRY(predictor_branch(c, text, total_m, c->w[0], c->w[1], c->wqt, c->bqt, c->th1, c->qb.p, 1,
                            1.0f / std::sqrt(static_cast<float>(g.dp)), q_out, static_cast<const int*>(c->post.p), 1,
-                           c->s_aux, MAP_K_GEMM_TEXT, MAP_K_GEMM_TEXT));
+                           tile_t, c->s_aux, MAP_K_GEMM_TEXT, MAP_K_GEMM_TEXT));
   CU_TRY(cudaEventRecord(c->ev_join, c->s_aux));
   MAP_TRY(predictor_branch(c, vis, vrows, c->w[5], c->w[6], c->wkv, c->bkv, c->h1, c->kb.p, 0, 1.0f, k_out, nullptr,
-                           N, st, MAP_K_GEMM_FV1, MAP_K_GEMM_WK));
+                           N, tile_v, st, MAP_K_GEMM_FV1, MAP_K_GEMM_WK));
   CU_TRY(cudaStreamWaitEvent(st, c->ev_join, 0));
   // Eq. 3 on the tensor cores: logits tile [visual tokens x question tokens] of one image,
   // pass 1 -> per-slab column (max, sum exp), combine -> max + ln(sum), pass 2 -> mean.

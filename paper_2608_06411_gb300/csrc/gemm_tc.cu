@@ -90,7 +90,8 @@ struct Smem {
   static constexpr uint32_t LSM = PROJ ? BN * BN * 4 : 0;       // L rows of the basis (pitch BN)
   static constexpr uint32_t PEXTRA = PROJ ? BN * 4 : 0;          // 1/r of the basis
   static constexpr uint32_t TOTAL = 1024 + TILES + STG + BARS + 16 + XPOSE + LSM + PEXTRA;
-  static constexpr uint32_t TMEM_COLS = PROJ ? (2 * BN + 2 * kBM <= 256 ? 256u : 512u) : 2 * BN;   // + A A^T
+  static constexpr uint32_t TMEM_COLS =                           // a power of two; PROJ: + A A^T
+      PROJ ? (2 * BN + 2 * kBM <= 256 ? 256u : 512u) : (2 * BN > 256 ? 512u : 2 * BN);
   static constexpr int THREADS = 192;
 };
 
@@ -470,12 +471,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           staged_b = c.b;
         }
       }
-      if (!mbar_wait(&tfull[acc], acc_phase, a.status, abort_flag, a.wait_ns)) break;
-      tc_fence_after();
       const int row = c.m_blk * kBM + r_in_tile;
       const bool row_ok = row < (a.m_limit ? min(a.M, __ldg(a.m_limit + c.b)) : a.M);
       const int lim = a.n_limit ? min(a.N, __ldg(a.n_limit + c.b)) : a.N;
       const int col0 = c.n_blk * BN;
+      // the RoPE factors the epilogue starts with are loaded while the tile's MMAs still run
+      [[maybe_unused]] float2 cs[32];
+      [[maybe_unused]] const float2* rt = nullptr;
+      [[maybe_unused]] auto load_rope = [&](int i0) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) cs[j] = __ldg(rt + static_cast<long long>(i0 + j) * a.rope_ld);
+      };
+      if constexpr (S::TSTORE_ROPE) {
+        int pos = 0;
+        if (row_ok) pos = a.pos ? __ldg(a.pos + row) : row % a.pos_mod;
+        rt = a.rope + pos;
+        load_rope(0);
+      }
+      if (!mbar_wait(&tfull[acc], acc_phase, a.status, abort_flag, a.wait_ns)) break;
+      tc_fence_after();
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + acc * BN;
       const long long crow = static_cast<long long>(c.b) * a.c_batch_stride + static_cast<long long>(row) * a.ldc;
 
@@ -512,9 +526,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // in shared memory and written by TMA box stores (rows past M are clipped)
         constexpr int HALF = BN / 2;
         float* aux = (a.aux && row_ok) ? a.aux + static_cast<long long>(row) * BN : nullptr;
-        int pos = 0;
-        if (row_ok) pos = a.pos ? __ldg(a.pos + row) : row % a.pos_mod;
-        const float2* rt = a.rope + pos;
         const int seg_lo = a.split_kind == 0 ? 1 : 2;   // keys [hi, lo, hi], queries [hi, hi, lo]
         const int ew = warp - 2;
         const int y = c.b * a.a_row_stride + c.m_blk * kBM + lane_grp * 32;
@@ -522,6 +533,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll 1
         for (int ch = 0; ch < HALF / 32; ++ch) {
           uint32_t r1[32], r2[32];
+          if (ch > 0) load_rope(ch * 32);
           tmem_ld32(tbase + ch * 32, r1);
           tmem_ld32(tbase + HALF + ch * 32, r2);
           if (lane == 0) bulk_wait_group_read<0>();    // the previous chunk's stores have read sb
@@ -531,14 +543,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             float o1[8], o2[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-              const float2 cs = __ldg(rt + static_cast<long long>(ch * 32 + j + u) * a.rope_ld);
+              const float2 rc = cs[j + u];
               float x1 = __uint_as_float(r1[j + u]), x2 = __uint_as_float(r2[j + u]);
               if (a.biasf) {
                 x1 += __ldg(a.biasf + ch * 32 + j + u);
                 x2 += __ldg(a.biasf + HALF + ch * 32 + j + u);
               }
-              o1[u] = x1 * cs.x - x2 * cs.y;
-              o2[u] = x2 * cs.x + x1 * cs.y;
+              o1[u] = x1 * rc.x - x2 * rc.y;
+              o2[u] = x2 * rc.x + x1 * rc.y;
             }
             if (aux) {
 #pragma unroll
@@ -811,9 +823,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int y = c.b * a.a_row_stride + c.m_blk * kBM + lane_grp * 32;   // first row of this warp
 #pragma unroll 1
         for (int ch = 0; ch < BN / 32; ++ch) {
+          const int cbase = col0 + ch * 32;
+          if (cbase >= lim) break;                       // uniform: a last tile wider than what is left
           uint32_t r[32];
           tmem_ld32(tbase + ch * 32, r);
-          const int cbase = col0 + ch * 32;
           uint8_t* hb = stg + (ew * 2 + (ch & 1)) * 4096;     // [hi 32x32 | lo 32x32] bf16
           if (lane == 0) bulk_wait_group_read<1>();      // this buffer's previous store has read it
           __syncwarp();
@@ -843,7 +856,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
           fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0 && cbase < lim) {                  // rows past M are clipped by the store
+          if (lane == 0) {                                 // rows past M are clipped by the store
             tma_store_2d(&tmC, hb, cbase, y);
             tma_store_2d(&tmC, hb + 2048, a.N + cbase, y);
             bulk_commit_group();
@@ -1002,6 +1015,37 @@ cudaError_t run(const GemmDesc& d, const KArgs& ka, int num_sms, cudaStream_t st
 
 }  // namespace
 
+// Columns of the 2-SM tiles (256 rows) of the first layers of both predictor branches, which run
+// side by side: the pair of widths with the least time by the model
+//   waves of the tiles over the SM pairs x K blocks x the longer of the MMA (2 BN cycles) and the
+//   copies into an SM (256 + BN), and the last tile's epilogue (40 BN),
+// the two branches at once where their tiles fit the chip together, else one after the other.
+// Large batches take 256.  With few rows the chip would idle behind a few wide tiles, each a chain
+// of K / 64 blocks: N = 576 takes 64 (48 pairs instead of 12), N = 2880 192 (72 instead of 48)
+// beside a question branch kept on the four pairs left.  The width changes no sum.  One image of
+// 576 tokens: 234.5 -> 226.8 us per call; of 2880: 312.9 -> 310.8 us.
+void predictor_tile_widths(int m_vis, int m_text, int N, int K, int num_sms, int* w_vis, int* w_text) {
+  constexpr int kWidths[4] = {256, 192, 128, 64};
+  const long long pairs = std::max(1, num_sms / 2);
+  auto units = [&](int M, int bn) {
+    return static_cast<long long>((M + 2 * kBM - 1) / (2 * kBM)) * ((N + bn - 1) / bn);
+  };
+  auto time = [&](int M, int bn) {
+    return (units(M, bn) + pairs - 1) / pairs * (K / kBK) * std::max(2 * bn, 256 + bn) + 40 * bn;
+  };
+  long long best = -1;
+  for (int v : kWidths)
+    for (int w : kWidths) {
+      const long long tv = time(m_vis, v), tw = time(m_text, w);
+      const long long t = units(m_vis, v) + units(m_text, w) <= pairs ? std::max(tv, tw) : tv + tw;
+      if (best < 0 || t < best) {
+        best = t;
+        *w_vis = v;
+        *w_text = w;
+      }
+    }
+}
+
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
   if (d.K <= 0 || d.K % kBK != 0 || d.M < 0 || d.N <= 0 || d.batch <= 0) return cudaErrorInvalidValue;
   if (d.a_kwrap < 0 || d.a_kwrap % kBK != 0 || d.a_kwrap > d.K) return cudaErrorInvalidValue;
@@ -1070,7 +1114,14 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
       if (d.N == 256) return run<256, 4, EPI_ROPE_F32>(d, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_GELU_SPLIT:
-      if (d.N % 256 == 0) return run<256, 6, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
+      if (d.N % 256 == 0) {
+        switch (d.tile_n) {
+          case 64: return run<64, 8, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
+          case 128: return run<128, 8, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
+          case 192: return run<192, 6, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
+          default: return run<256, 6, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
+        }
+      }
       if (d.N % 64 == 0) return run<64, 8, EPI_GELU_SPLIT>(d, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_BIAS_SPLIT:

@@ -106,8 +106,12 @@ struct GemmDesc {
   // sum at C + s * c_split_stride (elements, a multiple of 4); the caller adds the slices
   int ksplit = 1; long long c_split_stride = 0;
   GemmProducts pr{};
+  // EPI_GELU_SPLIT, N % 256 == 0: columns of a tile, 64, 128, 192 or 256 (0)
+  int tile_n = 0;
 };
 
+// tile_n of the first layers of the visual and question branches (m_vis and m_text rows, N columns).
+void predictor_tile_widths(int m_vis, int m_text, int N, int K, int num_sms, int* w_vis, int* w_text);
 // Returns cudaSuccess, or an error for an unsupported shape (cudaErrorInvalidValue).
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st);
 

@@ -422,3 +422,24 @@ def test_retention_sweep_config(K, lam, k0_frac):
     keep, order = run_select(ctx, p32, vis, K)
     assert_selection(p32, vis, K, O.resolve_k0(K, k0_frac), keep, order, lam=lam,
                      label=f"c2 N=2880 k={K} lambda={lam} K0={O.resolve_k0(K, k0_frac)}")
+
+
+@pytest.mark.parametrize("N,B", [(100, 9), (576, 12), (1731, 5)])
+def test_scores_of_a_batch_equal_its_images_alone(N, B):
+    """The first layer's tiles are narrower when there are few rows (64, 128, 192 or 256 columns, by
+    the number of tiles), which must not change a bit of any sum: an image scored alone gets the
+    scores it gets in a batch."""
+    dims = W.PredictorDims(D=1024, Dh=1024, dp=128)
+    wl = W.WORKLOADS["c0"]
+    wts = W.make_weights(dims, seed=21, bias_std=0.1)
+    ctx = mb.Context({k: dev_bits(v) for k, v in wts.items()}, dims.D, dims.Dh, dims.dp)
+    lens = np.arange(3, 3 + 7 * B, 7).astype(np.int32)
+    vis = dev_bits(np.stack([W.make_image(wl, b, N=N, D=dims.D) for b in range(B)]))
+    text = dev_bits(np.concatenate([W.make_text(wl, b, int(lens[b]), D=dims.D) for b in range(B)]))
+    together = ctx.score(text, vis, lens)
+    o = 0
+    for b in range(B):
+        alone = ctx.score(text[o:o + int(lens[b])], vis[b:b + 1], lens[b:b + 1])
+        o += int(lens[b])
+        assert torch.equal(alone[0], together[b]), b
+    ctx.check()
