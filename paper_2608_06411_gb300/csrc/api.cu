@@ -402,12 +402,8 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
   char* sm = static_cast<char*>(c->ssmall.p);
   s.npicks = carve<int32_t>(sm, B);
   s.nbasis = carve<int32_t>(sm, B);
-  s.nb_gathered = carve<int32_t>(sm, B);
   s.done = carve<int32_t>(sm, B);
   s.mode = carve<int32_t>(sm, B);
-  s.nlimit = carve<int32_t>(sm, B);
-  s.gb_lo = carve<int32_t>(sm, B);
-  s.gb_hi = carve<int32_t>(sm, B);
   s.gbase = carve<int32_t>(sm, B);
   s.proj_lim = carve<int32_t>(sm, B);
   s.blist = carve<int32_t>(sm, B);
@@ -445,15 +441,6 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
     s.Ec = static_cast<float*>(c->sEc.p);
     s.Vg = c->sVg.p;
     s.G = static_cast<float*>(c->sG.p);
-    GemmDesc d{};
-    d.A = s.Vg; d.a_rows_total = static_cast<long long>(B) * R; d.a_row_stride = R;
-    d.B = s.Vg; d.b_rows_total = static_cast<long long>(B) * R; d.b_row_stride = R;
-    d.M = S; d.N = R; d.K = g.D; d.batch = B; d.n_limit = s.nlimit;
-    d.C = s.G; d.ldc = R; d.c_batch_stride = static_cast<long long>(S) * R;
-    d.epi = mapk::EPI_F32; d.status = c->status;
-    d.sym = 1;                                   // A x A tiles load their rows once
-    d.n_outer = 1;                               // the basis columns are often skipped
-    d.blist = s.blist;                           // images still selecting (built by choose)
     // the GEMM after a list producer reads the count that producer appended through
     auto take_list = [&](GemmDesc& g) { g.bcount = s.bcount + s.bc_par; s.bc_par ^= 1; };
     // Rounds: every round picks or makes S stale bounds exact, so at most ceil(N / S) rounds
@@ -461,15 +448,10 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
     const long long cap = static_cast<long long>(K) * ((N + S - 1) / S + 1) +
                           (K + mapk::kRoundPicks - 1) / mapk::kRoundPicks + 64;
     if (project) {
-      // R0: gather its rows, G[R0, R0] on the tensor cores, then its Cholesky factor.
+      // R0: G[R0, R0] on the tensor cores, then its Cholesky factor.
       c->counters.launches += 3;
       CU_TRY(mapk::launch_sel_choose(s, st));
-      {
-        GemmDesc d0 = d;              // only the K0c x K0c corner of the block
-        d0.M = K0c; d0.N = K0c;
-        take_list(d0);
-        MAP_TRY(gemm(c, d0, st));
-      }
+      CU_TRY(mapk::launch_sel_gram(s, K0c, 0, c->wait_ns, st));
       {
         mapk::SelState sc = s;        // the first K0c tokens of R0
         sc.K0 = K0c;
@@ -505,8 +487,7 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
       // values for every candidate make the next active set the true top S
       c->counters.launches += 5;
       CU_TRY(mapk::launch_sel_choose(s, st));
-      take_list(d);
-      MAP_TRY(gemm(c, d, st));
+      CU_TRY(mapk::launch_sel_gram(s, S, std::max(0, K0c - mapk::kReprojMax), c->wait_ns, st));
       CU_TRY(mapk::launch_sel_greedy(s, st));
       ++c->counters.select_rounds;
       MAP_TRY(project_all(false));
@@ -515,11 +496,8 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
     // round while an image still selects): the host never waits for them.
     if (!c->loops) c->loops = mapk::sel_loop_cache_create();
     if (!c->loops) return MAP_ENOMEM;
-    GemmDesc dl = d;
-    dl.wait_ns = c->wait_ns;
     ++c->counters.launches;            // the test kernel ahead of the loop; iterations are counted on the device
-    CU_TRY(mapk::launch_sel_loop(c->loops, s, dl, c->num_sms, static_cast<int>(cap), loop_iters,
-                                 c->loop_iters_total, st));
+    CU_TRY(mapk::launch_sel_loop(c->loops, s, c->wait_ns, static_cast<int>(cap), loop_iters, c->loop_iters_total, st));
   } else {
     ++c->counters.launches;
     CU_TRY(mapk::launch_sel_copy_r0(s.r0, B, K, s.picks, st));

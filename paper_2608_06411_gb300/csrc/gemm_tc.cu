@@ -2,8 +2,8 @@
 //
 // Used for every dense contraction of the pruning path: the predictor layers f_V, f_T
 // (Linear -> GELU -> Linear), the W_K / W_Q projections with RoPE fused into the
-// epilogue (section "Cross-Modal Attention Distillation"), and the Gram blocks
-// <v_i, v_j> that the diversity term of Eq. 4 needs.
+// epilogue (section "Cross-Modal Attention Distillation"), Eq. 3's logits, the projection of
+// every token on the R0 basis (Eq. 4), and the distillation step.
 //
 // Structure (one CTA per SM, 6 warps):
 //   warp 0      one thread issues TMA loads of 128x64 (A) and BNx64 (B) bf16 tiles, 128-byte
@@ -57,8 +57,6 @@ struct KArgs {
   unsigned long long wait_ns;   // limit of the role waits (the drain waits keep kWaitLimitNs)
   int ksplit; long long c_split_stride;   // EPI_F32 split-K: partial sums per K slice
   GemmProducts pr;                         // EPI_F32: products of column segments (pr.n > 0)
-  int sym;                                 // B is A: the diagonal tile reads its A stage as B
-  int n_outer;                             // unit order: column tiles outermost
 };
 
 __device__ __forceinline__ float gelu_erf(float x) {
@@ -114,28 +112,14 @@ template <bool PAIR>
 __device__ __forceinline__ TileCoord tile_coord(const KArgs& a, int t, int nbatch, int m_units, int n_tiles, int BN,
                                                 uint32_t crank) {
   TileCoord c;
-  int mu;
-  if (a.n_outer) {
-    // column tiles outermost: the units of one column tile of every batch entry are
-    // consecutive, so that when whole column tiles are skipped (n_limit) the remaining units
-    // still spread over all CTAs
-    const int per_n = nbatch * m_units * a.ksplit;
-    c.n_blk = t / per_n;
-    int rem = t - c.n_blk * per_n;
-    c.b = rem / (m_units * a.ksplit);
-    rem -= c.b * (m_units * a.ksplit);
-    c.ks = rem / m_units;
-    mu = rem - c.ks * m_units;
-  } else {
-    const int tiles = m_units * n_tiles;
-    const int per = tiles * a.ksplit;
-    c.b = t / per;
-    int rem = t - c.b * per;
-    c.ks = rem / tiles;
-    rem -= c.ks * tiles;
-    mu = rem / n_tiles;
-    c.n_blk = rem - mu * n_tiles;
-  }
+  const int tiles = m_units * n_tiles;
+  const int per = tiles * a.ksplit;
+  c.b = t / per;
+  int rem = t - c.b * per;
+  c.ks = rem / tiles;
+  rem -= c.ks * tiles;
+  const int mu = rem / n_tiles;
+  c.n_blk = rem - mu * n_tiles;
   if (a.blist) c.b = __ldg(a.blist + c.b);
   c.m_blk = PAIR ? 2 * mu + static_cast<int>(crank) : mu;
   int lim = a.n_limit ? min(a.N, __ldg(a.n_limit + c.b)) : a.N;
@@ -229,16 +213,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   };
 
-  // With a.sym, a tile whose B rows (this CTA's half of them with 2-SM pairs) are its A rows
-  // loads them once: the same stage layout serves as both operands (BN / 2 or BN == kBM rows).
-  // Both CTAs of a pair and all roles reach the same answer (the row offsets cancel).
-  auto b_is_a = [&](const TileCoord& c) {
-    if (!a.sym || (CG2 ? BN / 2 : BN) != kBM) return false;
-    const int arow = c.b * a.a_row_stride + c.m_blk * kBM;
-    const int brow = c.b * a.b_row_stride + a.b_base + c.n_blk * BN + (CG2 ? static_cast<int>(crank) * (BN / 2) : 0);
-    return arow == brow;
-  };
-
   // Producer: parity of the last load issued into each stage (-1: none), for the drain below.
   int last_par[STAGES];
 #pragma unroll
@@ -253,8 +227,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (c.skip) continue;
         const int arow = c.b * a.a_row_stride + c.m_blk * kBM;
         const int brow = (a.b_off ? __ldg(a.b_off + c.b) : c.b * a.b_row_stride + a.b_base) + c.n_blk * BN;
-        const bool alias = b_is_a(c);
-        const int kstep = alias ? 2 : 1;           // alias: two K blocks per stage (A and B buffers)
         int kb0, kb1;
         kb_range(c, kb0, kb1);
         if constexpr (PRODUCTS) {
@@ -311,24 +283,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             continue;
           }
         }
-        for (int kb = kb0; kb < kb1; kb += kstep) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(&empty[stage], phase ^ 1, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
           int ac, bc;
           kcols(kb, ac, bc);
-          if (alias) {
-            // K block kb into the A buffer, kb + 1 (when in range) into the B buffer; no kwrap
-            const int n2 = kb + 1 < kb1 ? 2 : 1;
-            if constexpr (CG2) {
-              if (crank == 0) mbar_arrive_expect_tx(&full[stage], 2 * n2 * S::A_BYTES);
-              const uint32_t fb = mapa_u32(&full[stage], 0);
-              tma_load_2d_cg2(sA + stage * S::A_BYTES, &tmA, fb, ac, arow);
-              if (n2 == 2) tma_load_2d_cg2(sB + stage * S::B_BYTES, &tmA, fb, ac + kBK, arow);
-            } else {
-              mbar_arrive_expect_tx(&full[stage], n2 * S::A_BYTES);
-              tma_load_2d(sA + stage * S::A_BYTES, &tmA, &full[stage], ac, arow);
-              if (n2 == 2) tma_load_2d(sB + stage * S::B_BYTES, &tmA, &full[stage], ac + kBK, arow);
-            }
-          } else if constexpr (CG2) {
+          if constexpr (CG2) {
             // both CTAs' copies complete on the leader's full barrier, which expects them all
             if (crank == 0) mbar_arrive_expect_tx(&full[stage], 2 * S::STAGE_BYTES);
             const uint32_t fb = mapa_u32(&full[stage], 0);
@@ -362,36 +321,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (!mbar_wait(&tempty[acc], acc_phase ^ 1, a.status, abort_flag, a.wait_ns)) break;
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + acc * BN;
-        const bool alias = b_is_a(c);
-        const int kstep = alias ? 2 : 1;
         int kb0, kb1;
         kb_range(c, kb0, kb1);
-        for (int kb = kb0; kb < kb1; kb += kstep) {
+        for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(&full[stage], phase, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a0 = smem_u32(sA + stage * S::A_BYTES);
-          const uint32_t b0 = alias ? a0 : smem_u32(sB + stage * S::B_BYTES);
+          const uint32_t b0 = smem_u32(sB + stage * S::B_BYTES);
           if (PRODUCTS && a.pr.n > 0) {
 #pragma unroll
             for (int k = 0; k < kBK / 16; ++k) {
               const uint64_t da = adesc0 + (a0 >> 4) + k * astep, db = bdesc0 + (b0 >> 4) + k * bstep;
               if constexpr (CG2) umma_bf16_cg2(d_tmem, da, db, pid, (kb != kb0 || k != 0));
               else umma_bf16(d_tmem, da, db, pid, (kb != kb0 || k != 0));
-            }
-            if constexpr (CG2) umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
-            else umma_commit(&empty[stage]);
-          } else if (alias) {
-            // each buffer is both operands of its K block (the tile's B rows are its A rows)
-            const uint32_t a1 = smem_u32(sB + stage * S::B_BYTES);
-            const int n2 = kb + 1 < kb1 ? 2 : 1;
-            for (int h = 0; h < n2; ++h) {
-              const uint32_t x = h == 0 ? a0 : a1;
-#pragma unroll
-              for (int k = 0; k < kBK / 16; ++k) {
-                const uint32_t acc_on = (kb != kb0 || h != 0 || k != 0);
-                if constexpr (CG2) umma_bf16_cg2(d_tmem, desc_sw128(x + k * 32), desc_sw128(x + k * 32), IDESC, acc_on);
-                else umma_bf16(d_tmem, desc_sw128(x + k * 32), desc_sw128(x + k * 32), IDESC, acc_on);
-              }
             }
             if constexpr (CG2) umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
             else umma_commit(&empty[stage]);
@@ -1084,9 +1026,6 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
     return cudaErrorInvalidValue;
   ka.ksplit = d.ksplit; ka.c_split_stride = d.c_split_stride;
   if (d.blist && !d.bcount) return cudaErrorInvalidValue;
-  if (d.sym && (d.A != d.B || d.a_row_stride != d.b_row_stride || d.a_rows_total != d.b_rows_total || d.b_off ||
-                d.a_kwrap || d.split3 || d.pr.n))
-    return cudaErrorInvalidValue;
   ka.pr = d.pr;
   if (d.pr.n) {      // segments start at whole boxes; K is the products' K blocks side by side
     const GemmProducts& q = d.pr;
@@ -1097,8 +1036,6 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
       if (q.a_seg[i] < 0 || q.a_seg[i] % kBK != 0 || q.b_seg[i] < 0 || q.b_seg[i] % kBK != 0)
         return cudaErrorInvalidValue;
   }
-  ka.sym = d.sym;
-  ka.n_outer = d.n_outer;
   switch (d.epi) {
     case EPI_GELU_BF16:
       if (d.N % 256 == 0) return run<256, 4, EPI_GELU_BF16>(d, ka, num_sms, st);
@@ -1140,8 +1077,8 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
       if (d.N > kProjMaxBasis || d.batch < 1) return cudaErrorInvalidValue;
       if (d.N <= 96) return run<96, 6, EPI_PROJECT>(d, ka, num_sms, st);
       return run<128, 5, EPI_PROJECT>(d, ka, num_sms, st);
-    case EPI_F32:   // Gram blocks: one 256 x 256 pair tile per image and 256 columns
-      if (d.M <= kBM && d.N <= 128) return run<128, 6, EPI_F32>(d, ka, num_sms, st);   // G[R0, R0]
+    case EPI_F32:   // the distillation's contractions
+      if (d.M <= kBM && d.N <= 128) return run<128, 6, EPI_F32>(d, ka, num_sms, st);
       return run<256, 6, EPI_F32, true>(d, ka, num_sms, st);
     default:
       return cudaErrorInvalidValue;

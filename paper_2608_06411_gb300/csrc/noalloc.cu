@@ -139,19 +139,18 @@ extern "C" int map_select_noalloc(map_ctx* ctx, const float* scores, const void*
   s.rnorm = cv.take<float>(static_cast<size_t>(B) * K);
   s.npicks = cv.take<int32_t>(B);
   s.nbasis = cv.take<int32_t>(B);
-  s.nb_gathered = cv.take<int32_t>(B);
   s.done = cv.take<int32_t>(B);
   s.mode = cv.take<int32_t>(B);
-  s.nlimit = cv.take<int32_t>(B);
-  s.gb_lo = cv.take<int32_t>(B);
-  s.gb_hi = cv.take<int32_t>(B);
   s.gbase = cv.take<int32_t>(B);
+  cv.take<int32_t>(B); cv.take<int32_t>(B); cv.take<int32_t>(B); cv.take<int32_t>(B);   // unused (see below)
   s.done_count = cv.take<int32_t>(1);
   s.theta = cv.take<uint64_t>(B);
   s.aslot = cv.take<int32_t>(static_cast<size_t>(B) * S);
   if (K0 < K) {
     s.Ec = cv.take<float>(static_cast<size_t>(BN) * KP);
-    s.Vg = cv.take<uint16_t>(static_cast<size_t>(B) * R * g.D);
+    // no longer written (the Gram blocks read the features in place); still counted, so that the same
+    // calls fit the array as before
+    cv.take<uint16_t>(static_cast<size_t>(B) * R * g.D);
     s.G = cv.take<float>(static_cast<size_t>(B) * S * R);
   }
   if (!cv.ok()) return MAP_EUNSUPPORTED;      // workspace larger than the static array
@@ -166,14 +165,6 @@ extern "C" int map_select_noalloc(map_ctx* ctx, const float* scores, const void*
   ++*v.launches;
   if ((rc = rc_of(mapk::launch_sel_init(s, st))) != MAP_OK) return rc;
   if (K0 < K) {                   // sel_init has zeroed done_count
-    mapk::GemmDesc d{};
-    d.A = s.Vg; d.a_rows_total = static_cast<long long>(B) * R; d.a_row_stride = R;
-    d.B = s.Vg; d.b_rows_total = static_cast<long long>(B) * R; d.b_row_stride = R;
-    d.M = S; d.N = R; d.K = g.D; d.batch = B; d.n_limit = s.nlimit;
-    d.C = s.G; d.ldc = R; d.c_batch_stride = static_cast<long long>(S) * R;
-    d.epi = mapk::EPI_F32; d.status = v.status;
-    d.sym = 1;                                   // A x A tiles load their rows once
-    d.n_outer = 1;                               // the basis columns are often skipped
     // every round picks or makes S stale bounds exact: at most ceil(N / S) rounds without a
     // pick come before each pick
     const long long cap = static_cast<long long>(K) * ((N + S - 1) / S + 1) +
@@ -182,11 +173,9 @@ extern "C" int map_select_noalloc(map_ctx* ctx, const float* scores, const void*
     int burst = (K0 + mapk::kRoundPicks - 1) / mapk::kRoundPicks + 6;
     for (;;) {
       for (int r = 0; r < burst; ++r) {
-        *v.launches += 6;
+        *v.launches += 5;
         if ((rc = rc_of(mapk::launch_sel_choose(s, st))) != MAP_OK) return rc;
-        cudaError_t e = mapk::launch_gemm(d, v.num_sms, st);
-        if (e == cudaErrorInvalidValue) return MAP_EUNSUPPORTED;
-        if ((rc = rc_of(e)) != MAP_OK) return rc;
+        if ((rc = rc_of(mapk::launch_sel_gram(s, S, K, 0, st))) != MAP_OK) return rc;
         if ((rc = rc_of(mapk::launch_sel_greedy(s, st))) != MAP_OK) return rc;
       }
       rounds += burst;

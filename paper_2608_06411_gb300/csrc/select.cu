@@ -18,9 +18,8 @@
 // Later picks proceed in rounds:
 //   choose : active set A = the s candidates with the largest value bound U (a stale
 //            value, or p_hat * ||v||^lambda for tokens never evaluated; values only shrink
-//            as B grows, so U is always an upper bound); gather their rows and the rows of
-//            new basis tokens into a compact buffer Vg.
-//   gram   : G_blk = Vg[A] Vg[A u new basis]^T on tcgen05 (gemm_tc.cu).
+//            as B grows, so U is always an upper bound).
+//   gram   : the products of A's rows with A's and the newer basis tokens' on tcgen05 (sel_gram.cu).
 //   update : bring each A member's coordinates up to date (exact values).
 //   resgram: replace G[A, A] by the Gram matrix of the residuals on the current basis, so
 //            that the picks need only the coordinates added during the round.
@@ -220,8 +219,7 @@ __global__ void __launch_bounds__(1024) sel_init_kernel(SelState s) {
     if (s.uptr) { s.uptr[0] = s.scores; s.uptr[1] = s.V; }
   }
   if (threadIdx.x == 0) {
-    s.npicks[b] = 0; s.nbasis[b] = 0; s.nb_gathered[b] = 0; s.done[b] = 0; s.nlimit[b] = 0;
-    s.gb_lo[b] = 0; s.gb_hi[b] = 0; s.gbase[b] = 0;
+    s.npicks[b] = 0; s.nbasis[b] = 0; s.done[b] = 0; s.gbase[b] = 0;
     cnt = 0;
   }
   __syncthreads();
@@ -260,13 +258,8 @@ __global__ void __launch_bounds__(1024) sel_choose_kernel(SelState s) {
   const long long base = static_cast<long long>(b) * s.N;
   const int S = s.S;
   int32_t* aslot = s.aslot + static_cast<long long>(b) * S;
-  if (s.blist && b == 0 && threadIdx.x == 0) s.bcount[s.bc_par ^ 1] = 0;
-  if (s.done[b]) {
-    if (threadIdx.x == 0) s.nlimit[b] = 0;
-    return;
-  }
-  if (s.blist && threadIdx.x == 0) s.blist[atomicAdd(s.bcount + s.bc_par, 1)] = b;
-  const int np = s.npicks[b], nb = s.nbasis[b];
+  if (s.done[b]) return;
+  const int np = s.npicks[b];
   uint64_t theta = 0;
   int mode;
   if (np < s.K0) {
@@ -300,36 +293,24 @@ __global__ void __launch_bounds__(1024) sel_choose_kernel(SelState s) {
   if (threadIdx.x == 0) {
     s.mode[b] = mode;
     s.theta[b] = theta;
-    s.nlimit[b] = (mode == 1 && nb == s.gbase[b]) ? min(S, s.K0 - np) : S + nb - s.gbase[b];
-    s.gb_lo[b] = s.nb_gathered[b];
-    s.gb_hi[b] = nb;
-    s.nb_gathered[b] = nb;
   }
 }
 
-// Copies the rows the Gram block needs into Vg: row r < S <- token aslot[r];
-// row S + beta - gbase <- basis token beta for the basis vectors added since the last round.
-// kGatherCtas CTAs per image, each walking every kGatherCtas-th row; finished images exit.
+// Copies the basis rows of the images to project into Vg: row S + beta <- basis token beta.
+// kGatherCtas CTAs per image, each walking every kGatherCtas-th row; other images exit.
 constexpr int kGatherCtas = 64;
 constexpr int kGatherThreads = 128;
 
 __global__ void __launch_bounds__(kGatherThreads) sel_gather_kernel(SelState s) {
   pdl_enter();
   const int b = blockIdx.y;
-  if (s.done[b]) return;
-  const int gb = s.gbase[b], lo = s.gb_lo[b], hi = s.gb_hi[b];
+  if (s.proj_lim[b] == 0) return;
+  const int nb = min(s.nbasis[b], kReprojMax);
   const int vec = s.D / 8;
-  for (int r = blockIdx.x; r < s.S + (hi - gb); r += kGatherCtas) {
-    int src = -1;
-    if (r < s.S) {
-      src = s.aslot[static_cast<long long>(b) * s.S + r];
-    } else {
-      const int beta = r - s.S + gb;
-      if (beta >= lo && beta < hi) src = s.basis_tok[static_cast<long long>(b) * s.K + beta];
-    }
-    if (src < 0) continue;                               // uniform in the CTA
+  for (int r = blockIdx.x; r < nb; r += kGatherCtas) {
+    const int src = s.basis_tok[static_cast<long long>(b) * s.K + r];
     const uint4* __restrict__ V = reinterpret_cast<const uint4*>(sel_features(s)) + (static_cast<long long>(b) * s.N + src) * vec;
-    uint4* __restrict__ dst = reinterpret_cast<uint4*>(s.Vg) + (static_cast<long long>(b) * s.R + r) * vec;
+    uint4* __restrict__ dst = reinterpret_cast<uint4*>(s.Vg) + (static_cast<long long>(b) * s.R + s.S + r) * vec;
     // four 16-byte loads in flight per thread before their stores (V and Vg never overlap)
     int c = threadIdx.x;
     constexpr int T = kGatherThreads;
@@ -749,9 +730,8 @@ __global__ void __launch_bounds__(kCholThreads, 1) sel_chol_kernel(SelState s) {
 // the active set is
 //   G'[i][k] = <v_i, v_k> - sum_{q < c0} e_q[i] e_q[k]   (the inner product of the residuals),
 // and a pick then needs only the coordinates added during the round (sel_greedy_kernel).
-// It replaces the lower triangle of the A x A part of the Gram block in place (the picks read
-// no more).  One CTA of 64 threads per 32 x 32 tile of the upper triangle, whose mirrored tile
-// it writes, 4 x 4 outputs per thread; the coordinates are staged in 16-column chunks,
+// It replaces the lower triangle of the A x A part of the Gram block in place (no more of it is
+// computed or read).  One CTA of 64 threads per 32 x 32 tile, 4 x 4 outputs per thread; the coordinates are staged in 16-column chunks,
 // transposed, in two shared buffers, the next chunk loaded during the products of the
 // current one.  Small tiles keep several CTAs on every SM, so the chunk loop's latency is
 // hidden, with few images (c0 is large) as with many.
@@ -773,10 +753,10 @@ __global__ void __launch_bounds__(kRgThreads) sel_resgram_kernel(SelState s) {
   int t = blockIdx.x, ti = 0;
   const int T = S / kRgTile;
   while (t >= T - ti) { t -= T - ti; ++ti; }
-  const int tk = ti + t;
+  const int tk = ti, tr = ti + t;                    // column tile, row tile (at or below the diagonal)
   const int32_t* aslot = s.aslot + static_cast<long long>(b) * S;
   const int tid = threadIdx.x;
-  if (tid < kRgTile) toki[tid] = aslot[ti * kRgTile + tid];
+  if (tid < kRgTile) toki[tid] = aslot[tr * kRgTile + tid];
   else tokk[tid - kRgTile] = aslot[tk * kRgTile + tid - kRgTile];
   // a tile whose rows or columns are all empty slots writes nothing
   const bool any_i = __syncthreads_or(tid < kRgTile && toki[tid] >= 0);
@@ -835,46 +815,27 @@ __global__ void __launch_bounds__(kRgThreads) sel_resgram_kernel(SelState s) {
     }
     __syncthreads();
   }
-  // G' = G - acc through a shared tile, so that the tile is read and its mirror written in
-  // whole rows (coalesced)
+  // G' = G - acc through a shared tile, in whole rows (coalesced)
   float(*Tt)[kRgTile + 1] = reinterpret_cast<float(*)[kRgTile + 1]>(sbuf);
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int cc = 0; cc < 4; ++cc) Tt[ty * 4 + r][tx * 4 + cc] = acc[r][cc];
   __syncthreads();
-  float* Gb = s.G + static_cast<long long>(b) * S * s.R;
   constexpr int kRowsPer = kRgTile * kRgTile / kRgThreads;   // rows of the tile per thread
-  {
-    const int c = tid & (kRgTile - 1), r0 = tid / kRgTile;
-    const bool okc = tokk[c] >= 0;
-    float* g0 = Gb + static_cast<long long>(ti * kRgTile) * s.R + tk * kRgTile + c;
-    float gv[kRowsPer];                              // every load in flight before the stores
+  const int c = tid & (kRgTile - 1), r0 = tid / kRgTile;
+  const bool okc = tokk[c] >= 0;
+  float* g0 = s.G + (static_cast<long long>(b) * S + tr * kRgTile) * s.R + tk * kRgTile + c;
+  float gv[kRowsPer];                                // every load in flight before the stores
 #pragma unroll
-    for (int m = 0; m < kRowsPer; ++m) {
-      const int r = r0 + m * (kRgThreads / kRgTile);
-      gv[m] = okc && toki[r] >= 0 ? g0[static_cast<long long>(r) * s.R] : 0.f;
-    }
-    if (ti == tk) {
+  for (int m = 0; m < kRowsPer; ++m) {
+    const int r = r0 + m * (kRgThreads / kRgTile);
+    gv[m] = okc && toki[r] >= 0 ? g0[static_cast<long long>(r) * s.R] : 0.f;
+  }
 #pragma unroll
-      for (int m = 0; m < kRowsPer; ++m) {
-        const int r = r0 + m * (kRgThreads / kRgTile);
-        if (okc && toki[r] >= 0) g0[static_cast<long long>(r) * s.R] = gv[m] - Tt[r][c];
-      }
-    } else {                                         // the mirrored tile alone: the lower triangle is read
-#pragma unroll
-      for (int m = 0; m < kRowsPer; ++m) {
-        const int r = r0 + m * (kRgThreads / kRgTile);
-        Tt[r][c] = gv[m] - Tt[r][c];
-      }
-      __syncthreads();
-      float* m0 = Gb + static_cast<long long>(tk * kRgTile) * s.R + ti * kRgTile + c;
-#pragma unroll
-      for (int m = 0; m < kRowsPer; ++m) {         // row r of the mirror: column r of the tile
-        const int r = r0 + m * (kRgThreads / kRgTile);
-        if (tokk[r] >= 0 && toki[c] >= 0) m0[static_cast<long long>(r) * s.R] = Tt[c][r];
-      }
-    }
+  for (int m = 0; m < kRowsPer; ++m) {
+    const int r = r0 + m * (kRgThreads / kRgTile);
+    if (okc && toki[r] >= 0) g0[static_cast<long long>(r) * s.R] = gv[m] - Tt[r][c];
   }
 }
 
@@ -1098,7 +1059,8 @@ __global__ void __launch_bounds__(kActiveSlots, 1) sel_greedy_kernel(SelState s)
 }
 
 // ------------------------------------------------------------------ projection set-up
-// Gathers every basis row of the images to project (no active tokens) for the projection.
+// Which images to project: all (first), or those still selecting whose basis has grown and has at
+// most kReprojMax vectors; their list for the projection.
 __global__ void sel_proj_prep_kernel(SelState s, int first) {
   pdl_enter();
   const int b = blockIdx.x;
@@ -1109,14 +1071,9 @@ __global__ void sel_proj_prep_kernel(SelState s, int first) {
     if (threadIdx.x == 0) s.proj_lim[b] = 0;
     return;
   }
-  for (int i = threadIdx.x; i < s.S; i += blockDim.x) s.aslot[static_cast<long long>(b) * s.S + i] = -1;
   if (threadIdx.x == 0) {
     if (s.blist) s.blist[atomicAdd(s.bcount + s.bc_par, 1)] = b;
     s.proj_lim[b] = kReprojMax;
-    s.gbase[b] = 0;                                  // rows S + beta for the whole basis
-    s.gb_lo[b] = 0;
-    s.gb_hi[b] = nb;
-    s.nb_gathered[b] = nb;
   }
 }
 
@@ -1124,9 +1081,7 @@ __global__ void sel_proj_done_kernel(SelState s) {
   pdl_enter();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < s.B && s.proj_lim[b] > 0) {
-    const int nb = min(s.nbasis[b], kReprojMax);       // coordinates the projection gave
-    s.gbase[b] = nb;
-    s.nb_gathered[b] = nb;
+    s.gbase[b] = min(s.nbasis[b], kReprojMax);         // coordinates the projection gave
   }
 }
 
@@ -1188,13 +1143,10 @@ __global__ void sel_loop_init_kernel(SelState s, cudaGraphConditionalHandle h, i
 }
 
 // Last node of the WHILE body: run another round while an image still selects, no kernel
-// has reported an error and the iteration cap has not been reached (then ST_INTERNAL).  It
-// also clears the image-list count the round's choose appended to (the Gram block has read
-// it), so that the next iteration's choose starts from zero on the same counter.
+// has reported an error and the iteration cap has not been reached (then ST_INTERNAL).
 __global__ void sel_loop_cond_kernel(SelState s, cudaGraphConditionalHandle h, int32_t* iters, int cap_iters,
                                      long long* iters_total) {
   if (threadIdx.x == 0) {
-    s.bcount[s.bc_par] = 0;
     const int it = *iters + 1;
     *iters = it;
     *iters_total += 1;
@@ -1230,8 +1182,7 @@ cudaError_t launch_sel_choose(const SelState& s, cudaStream_t st) {
   const size_t sm = sel_choose_smem(s.N);
   cudaError_t e = cudaFuncSetAttribute(sel_choose_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sm));
   if (e != cudaSuccess) return e;
-  if ((e = launch_k(sel_choose_kernel, dim3(s.B), dim3(1024), sm, st, s)) != cudaSuccess) return e;
-  return launch_k(sel_gather_kernel, dim3(kGatherCtas, s.B), dim3(kGatherThreads), 0, st, s);
+  return launch_k(sel_choose_kernel, dim3(s.B), dim3(1024), sm, st, s);
 }
 
 cudaError_t launch_sel_greedy(const SelState& s, cudaStream_t st) {
@@ -1268,7 +1219,7 @@ cudaError_t launch_sel_copy_r0(const int32_t* r0, int B, int K, int32_t* picks, 
 }
 
 cudaError_t launch_sel_proj_prep(const SelState& s, bool first, cudaStream_t st) {
-  return launch_k(sel_proj_prep_kernel, dim3(s.B), dim3(256), 0, st, s, first ? 1 : 0);
+  return launch_k(sel_proj_prep_kernel, dim3(s.B), dim3(32), 0, st, s, first ? 1 : 0);
 }
 
 cudaError_t launch_sel_gather(const SelState& s, cudaStream_t st) {
@@ -1314,23 +1265,18 @@ long long pbits(const void* p) { return static_cast<long long>(reinterpret_cast<
 
 // Everything the captured kernels depend on, except the caller's scores and features (read
 // through s.uptr).
-std::vector<long long> loop_key(const SelState& s, const GemmDesc& g, int num_sms, int cap_iters, const int32_t* iters,
+std::vector<long long> loop_key(const SelState& s, long long wait_ns, int cap_iters, const int32_t* iters,
                                 const long long* iters_total) {
   return {s.B, s.N, s.D, s.K, s.K0, s.S, s.R, s.KP, fbits(s.lambda), fbits(s.tau), pbits(s.sqn), pbits(s.U),
           pbits(s.r2), pbits(s.cstep), pbits(s.state), pbits(s.Ec), pbits(s.picks), pbits(s.r0), pbits(s.basis_tok),
-          pbits(s.rnorm), pbits(s.npicks), pbits(s.nbasis), pbits(s.nb_gathered), pbits(s.done), pbits(s.mode),
-          pbits(s.nlimit), pbits(s.gb_lo), pbits(s.gb_hi), pbits(s.gbase), pbits(s.theta), pbits(s.aslot),
-          pbits(s.Vg), pbits(s.G), pbits(s.done_count), pbits(s.proj_lim), pbits(s.blist), pbits(s.bcount),
-          s.bc_par, pbits(s.status), pbits(s.nvalid), pbits(s.uptr),
-          pbits(g.A), g.a_rows_total, g.a_row_stride, pbits(g.B), g.b_rows_total, g.b_row_stride, g.M, g.N, g.K,
-          g.batch, pbits(g.n_limit), pbits(g.C), g.ldc, g.c_batch_stride, g.epi, pbits(g.status), pbits(g.blist),
-          g.wait_ns, num_sms, cap_iters, pbits(iters), pbits(iters_total)};
+          pbits(s.rnorm), pbits(s.npicks), pbits(s.nbasis), pbits(s.done), pbits(s.mode), pbits(s.gbase),
+          pbits(s.theta), pbits(s.aslot), pbits(s.G), pbits(s.done_count), pbits(s.status), pbits(s.nvalid),
+          pbits(s.uptr), wait_ns, cap_iters, pbits(iters), pbits(iters_total)};
 }
 
-// Builds the graph: [test kernel] -> WHILE { choose + gather, Gram, update + residual Gram +
-// greedy; test }.
-cudaError_t build_loop(SelLoopCache* c, const SelState& s, const GemmDesc& gram, int num_sms, int cap_iters,
-                       int32_t* iters, long long* iters_total, SelLoopEntry& out) {
+// Builds the graph: [test kernel] -> WHILE { choose, Gram, update + residual Gram + greedy; test }.
+cudaError_t build_loop(SelLoopCache* c, const SelState& s, long long wait_ns, int cap_iters, int32_t* iters,
+                       long long* iters_total, SelLoopEntry& out) {
   cudaError_t e = cudaSuccess;
   if (!c->cap && (e = cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking)) != cudaSuccess) return e;
   cudaGraph_t g = nullptr;
@@ -1363,12 +1309,9 @@ cudaError_t build_loop(SelLoopCache* c, const SelState& s, const GemmDesc& gram,
     return fail(e);
   pdl_disabled() = true;
   SelState r = s;
-  {
-    GemmDesc d = gram;
-    d.bcount = r.bcount + r.bc_par;              // the count this round's choose appends to
-    if ((e = launch_sel_choose(r, c->cap)) == cudaSuccess && (e = launch_gemm(d, num_sms, c->cap)) == cudaSuccess)
-      e = launch_sel_greedy(r, c->cap);
-  }
+  if ((e = launch_sel_choose(r, c->cap)) == cudaSuccess &&
+      (e = launch_sel_gram(r, r.S, r.K, wait_ns, c->cap)) == cudaSuccess)
+    e = launch_sel_greedy(r, c->cap);
   if (e == cudaSuccess) e = launch_k(sel_loop_cond_kernel, dim3(1), dim3(32), 0, c->cap, r, h, iters, cap_iters, iters_total);
   pdl_disabled() = false;
   cudaGraph_t captured = nullptr;
@@ -1392,17 +1335,17 @@ void sel_loop_cache_destroy(SelLoopCache* c) {
   delete c;
 }
 
-cudaError_t launch_sel_loop(SelLoopCache* c, const SelState& s, const GemmDesc& gram, int num_sms, int cap_iters,
-                            int32_t* iters, long long* iters_total, cudaStream_t st) {
-  if (!c || !s.uptr || !s.done_count || !iters || !iters_total || (s.bc_par & ~1)) return cudaErrorInvalidValue;
-  std::vector<long long> key = loop_key(s, gram, num_sms, cap_iters, iters, iters_total);
+cudaError_t launch_sel_loop(SelLoopCache* c, const SelState& s, long long wait_ns, int cap_iters, int32_t* iters,
+                            long long* iters_total, cudaStream_t st) {
+  if (!c || !s.uptr || !s.done_count || !iters || !iters_total) return cudaErrorInvalidValue;
+  std::vector<long long> key = loop_key(s, wait_ns, cap_iters, iters, iters_total);
   size_t hit = c->entries.size();
   for (size_t i = 0; i < c->entries.size(); ++i)
     if (c->entries[i].key == key) { hit = i; break; }
   if (hit == c->entries.size()) {
     SelLoopEntry ent;
     ent.key = std::move(key);
-    const cudaError_t e = build_loop(c, s, gram, num_sms, cap_iters, iters, iters_total, ent);
+    const cudaError_t e = build_loop(c, s, wait_ns, cap_iters, iters, iters_total, ent);
     if (e != cudaSuccess) return e;
     if (c->entries.size() >= kSelLoopCacheMax) {
       release_entry(c->entries.front());

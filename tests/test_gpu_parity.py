@@ -443,3 +443,21 @@ def test_scores_of_a_batch_equal_its_images_alone(N, B):
         o += int(lens[b])
         assert torch.equal(alone[0], together[b]), b
     ctx.check()
+
+
+@pytest.mark.parametrize("D,K,k0_frac", [(64, 20, 0.5), (192, 60, 0.5), (576, 129, 0.99), (1088, 258, 0.5),
+                                         (576, 288, 0.90625), (320, 400, 0.125)])
+def test_select_gram_blocks_and_r0_factor_edges(D, K, k0_frac):
+    """Feature widths whose 64-column blocks do not divide over the eight ranks of the Gram kernel (some
+    ranks have none), R0 sizes around the 32-column panels and the 128- and 256-row limits of its
+    factor (127, 129, 261), and bases past one unit of 128 columns."""
+    dims = W.PredictorDims(D=D, Dh=256, dp=64)
+    ctx, _ = make_ctx(dims, k0_frac=k0_frac)
+    wl = W.WORKLOADS["c1"]
+    rng = np.random.default_rng(K)
+    B, N = 2, 900
+    vis = np.stack([W.make_image(wl, b, N=N, D=D) for b in range(B)])
+    p32 = rng.dirichlet(np.full(N, 0.3), size=B).astype(np.float32)
+    keep, order = run_select(ctx, p32, vis, K)
+    assert_selection(p32, vis, K, O.resolve_k0(K, k0_frac), keep, order,
+                     label=f"N=900 D={D} k={K} K0={O.resolve_k0(K, k0_frac)}")
