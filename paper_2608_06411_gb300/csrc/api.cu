@@ -51,7 +51,7 @@ struct map_ctx {
   int32_t* h_done = nullptr;        // pinned, mapped
   int* h_status_dev = nullptr; int32_t* h_done_dev = nullptr;   // their device aliases
   cudaStream_t s_in = nullptr, s_out = nullptr;   // map_prune copy streams (host buffers)
-  cudaStream_t s_aux = nullptr;     // question branch of the predictor, concurrent with the visual one
+  cudaStream_t s_aux = nullptr;     // question branch of the distillation step, beside the visual one
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   bool timing = false;
   std::vector<TimedPair> pairs;
@@ -200,42 +200,76 @@ GemmDesc linear_desc(map_ctx* c, const void* x, long long rows, int K, const voi
   return d;
 }
 
-// Predictor for one modality (Eq. 3): x [rows, D] -> RoPE(Wp f(x)) * scale [rows, dp] with
+// Predictor of one modality (Eq. 3): x [rows, D] -> RoPE(Wp f(x)) * scale [rows, dp] with
 // f = Linear -> GELU -> Linear, stored as three bf16 segments [rows, 3 dp] (split_kind 0:
 // hi|lo|hi, 1: hi|hi|lo) and, if aux is given, as fp32 too.  The hidden activation
 // h1 = GELU(W1 x + b1) is kept as a bf16 hi/lo pair [rows, 2 Dh] (about 16 significant bits);
 // the second layer and the projection are one folded matrix Wf = Wp W2 with bias Wp b2.
-int predictor_branch(map_ctx* c, const void* x, long long rows, const void* w1, const void* b1, const void* wf,
-                     const float* bf, DevBuf& h1, void* out3, int split_kind, float scale, float* aux,
-                     const int* pos, int pos_mod, int tile_n, cudaStream_t st, int tid_l1, int tid_p) {
+struct Modality {
+  const void* x; long long rows;
+  const void* w1; const void* b1; const void* wf; const float* bf;
+  void* h1; void* out3; int split_kind; float scale; float* aux;
+  const int* pos; int pos_mod;
+  const int* seg_valid; int seg_len;                 // rows that hold data (GemmDesc)
+};
+
+GemmDesc layer1_desc(map_ctx* c, const Modality& m, int tile_n) {
   const map_config& g = c->cfg;
-  MAP_TRY(ensure(h1, static_cast<size_t>(rows) * g.Dh * 4));
-  {
-    Timed t(c, st, tid_l1);
-    GemmDesc d = linear_desc(c, x, rows, g.D, w1, g.Dh, b1, h1.p, mapk::EPI_GELU_SPLIT);
-    d.ldc = 2LL * g.Dh;
-    d.tile_n = tile_n;
-    MAP_TRY(gemm(c, d, st));
+  GemmDesc d = linear_desc(c, m.x, m.rows, g.D, m.w1, g.Dh, m.b1, m.h1, mapk::EPI_GELU_SPLIT);
+  d.ldc = 2LL * g.Dh;
+  d.tile_n = tile_n;
+  d.seg_valid = m.seg_valid; d.seg_len = m.seg_len;
+  return d;
+}
+
+GemmDesc projection_desc(map_ctx* c, const Modality& m) {
+  const map_config& g = c->cfg;
+  // K = 3 Dh: h_hi Wf_hi + h_hi Wf_lo + h_lo Wf_hi, A = [hi | lo] against
+  // [Wf_hi | Wf_hi | Wf_lo], each block of h_hi used twice in a row (split3 K order)
+  GemmDesc d = linear_desc(c, m.h1, m.rows, 3 * g.Dh, m.wf, g.dp, nullptr, m.out3, mapk::EPI_ROPE_SPLIT3);
+  d.a_kwrap = 2 * g.Dh;
+  d.split3 = 1;
+  d.biasf = m.bf;
+  d.ldc = 3LL * g.dp;
+  d.rope = static_cast<const float2*>(c->rope.p);
+  d.rope_ld = c->rope_rows;
+  d.pos = g.rope_on ? m.pos : nullptr;      // without RoPE every position is 0: cos 1, sin 0
+  d.pos_mod = g.rope_on ? m.pos_mod : 1;
+  d.split_kind = m.split_kind;
+  d.scale = m.scale;
+  d.aux = m.aux;
+  d.seg_valid = m.seg_valid; d.seg_len = m.seg_len;
+  return d;
+}
+
+int gemm_groups(map_ctx* c, GemmDesc d, GemmDesc d2, cudaStream_t st) {
+  ++c->counters.launches;
+  d.wait_ns = d2.wait_ns = c->wait_ns;
+  cudaError_t e = mapk::launch_gemm_groups(d, d2, c->num_sms, st);
+  if (e == cudaErrorInvalidValue) return MAP_EUNSUPPORTED;
+  return cuda_err(e);
+}
+
+// Both modalities, a layer of both in one launch: the question rows' tiles, too few for the chip,
+// fill the visual rows' last wave instead of taking waves and a launch chain of their own (on a second
+// stream they ran after the visual ones wherever those fill the chip: 95 of 2180 us with 64 images).
+// With event timing on, each layer of each modality is its own launch.
+int predictor(map_ctx* c, const Modality& vis, const Modality& text, int tile_n, cudaStream_t st) {
+  if (!c->timing) {
+    MAP_TRY(gemm_groups(c, layer1_desc(c, vis, tile_n), layer1_desc(c, text, tile_n), st));
+    return gemm_groups(c, projection_desc(c, vis), projection_desc(c, text), st);
   }
   {
-    // K = 3 Dh: h_hi Wf_hi + h_hi Wf_lo + h_lo Wf_hi, A = [hi | lo] against
-    // [Wf_hi | Wf_hi | Wf_lo], each block of h_hi used twice in a row (split3 K order)
-    Timed t(c, st, tid_p);
-    GemmDesc d = linear_desc(c, h1.p, rows, 3 * g.Dh, wf, g.dp, nullptr, out3, mapk::EPI_ROPE_SPLIT3);
-    d.a_kwrap = 2 * g.Dh;
-    d.split3 = 1;
-    d.biasf = bf;
-    d.ldc = 3LL * g.dp;
-    d.rope = static_cast<const float2*>(c->rope.p);
-    d.rope_ld = c->rope_rows;
-    d.pos = g.rope_on ? pos : nullptr;      // without RoPE every position is 0: cos 1, sin 0
-    d.pos_mod = g.rope_on ? pos_mod : 1;
-    d.split_kind = split_kind;
-    d.scale = scale;
-    d.aux = aux;
-    MAP_TRY(gemm(c, d, st));
+    Timed t(c, st, MAP_K_GEMM_TEXT);
+    MAP_TRY(gemm(c, layer1_desc(c, text, tile_n), st));
+    MAP_TRY(gemm(c, projection_desc(c, text), st));
   }
-  return MAP_OK;
+  {
+    Timed t(c, st, MAP_K_GEMM_FV1);
+    MAP_TRY(gemm(c, layer1_desc(c, vis, tile_n), st));
+  }
+  Timed t(c, st, MAP_K_GEMM_WK);
+  return gemm(c, projection_desc(c, vis), st);
 }
 
 // nv (host, B entries, or nullptr = every image has N tokens): valid visual tokens per image;
@@ -281,20 +315,17 @@ int score_impl(map_ctx* c, const void* text, const void* vis, const int32_t* len
   const int dp3 = 3 * g.dp;
   MAP_TRY(ensure(c->kb, static_cast<size_t>(vrows) * dp3 * 2));
   MAP_TRY(ensure(c->qb, static_cast<size_t>(total_m) * dp3 * 2));
-  // The two branches are independent until Eq. 3: the question branch runs on a second stream
-  // (it fills SMs that a small batch's visual GEMMs leave idle), joined before the logits.
-  MAP_TRY(ensure_aux(c));
-  int tile_v = 0, tile_t = 0;
-  mapk::predictor_tile_widths(static_cast<int>(vrows), static_cast<int>(total_m), g.Dh, g.D, c->num_sms, &tile_v, &tile_t);
-  CU_TRY(cudaEventRecord(c->ev_fork, st));
-  CU_TRY(cudaStreamWaitEvent(c->s_aux, c->ev_fork, 0));
-  MAP_TRY(predictor_branch(c, text, total_m, c->w[0], c->w[1], c->wqt, c->bqt, c->th1, c->qb.p, 1,
-                           1.0f / std::sqrt(static_cast<float>(g.dp)), q_out, static_cast<const int*>(c->post.p), 1,
-                           tile_t, c->s_aux, MAP_K_GEMM_TEXT, MAP_K_GEMM_TEXT));
-  CU_TRY(cudaEventRecord(c->ev_join, c->s_aux));
-  MAP_TRY(predictor_branch(c, vis, vrows, c->w[5], c->w[6], c->wkv, c->bkv, c->h1, c->kb.p, 0, 1.0f, k_out, nullptr,
-                           N, tile_v, st, MAP_K_GEMM_FV1, MAP_K_GEMM_WK));
-  CU_TRY(cudaStreamWaitEvent(st, c->ev_join, 0));
+  MAP_TRY(ensure(c->h1, static_cast<size_t>(vrows) * g.Dh * 4));
+  MAP_TRY(ensure(c->th1, static_cast<size_t>(total_m) * g.Dh * 4));
+  const Modality mt{text, total_m, c->w[0], c->w[1], c->wqt, c->bqt, c->th1.p, c->qb.p, 1,
+                    1.0f / std::sqrt(static_cast<float>(g.dp)), q_out, static_cast<const int*>(c->post.p), 1, nullptr, 0};
+  const Modality mv{vis, vrows, c->w[5], c->w[6], c->wkv, c->bkv, c->h1.p, c->kb.p, 0, 1.0f, k_out, nullptr, N, d_nv, N};
+  long long valid = vrows;
+  if (nv) {
+    valid = 0;
+    for (int b = 0; b < B; ++b) valid += nv[b];
+  }
+  MAP_TRY(predictor(c, mv, mt, mapk::predictor_tile_width(valid, total_m, g.Dh, g.D, c->num_sms), st));
   // Eq. 3 on the tensor cores: logits tile [visual tokens x question tokens] of one image,
   // pass 1 -> per-slab column (max, sum exp), combine -> max + ln(sum), pass 2 -> mean.
   const int m_tiles = (N + 127) / 128, nparts = 4 * m_tiles;
@@ -464,6 +495,7 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
       pd.B = s.Vg; pd.b_rows_total = static_cast<long long>(B) * R; pd.b_row_stride = R; pd.b_base = S;
       pd.M = N; pd.N = kProjMaxBasis; pd.K = g.D; pd.batch = B; pd.n_limit = s.proj_lim;
       pd.blist = s.blist;                         // images to project (built by proj_prep)
+      pd.m_limit = s.nvalid;
       pd.C = nullptr; pd.ldc = 0; pd.c_batch_stride = 0;
       pd.epi = mapk::EPI_PROJECT; pd.status = c->status;
       pd.proj.state = s.state; pd.proj.scores = scores; pd.proj.Ec = s.Ec; pd.proj.KP = KP;

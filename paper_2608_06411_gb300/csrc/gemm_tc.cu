@@ -35,15 +35,24 @@ namespace {
 constexpr int kBM = 128;
 constexpr int kBK = 64;
 
+// What the two row groups of one launch do not share (GemmDesc's fields of the same names).
+struct RowGroup {
+  int M;
+  void* C;
+  const __nv_bfloat16* bias;
+  const float* biasf;
+  const int* pos; int pos_mod;
+  int split_kind; float scale; float* aux;
+  const int* seg_valid; int seg_len;
+};
+
 struct KArgs {
+  RowGroup grp[2]; int groups;
   int M, N, K, batch, a_row_stride, b_row_stride;
   const int* n_limit;
-  void* C; long long ldc; long long c_batch_stride;
-  const __nv_bfloat16* bias;
+  long long ldc; long long c_batch_stride;
   const float2* rope; int rope_half; int rope_ld;
-  const int* pos; int pos_mod;
   int* status;
-  int split_kind; float scale; float* aux;
   const int* b_off;
   float2* stats; int stat_ld;
   const int* col_count;
@@ -51,7 +60,6 @@ struct KArgs {
   ProjArgs proj;
   int a_kwrap;
   int split3;
-  const float* biasf;
   const int* blist; const int* bcount;
   const int* m_limit;
   unsigned long long wait_ns;   // limit of the role waits (the drain waits keep kWaitLimitNs)
@@ -103,34 +111,118 @@ __device__ __forceinline__ float proj_value(float p, float r2, float sq, float l
   return v > 0.f ? v : 0.f;
 }
 
-struct TileCoord { int b, m_blk, n_blk, ks; bool skip; };
+struct TileCoord { int b, m_blk, n_blk, ks, grp; bool skip; };
+
+// The tensor maps of a launch: A, B and the box-stored output of each row group.
+struct Maps { CUtensorMap A[2], B[2], C[2]; };
 
 // Work unit t -> tile.  With PAIR the unit is a pair of vertically adjacent M tiles with the
 // same N tile, processed by the two CTAs of a cluster (rank 0 the upper, rank 1 the lower).
 // With split-K (ksplit > 1) a unit is also one K slice ks of its tile.
-template <bool PAIR>
+// PROJECT (one column tile, no split-K) with m_limit: only the row tiles with rows of an image are
+// units, found by a walk over the listed images (up to 64; with more, tiles past an image's rows are
+// skipped where they come up).
+constexpr int kProjWalkMax = 64;
+__device__ inline bool proj_walks(const KArgs& a, int nbatch) { return a.m_limit && nbatch <= kProjWalkMax; }
+// Image (list position) and row tile of unit t, or, when t is past the units, b = -1 - (their number).
+__device__ inline void proj_walk(const KArgs& a, int nbatch, int t, int& b, int& mu) {
+  int found = 0;
+  for (int i = 0; i < nbatch; ++i) {
+    const int img = a.blist ? __ldg(a.blist + i) : i;
+    const int n = (min(a.M, __ldg(a.m_limit + img)) + kBM - 1) / kBM;
+    if (t < found + n) {
+      b = i;
+      mu = t - found;
+      return;
+    }
+    found += n;
+  }
+  b = -1 - found;
+  mu = 0;
+}
+
+template <bool PAIR, bool PROJECT>
 __device__ __forceinline__ TileCoord tile_coord(const KArgs& a, int t, int nbatch, int m_units, int n_tiles, int BN,
                                                 uint32_t crank) {
   TileCoord c;
-  const int tiles = m_units * n_tiles;
-  const int per = tiles * a.ksplit;
-  c.b = t / per;
-  int rem = t - c.b * per;
-  c.ks = rem / tiles;
-  rem -= c.ks * tiles;
-  const int mu = rem / n_tiles;
-  c.n_blk = rem - mu * n_tiles;
+  int mu;
+  if (PROJECT && proj_walks(a, nbatch)) {
+    proj_walk(a, nbatch, t, c.b, mu);
+    c.ks = c.n_blk = 0;
+  } else {
+    const int tiles = m_units * n_tiles;
+    const int per = tiles * a.ksplit;
+    c.b = t / per;
+    int rem = t - c.b * per;
+    c.ks = rem / tiles;
+    rem -= c.ks * tiles;
+    mu = rem / n_tiles;
+    c.n_blk = rem - mu * n_tiles;
+  }
   if (a.blist) c.b = __ldg(a.blist + c.b);
   c.m_blk = PAIR ? 2 * mu + static_cast<int>(crank) : mu;
+  c.grp = 0;
   int lim = a.n_limit ? min(a.N, __ldg(a.n_limit + c.b)) : a.N;
   c.skip = c.n_blk * BN >= lim;
+  if (PROJECT && a.m_limit && mu * kBM >= __ldg(a.m_limit + c.b)) c.skip = true;
+  return c;
+}
+
+// Row groups: the predictor's two modalities in one launch (same N and K, other rows and weights),
+// the units of the first followed by those of the second, so that neither waits for the other's
+// last wave.  With seg_valid, a group's rows come in segments of seg_len of which the first
+// seg_valid[s] hold data: only row tiles with such rows are units, counted and found by a walk over
+// the segments (up to kWalkMax of them: a few hundred cycles a tile; with more, tiles without data
+// are skipped where they come up).
+constexpr int kWalkMax = 64;
+
+__device__ __forceinline__ bool walks(const RowGroup& q) {
+  return q.seg_valid && (q.M + q.seg_len - 1) / q.seg_len <= kWalkMax;
+}
+// The i-th row tile (of `rows` rows) with data, or, when i is past them, -1 - (their number).
+__device__ inline int walk_tiles(const RowGroup& q, int rows, int i) {
+  int next = 0, found = 0;                           // first tile not yet counted, tiles counted
+  for (int s = 0; s * q.seg_len < q.M; ++s) {
+    const int r0 = s * q.seg_len, r1 = min(q.M, r0 + __ldg(q.seg_valid + s));
+    const int first = max(r0 / rows, next), last = (r1 - 1) / rows;
+    if (r1 <= r0 || last < first) continue;
+    if (i < found + last - first + 1) return first + (i - found);
+    found += last - first + 1;
+    next = last + 1;
+  }
+  return -1 - found;
+}
+__device__ __forceinline__ int group_units(const RowGroup& q, int rows) {
+  return walks(q) ? -1 - walk_tiles(q, rows, 0x7FFFFFFF) : (q.M + rows - 1) / rows;
+}
+
+template <bool PAIR>
+__device__ __forceinline__ TileCoord group_coord(const KArgs& a, int t, int units0, int n_tiles, uint32_t crank) {
+  constexpr int ROWS = PAIR ? 2 * kBM : kBM;
+  TileCoord c;
+  c.b = c.ks = 0;
+  c.grp = t >= units0 * n_tiles;
+  if (c.grp) t -= units0 * n_tiles;
+  const RowGroup& q = a.grp[c.grp];
+  int mu = t / n_tiles;
+  c.n_blk = t - mu * n_tiles;
+  c.skip = false;
+  if (walks(q)) {
+    mu = walk_tiles(q, ROWS, mu);
+  } else if (q.seg_valid) {
+    const int r0 = mu * ROWS, r1 = min(q.M, r0 + ROWS);
+    c.skip = true;
+    for (int s = r0 / q.seg_len; s * q.seg_len < r1; ++s)
+      if (max(r0, s * q.seg_len) < s * q.seg_len + __ldg(q.seg_valid + s)) c.skip = false;
+  }
+  c.m_blk = PAIR ? 2 * mu + static_cast<int>(crank) : mu;
   return c;
 }
 
 template <int BN, int STAGES, int EPI, bool CG2>
 __global__ void __launch_bounds__(Smem<BN, STAGES, EPI, CG2>::THREADS, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmC, KArgs a) {
+gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs a) {
+  constexpr bool GROUPED = EPI == EPI_GELU_SPLIT || EPI == EPI_ROPE_SPLIT3;
   using S = Smem<BN, STAGES, EPI, CG2>;
   constexpr bool PAIR = CG2;
   constexpr uint32_t IDESC = idesc_bf16(CG2 ? 2 * kBM : kBM, BN);
@@ -166,7 +258,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     *abort_flag = 0;
     fence_mbar_init();
   }
-  if (warp == 0 && lane == 0) { tma_prefetch_desc(&tmA); tma_prefetch_desc(&tmB); }
+  if (warp == 0 && lane == 0) { tma_prefetch_desc(&maps.A[0]); tma_prefetch_desc(&maps.B[0]); }
   pdl_enter();                                    // inputs below come from the previous kernel
   if (warp == 1) {
     if constexpr (CG2) { tmem_alloc_cg2(tmem_slot, S::TMEM_COLS); tmem_relinquish_cg2(); }
@@ -178,10 +270,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const uint32_t tmem_base = *tmem_slot;
 
   const int m_tiles = (a.M + kBM - 1) / kBM;
+  constexpr int UNIT_ROWS = PAIR ? 2 * kBM : kBM;
+  int group0 = 0;                                 // row units of the first group
+  if constexpr (GROUPED) group0 = group_units(a.grp[0], UNIT_ROWS);
   const int m_units = PAIR ? (m_tiles + 1) / 2 : m_tiles;
   const int n_tiles = (a.N + BN - 1) / BN;
   const int nbatch = a.blist ? min(a.batch, *a.bcount) : a.batch;
-  const int total = nbatch * m_units * n_tiles * a.ksplit;
+  int total = nbatch * m_units * n_tiles * a.ksplit;
+  if constexpr (GROUPED) {
+    total = group0;
+    if (a.groups > 1) total += group_units(a.grp[1], UNIT_ROWS);
+    total *= n_tiles;
+  }
+  if constexpr (EPI == EPI_PROJECT) {
+    if (proj_walks(a, nbatch)) {
+      int none;
+      proj_walk(a, nbatch, 0x7FFFFFFF, total, none);
+      total = -1 - total;
+    }
+  }
+  auto coord = [&](int t) {
+    if constexpr (GROUPED) return group_coord<PAIR>(a, t, group0, n_tiles, crank);
+    else return tile_coord<PAIR, EPI == EPI_PROJECT>(a, t, nbatch, m_units, n_tiles, BN, crank);
+  };
   constexpr bool PRODUCTS = EPI == EPI_F32;       // the epilogue of the segmented products
   // K blocks of one product of image c.b
   auto product_kblocks = [&](const TileCoord& c) {
@@ -223,7 +334,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       uint32_t stage = 0, phase = 0;
       bool ok = true;
       for (int t = unit0; t < total && ok; t += units_step) {
-        TileCoord c = tile_coord<PAIR>(a, t, nbatch, m_units, n_tiles, BN, crank);
+        TileCoord c = coord(t);
         if (c.skip) continue;
         const int arow = c.b * a.a_row_stride + c.m_blk * kBM;
         const int brow = (a.b_off ? __ldg(a.b_off + c.b) : c.b * a.b_row_stride + a.b_base) + c.n_blk * BN;
@@ -261,15 +372,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               const int k0 = j * kBK;
               if (amn) {
 #pragma unroll
-                for (int h = 0; h < kBM; h += 64) load(da + h * 128, &tmA, aseg + m0 + h, arb + k0);
+                for (int h = 0; h < kBM; h += 64) load(da + h * 128, &maps.A[0], aseg + m0 + h, arb + k0);
               } else {
-                load(da, &tmA, aseg + k0, arb + m0);
+                load(da, &maps.A[0], aseg + k0, arb + m0);
               }
               if (bmn) {
 #pragma unroll
-                for (int h = 0; h < BR; h += 64) load(db + h * 128, &tmB, bseg + n0 + h, brb + k0);
+                for (int h = 0; h < BR; h += 64) load(db + h * 128, &maps.B[0], bseg + n0 + h, brb + k0);
               } else {
-                load(db, &tmB, bseg + k0, brb + n0);
+                load(db, &maps.B[0], bseg + k0, brb + n0);
               }
               last_par[stage] = static_cast<int>(phase);
               if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -283,6 +394,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             continue;
           }
         }
+        const CUtensorMap* const tmA = &maps.A[GROUPED ? c.grp : 0];
+        const CUtensorMap* const tmB = &maps.B[GROUPED ? c.grp : 0];
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(&empty[stage], phase ^ 1, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
           int ac, bc;
@@ -291,12 +404,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             // both CTAs' copies complete on the leader's full barrier, which expects them all
             if (crank == 0) mbar_arrive_expect_tx(&full[stage], 2 * S::STAGE_BYTES);
             const uint32_t fb = mapa_u32(&full[stage], 0);
-            tma_load_2d_cg2(sA + stage * S::A_BYTES, &tmA, fb, ac, arow);
-            tma_load_2d_cg2(sB + stage * S::B_BYTES, &tmB, fb, bc, brow + static_cast<int>(crank) * (BN / 2));
+            tma_load_2d_cg2(sA + stage * S::A_BYTES, tmA, fb, ac, arow);
+            tma_load_2d_cg2(sB + stage * S::B_BYTES, tmB, fb, bc, brow + static_cast<int>(crank) * (BN / 2));
           } else {
             mbar_arrive_expect_tx(&full[stage], S::STAGE_BYTES);
-            tma_load_2d(sA + stage * S::A_BYTES, &tmA, &full[stage], ac, arow);
-            tma_load_2d(sB + stage * S::B_BYTES, &tmB, &full[stage], bc, brow);
+            tma_load_2d(sA + stage * S::A_BYTES, tmA, &full[stage], ac, arow);
+            tma_load_2d(sB + stage * S::B_BYTES, tmB, &full[stage], bc, brow);
           }
           last_par[stage] = static_cast<int>(phase);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -316,7 +429,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const uint32_t astep = (amn ? 2048 : 32) >> 4, bstep = (bmn ? 2048 : 32) >> 4;
       const uint32_t pid = IDESC | (amn ? 1u << 15 : 0u) | (bmn ? 1u << 16 : 0u);
       for (int t = unit0; t < total && ok; t += units_step) {
-        TileCoord c = tile_coord<PAIR>(a, t, nbatch, m_units, n_tiles, BN, crank);
+        TileCoord c = coord(t);
         if (c.skip) continue;
         if (!mbar_wait(&tempty[acc], acc_phase ^ 1, a.status, abort_flag, a.wait_ns)) break;
         tc_fence_after();
@@ -380,7 +493,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t eg_phase = 0;
     bool eg_ok = true;
     for (int t = unit0; t < total && eg_ok; t += units_step) {
-      TileCoord c = tile_coord<PAIR>(a, t, nbatch, m_units, n_tiles, BN, crank);
+      TileCoord c = coord(t);
       if (c.skip) continue;
       if constexpr (S::PROJ) {
         if (c.b != staged_b) {                     // stage L and 1/r of this image's R0 basis
@@ -414,7 +527,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       }
       const int row = c.m_blk * kBM + r_in_tile;
-      const bool row_ok = row < (a.m_limit ? min(a.M, __ldg(a.m_limit + c.b)) : a.M);
+      const RowGroup& q = a.grp[GROUPED ? c.grp : 0];
+      const bool row_ok = row < (a.m_limit ? min(q.M, __ldg(a.m_limit + c.b)) : q.M);
       const int lim = a.n_limit ? min(a.N, __ldg(a.n_limit + c.b)) : a.N;
       const int col0 = c.n_blk * BN;
       // the RoPE factors the epilogue starts with are loaded while the tile's MMAs still run
@@ -426,7 +540,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       };
       if constexpr (S::TSTORE_ROPE) {
         int pos = 0;
-        if (row_ok) pos = a.pos ? __ldg(a.pos + row) : row % a.pos_mod;
+        if (row_ok) pos = q.pos ? __ldg(q.pos + row) : row % q.pos_mod;
         rt = a.rope + pos;
         load_rope(0);
       }
@@ -438,9 +552,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if constexpr (EPI == EPI_ROPE_F32) {
         // BN == dp: the whole row is in this tile; rotate pairs (i, i + dp/2).
         constexpr int HALF = BN / 2;
-        float* out = reinterpret_cast<float*>(a.C) + crow;
+        float* out = reinterpret_cast<float*>(q.C) + crow;
         int pos = 0;
-        if (row_ok) pos = a.pos ? __ldg(a.pos + row) : row % a.pos_mod;
+        if (row_ok) pos = q.pos ? __ldg(q.pos + row) : row % q.pos_mod;
         const float2* rt = a.rope + pos;
 #pragma unroll 1
         for (int ch = 0; ch < HALF / 32; ++ch) {
@@ -467,8 +581,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // BN == dp = 128; x = RoPE(acc + bias) * scale as bf16 (hi, lo) segments, staged per warp
         // in shared memory and written by TMA box stores (rows past M are clipped)
         constexpr int HALF = BN / 2;
-        float* aux = (a.aux && row_ok) ? a.aux + static_cast<long long>(row) * BN : nullptr;
-        const int seg_lo = a.split_kind == 0 ? 1 : 2;   // keys [hi, lo, hi], queries [hi, hi, lo]
+        float* aux = (q.aux && row_ok) ? q.aux + static_cast<long long>(row) * BN : nullptr;
+        const int seg_lo = q.split_kind == 0 ? 1 : 2;   // keys [hi, lo, hi], queries [hi, hi, lo]
         const int ew = warp - 2;
         const int y = c.b * a.a_row_stride + c.m_blk * kBM + lane_grp * 32;
         uint8_t* sb = stg + ew * 8192;                 // [hi1 | lo1 | hi2 | lo2], 32 rows x 64 B each
@@ -487,9 +601,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int u = 0; u < 8; ++u) {
               const float2 rc = cs[j + u];
               float x1 = __uint_as_float(r1[j + u]), x2 = __uint_as_float(r2[j + u]);
-              if (a.biasf) {
-                x1 += __ldg(a.biasf + ch * 32 + j + u);
-                x2 += __ldg(a.biasf + HALF + ch * 32 + j + u);
+              if (q.biasf) {
+                x1 += __ldg(q.biasf + ch * 32 + j + u);
+                x2 += __ldg(q.biasf + HALF + ch * 32 + j + u);
               }
               o1[u] = x1 * rc.x - x2 * rc.y;
               o2[u] = x2 * rc.x + x1 * rc.y;
@@ -503,7 +617,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               }
             }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) { o1[u] *= a.scale; o2[u] *= a.scale; }
+            for (int u = 0; u < 8; ++u) { o1[u] *= q.scale; o2[u] *= q.scale; }
             uint32_t h1[4], l1[4], h2[4], l2[4];
 #pragma unroll
             for (int u = 0; u < 8; u += 2) {
@@ -526,8 +640,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
             for (int sg = 0; sg < 3; ++sg) {
               const int x = sg * BN + ch * 32;
-              tma_store_2d(&tmC, sb + (sg == seg_lo ? 2048 : 0), x, y);
-              tma_store_2d(&tmC, sb + (sg == seg_lo ? 6144 : 4096), x + HALF, y);
+              tma_store_2d(&maps.C[GROUPED ? c.grp : 0], sb + (sg == seg_lo ? 2048 : 0), x, y);
+              tma_store_2d(&maps.C[GROUPED ? c.grp : 0], sb + (sg == seg_lo ? 6144 : 4096), x + HALF, y);
             }
             bulk_commit_group();
           }
@@ -535,13 +649,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       } else if constexpr (EPI == EPI_ROPE_SPLIT3) {
         // BN == dp; x = RoPE(acc) * scale, stored as bf16 (hi, lo) segments
         constexpr int HALF = BN / 2;
-        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.C) + crow;
-        float* aux = a.aux ? a.aux + static_cast<long long>(row) * BN : nullptr;
+        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(q.C) + crow;
+        float* aux = q.aux ? q.aux + static_cast<long long>(row) * BN : nullptr;
         int pos = 0;
-        if (row_ok) pos = a.pos ? __ldg(a.pos + row) : row % a.pos_mod;
+        if (row_ok) pos = q.pos ? __ldg(q.pos + row) : row % q.pos_mod;
         const float2* rt = a.rope + pos;
         // segment order: keys [hi, lo, hi], queries [hi, hi, lo]
-        const int seg_lo = a.split_kind == 0 ? 1 : 2;
+        const int seg_lo = q.split_kind == 0 ? 1 : 2;
 #pragma unroll 1
         for (int ch = 0; ch < HALF / 32; ++ch) {
           uint32_t r1[32], r2[32];
@@ -555,9 +669,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               for (int u = 0; u < 8; ++u) {
                 const float2 cs = __ldg(rt + static_cast<long long>(ch * 32 + j + u) * a.rope_ld);
                 float x1 = __uint_as_float(r1[j + u]), x2 = __uint_as_float(r2[j + u]);
-                if (a.biasf) {
-                  x1 += __ldg(a.biasf + ch * 32 + j + u);
-                  x2 += __ldg(a.biasf + HALF + ch * 32 + j + u);
+                if (q.biasf) {
+                  x1 += __ldg(q.biasf + ch * 32 + j + u);
+                  x2 += __ldg(q.biasf + HALF + ch * 32 + j + u);
                 }
                 o1[u] = x1 * cs.x - x2 * cs.y;
                 o2[u] = x2 * cs.x + x1 * cs.y;
@@ -571,7 +685,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
               }
 #pragma unroll
-              for (int u = 0; u < 8; ++u) { o1[u] *= a.scale; o2[u] *= a.scale; }
+              for (int u = 0; u < 8; ++u) { o1[u] *= q.scale; o2[u] *= q.scale; }
               uint32_t h1[4], l1[4], h2[4], l2[4];
 #pragma unroll
               for (int u = 0; u < 8; u += 2) {
@@ -640,7 +754,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           for (int j = 0; j < 32; ++j) acc_p += __expf(__uint_as_float(r[j]) - cn[j]);
         }
         if (row < a.M) {   // rows past the image's valid tokens (m_limit) get 0
-          float* out = reinterpret_cast<float*>(a.C) + static_cast<long long>(c.b) * a.c_batch_stride;
+          float* out = reinterpret_cast<float*>(q.C) + static_cast<long long>(c.b) * a.c_batch_stride;
           out[static_cast<long long>(c.n_blk) * a.M + row] =
               row_ok ? acc_p / static_cast<float>(ncol > 0 ? ncol : 1) : 0.f;
         }
@@ -738,7 +852,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // products with per-image A rows write C at the same rows
         const long long orow = a.pr.n > 0 && a.pr.a_off && !a.pr.a_mn
                                    ? (__ldg(a.pr.a_off + c.b) + static_cast<long long>(row)) * a.ldc : crow;
-        float* out = reinterpret_cast<float*>(a.C) + orow + col0 + c.ks * a.c_split_stride;
+        float* out = reinterpret_cast<float*>(q.C) + orow + col0 + c.ks * a.c_split_stride;
 #pragma unroll 1
         for (int ch = 0; ch < BN / 32; ++ch) {
           uint32_t r[32];
@@ -776,8 +890,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
           for (int j = 0; j < 32; j += 2) {
             float x0 = __uint_as_float(r[j]), x1 = __uint_as_float(r[j + 1]);
-            if (a.bias) {
-              const __nv_bfloat162 bb = __ldg(reinterpret_cast<const __nv_bfloat162*>(a.bias + cbase + j));
+            if (q.bias) {
+              const __nv_bfloat162 bb = __ldg(reinterpret_cast<const __nv_bfloat162*>(q.bias + cbase + j));
               x0 += __bfloat162float(bb.x);
               x1 += __bfloat162float(bb.y);
             }
@@ -799,13 +913,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {                                 // rows past M are clipped by the store
-            tma_store_2d(&tmC, hb, cbase, y);
-            tma_store_2d(&tmC, hb + 2048, a.N + cbase, y);
+            tma_store_2d(&maps.C[GROUPED ? c.grp : 0], hb, cbase, y);
+            tma_store_2d(&maps.C[GROUPED ? c.grp : 0], hb + 2048, a.N + cbase, y);
             bulk_commit_group();
           }
         }
       } else {
-        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(a.C) + crow + col0;
+        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(q.C) + crow + col0;
 #pragma unroll 1
         for (int ch = 0; ch < BN / 32; ++ch) {
           uint32_t r[32];
@@ -817,8 +931,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
             for (int j = 0; j < 32; j += 2) {
               float x0 = __uint_as_float(r[j]), x1 = __uint_as_float(r[j + 1]);
-              if (a.bias) {
-                const __nv_bfloat162 bb = __ldg(reinterpret_cast<const __nv_bfloat162*>(a.bias + cbase + j));
+              if (q.bias) {
+                const __nv_bfloat162 bb = __ldg(reinterpret_cast<const __nv_bfloat162*>(q.bias + cbase + j));
                 x0 += __bfloat162float(bb.x);
                 x1 += __bfloat162float(bb.y);
               }
@@ -896,22 +1010,20 @@ bool make_map(CUtensorMap* m, const void* base, long long rows, int K, int box_r
   return r == CUDA_SUCCESS;
 }
 
-template <int BN, int STAGES, int EPI, bool PAIR = false>
-cudaError_t run(const GemmDesc& d, const KArgs& ka, int num_sms, cudaStream_t st) {
-  using S = Smem<BN, STAGES, EPI, PAIR>;
-  CUtensorMap ta, tb;
+// Tensor maps of one row group.
+template <int BN, int EPI, bool PAIR, bool TSTORE>
+bool make_maps(const GemmDesc& d, CUtensorMap& ta, CUtensorMap& tb, CUtensorMap& tc) {
   const bool prod = d.pr.n > 0;
   const int acols = prod ? d.pr.a_cols : (d.a_kwrap > 0 ? d.a_kwrap : d.K);
   const int bcols = prod ? d.pr.b_cols : d.K;
-  if (!make_map(&ta, d.A, d.a_rows_total, acols, prod && d.pr.a_mn ? 64 : kBM)) return cudaErrorInvalidValue;
-  if (!make_map(&tb, d.B, d.b_rows_total, bcols, prod && d.pr.b_mn ? 64 : (PAIR ? BN / 2 : BN)))
-    return cudaErrorInvalidValue;
-  CUtensorMap tc = ta;
-  if constexpr (S::TSTORE) {       // output [rows, ldc] bf16, 32x32 boxes, 64-byte swizzle
+  if (!make_map(&ta, d.A, d.a_rows_total, acols, prod && d.pr.a_mn ? 64 : kBM)) return false;
+  if (!make_map(&tb, d.B, d.b_rows_total, bcols, prod && d.pr.b_mn ? 64 : (PAIR ? BN / 2 : BN))) return false;
+  tc = ta;
+  if constexpr (TSTORE) {       // output [rows, ldc] bf16, 32x32 boxes, 64-byte swizzle
     // box stores clip at a_rows_total, which is the row bound M only for one flat batch
-    if (d.batch != 1 || d.a_rows_total != d.M) return cudaErrorInvalidValue;
+    if (d.batch != 1 || d.a_rows_total != d.M) return false;
     auto fn = encode_fn();
-    if (!fn) return cudaErrorInvalidValue;
+    if (!fn) return false;
     cuuint64_t dims[2] = {static_cast<cuuint64_t>(d.ldc), static_cast<cuuint64_t>(d.a_rows_total)};
     cuuint64_t strides[1] = {static_cast<cuuint64_t>(d.ldc) * 2};
     cuuint32_t box[2] = {32, 32};
@@ -919,8 +1031,19 @@ cudaError_t run(const GemmDesc& d, const KArgs& ka, int num_sms, cudaStream_t st
     if (fn(&tc, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, d.C, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
            CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
         CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
+      return false;
   }
+  return true;
+}
+
+// d2: the second row group (predictor epilogues), or nullptr.
+template <int BN, int STAGES, int EPI, bool PAIR = false>
+cudaError_t run(const GemmDesc& d, const GemmDesc* d2, const KArgs& ka, int num_sms, cudaStream_t st) {
+  using S = Smem<BN, STAGES, EPI, PAIR>;
+  constexpr bool GROUPED = EPI == EPI_GELU_SPLIT || EPI == EPI_ROPE_SPLIT3;
+  Maps maps;
+  if (!make_maps<BN, EPI, PAIR, S::TSTORE>(d, maps.A[0], maps.B[0], maps.C[0])) return cudaErrorInvalidValue;
+  if (!make_maps<BN, EPI, PAIR, S::TSTORE>(d2 ? *d2 : d, maps.A[1], maps.B[1], maps.C[1])) return cudaErrorInvalidValue;
   auto kern = gemm_tc_kernel<BN, STAGES, EPI, PAIR>;
   static bool attr_set = false;
   if (!attr_set) {
@@ -928,10 +1051,15 @@ cudaError_t run(const GemmDesc& d, const KArgs& ka, int num_sms, cudaStream_t st
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  const int m_tiles = (d.M + kBM - 1) / kBM, n_tiles = (d.N + BN - 1) / BN;
+  const int n_tiles = (d.N + BN - 1) / BN, rows = PAIR ? 2 * kBM : kBM;
+  int units = d.batch * ((d.M + rows - 1) / rows) * n_tiles * ka.ksplit;
+  if (GROUPED) {
+    units = 0;
+    for (int g = 0; g < ka.groups; ++g) units += (ka.grp[g].M + rows - 1) / rows;   // the most there can be
+    units *= n_tiles;
+  }
+  if (units == 0) return cudaSuccess;
   if (PAIR) {
-    const int units = d.batch * ((m_tiles + 1) / 2) * n_tiles * ka.ksplit;
-    if (units == 0) return cudaSuccess;
     const int grid = 2 * std::max(1, std::min(units, num_sms / 2));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -947,53 +1075,78 @@ cudaError_t run(const GemmDesc& d, const KArgs& ka, int num_sms, cudaStream_t st
     attr[1].val.programmaticStreamSerializationAllowed = pdl_disabled() ? 0 : 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, ta, tb, tc, ka);
+    return cudaLaunchKernelEx(&cfg, kern, maps, ka);
   }
-  const int tiles = d.batch * m_tiles * n_tiles * ka.ksplit;
-  if (tiles == 0) return cudaSuccess;
-  const int grid = std::max(1, std::min(tiles, num_sms));
-  return launch_k(kern, dim3(grid), dim3(S::THREADS), S::TOTAL, st, ta, tb, tc, ka);
+  const int grid = std::max(1, std::min(units, num_sms));
+  return launch_k(kern, dim3(grid), dim3(S::THREADS), S::TOTAL, st, maps, ka);
+}
+
+// The fields of a row group.
+RowGroup row_group(const GemmDesc& d) {
+  RowGroup g{};
+  g.M = d.M; g.C = d.C;
+  g.bias = static_cast<const __nv_bfloat16*>(d.bias); g.biasf = d.biasf;
+  g.pos = d.pos; g.pos_mod = d.pos_mod > 0 ? d.pos_mod : 1;
+  g.split_kind = d.split_kind; g.scale = d.scale; g.aux = d.aux;
+  g.seg_valid = d.seg_valid; g.seg_len = d.seg_len;
+  return g;
 }
 
 }  // namespace
 
-// Columns of the 2-SM tiles (256 rows) of the first layers of both predictor branches, which run
-// side by side: the pair of widths with the least time by the model
+// Columns of the first predictor layer's 2-SM tiles (256 rows of either branch, one launch): the
+// width with the least time by the model
 //   waves of the tiles over the SM pairs x K blocks x the longer of the MMA (2 BN cycles) and the
-//   copies into an SM (256 + BN), and the last tile's epilogue (40 BN),
-// the two branches at once where their tiles fit the chip together, else one after the other.
-// Large batches take 256.  With few rows the chip would idle behind a few wide tiles, each a chain
-// of K / 64 blocks: N = 576 takes 64 (48 pairs instead of 12), N = 2880 192 (72 instead of 48)
-// beside a question branch kept on the four pairs left.  The width changes no sum.  One image of
-// 576 tokens: 234.5 -> 226.8 us per call; of 2880: 312.9 -> 310.8 us.
-void predictor_tile_widths(int m_vis, int m_text, int N, int K, int num_sms, int* w_vis, int* w_text) {
-  constexpr int kWidths[4] = {256, 192, 128, 64};
+//   copies into an SM (256 + BN), and the last tile's epilogue (40 BN).
+// Large batches take 256.  With few rows the chip would idle behind a few wide tiles, each a chain of
+// K / 64 blocks: 576 visual and 32 question rows take 64 (64 pairs instead of 16).  The width changes
+// no sum.
+int predictor_tile_width(long long m_vis, long long m_text, int N, int K, int num_sms) {
   const long long pairs = std::max(1, num_sms / 2);
-  auto units = [&](int M, int bn) {
-    return static_cast<long long>((M + 2 * kBM - 1) / (2 * kBM)) * ((N + bn - 1) / bn);
-  };
-  auto time = [&](int M, int bn) {
-    return (units(M, bn) + pairs - 1) / pairs * (K / kBK) * std::max(2 * bn, 256 + bn) + 40 * bn;
-  };
+  const long long rows = (m_vis + 2 * kBM - 1) / (2 * kBM) + (m_text + 2 * kBM - 1) / (2 * kBM);
   long long best = -1;
-  for (int v : kWidths)
-    for (int w : kWidths) {
-      const long long tv = time(m_vis, v), tw = time(m_text, w);
-      const long long t = units(m_vis, v) + units(m_text, w) <= pairs ? std::max(tv, tw) : tv + tw;
-      if (best < 0 || t < best) {
-        best = t;
-        *w_vis = v;
-        *w_text = w;
-      }
+  int width = 256;
+  for (int bn : {256, 192, 128, 64}) {
+    const long long units = rows * ((N + bn - 1) / bn);
+    const long long t = (units + pairs - 1) / pairs * (K / kBK) * std::max(2 * bn, 256 + bn) + 40 * bn;
+    if (best < 0 || t < best) {
+      best = t;
+      width = bn;
     }
+  }
+  return width;
 }
 
+namespace {
+cudaError_t check_desc(const GemmDesc& d);
+cudaError_t launch_checked(const GemmDesc& d, const GemmDesc* d2, int num_sms, cudaStream_t st);
+}  // namespace
+
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
+  const cudaError_t e = check_desc(d);
+  if (e != cudaSuccess) return e;
+  return d.M == 0 ? cudaSuccess : launch_checked(d, nullptr, num_sms, st);
+}
+
+cudaError_t launch_gemm_groups(const GemmDesc& d, const GemmDesc& d2, int num_sms, cudaStream_t st) {
+  cudaError_t e = check_desc(d);
+  if (e == cudaSuccess) e = check_desc(d2);
+  if (e != cudaSuccess) return e;
+  // what the groups share, and what only one group has
+  if ((d.epi != EPI_GELU_SPLIT && d.epi != EPI_ROPE_SPLIT3) || d2.epi != d.epi || d2.N != d.N || d2.K != d.K ||
+      d2.ldc != d.ldc || d2.a_kwrap != d.a_kwrap || d2.split3 != d.split3 || d2.rope != d.rope ||
+      d2.rope_ld != d.rope_ld || d2.tile_n != d.tile_n || d2.wait_ns != d.wait_ns || d2.status != d.status ||
+      d.batch != 1 || d2.batch != 1 || d.M == 0 || d2.M == 0)
+    return cudaErrorInvalidValue;
+  return launch_checked(d, &d2, num_sms, st);
+}
+
+namespace {
+cudaError_t check_desc(const GemmDesc& d) {
   if (d.K <= 0 || d.K % kBK != 0 || d.M < 0 || d.N <= 0 || d.batch <= 0) return cudaErrorInvalidValue;
   if (d.a_kwrap < 0 || d.a_kwrap % kBK != 0 || d.a_kwrap > d.K) return cudaErrorInvalidValue;
   if (d.split3 && (d.K % (3 * kBK) != 0 || d.a_kwrap != 2 * (d.K / 3))) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(d.A) | reinterpret_cast<uintptr_t>(d.B)) & 15) return cudaErrorInvalidValue;
-  if (d.M == 0) return cudaSuccess;
   // every output row and column block is written with 16-byte vector stores
   const bool scalar_out = d.epi == EPI_SM_STATS || d.epi == EPI_SM_MEAN;   // float / float2 stores
   const bool f32 = d.epi == EPI_F32 || d.epi == EPI_ROPE_F32;
@@ -1007,26 +1160,10 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
   if (scalar_out && (!d.stats || (reinterpret_cast<uintptr_t>(d.stats) & 7) || (reinterpret_cast<uintptr_t>(d.C) & 3)))
     return cudaErrorInvalidValue;
   if ((d.epi == EPI_GELU_SPLIT || d.epi == EPI_BIAS_SPLIT) && d.ldc < 2LL * d.N) return cudaErrorInvalidValue;
-  KArgs ka;
-  ka.M = d.M; ka.N = d.N; ka.K = d.K; ka.batch = d.batch;
-  ka.a_row_stride = d.a_row_stride; ka.b_row_stride = d.b_row_stride;
-  ka.n_limit = d.n_limit; ka.C = d.C; ka.ldc = d.ldc; ka.c_batch_stride = d.c_batch_stride;
-  ka.bias = static_cast<const __nv_bfloat16*>(d.bias);
-  ka.rope = d.rope; ka.rope_half = d.rope_half; ka.rope_ld = d.rope_ld; ka.pos = d.pos; ka.pos_mod = d.pos_mod > 0 ? d.pos_mod : 1;
-  ka.status = d.status;
-  ka.split_kind = d.split_kind; ka.scale = d.scale; ka.aux = d.aux; ka.b_off = d.b_off;
-  ka.stats = d.stats; ka.stat_ld = d.stat_ld; ka.col_count = d.col_count;
-  ka.b_base = d.b_base; ka.proj = d.proj;
-  ka.a_kwrap = d.a_kwrap; ka.biasf = d.biasf; ka.split3 = d.split3;
-  ka.blist = d.blist; ka.bcount = d.blist ? d.bcount : nullptr;
-  ka.m_limit = d.m_limit;
-  ka.wait_ns = d.wait_ns > 0 ? static_cast<unsigned long long>(d.wait_ns) : kWaitLimitNs;
   // split-K: fp32 partial tiles only, every slice at least one K block
   if (d.ksplit < 1 || (d.ksplit > 1 && (d.epi != EPI_F32 || d.ksplit > d.K / kBK || d.c_split_stride % 4 != 0)))
     return cudaErrorInvalidValue;
-  ka.ksplit = d.ksplit; ka.c_split_stride = d.c_split_stride;
   if (d.blist && !d.bcount) return cudaErrorInvalidValue;
-  ka.pr = d.pr;
   if (d.pr.n) {      // segments start at whole boxes; K is the products' K blocks side by side
     const GemmProducts& q = d.pr;
     if (d.epi != EPI_F32 || q.n < 0 || q.n > kMaxProducts || d.a_kwrap || d.split3 || d.b_off || d.b_base ||
@@ -1036,53 +1173,79 @@ cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st) {
       if (q.a_seg[i] < 0 || q.a_seg[i] % kBK != 0 || q.b_seg[i] < 0 || q.b_seg[i] % kBK != 0)
         return cudaErrorInvalidValue;
   }
+  if (d.seg_valid && (d.seg_len < 1 || d.batch != 1 || (d.epi != EPI_GELU_SPLIT && d.epi != EPI_ROPE_SPLIT3)))
+    return cudaErrorInvalidValue;
+  return cudaSuccess;
+}
+
+cudaError_t launch_checked(const GemmDesc& d, const GemmDesc* d2, int num_sms, cudaStream_t st) {
+  KArgs ka;
+  ka.grp[0] = row_group(d);
+  ka.grp[1] = row_group(d2 ? *d2 : d);
+  ka.groups = d2 ? 2 : 1;
+  ka.M = d.M; ka.N = d.N; ka.K = d.K; ka.batch = d.batch;
+  ka.a_row_stride = d.a_row_stride; ka.b_row_stride = d.b_row_stride;
+  ka.n_limit = d.n_limit; ka.ldc = d.ldc; ka.c_batch_stride = d.c_batch_stride;
+  ka.rope = d.rope; ka.rope_half = d.rope_half; ka.rope_ld = d.rope_ld;
+  ka.status = d.status;
+  ka.b_off = d.b_off;
+  ka.stats = d.stats; ka.stat_ld = d.stat_ld; ka.col_count = d.col_count;
+  ka.b_base = d.b_base; ka.proj = d.proj;
+  ka.a_kwrap = d.a_kwrap; ka.split3 = d.split3;
+  ka.blist = d.blist; ka.bcount = d.blist ? d.bcount : nullptr;
+  ka.m_limit = d.m_limit;
+  ka.wait_ns = d.wait_ns > 0 ? static_cast<unsigned long long>(d.wait_ns) : kWaitLimitNs;
+  ka.ksplit = d.ksplit; ka.c_split_stride = d.c_split_stride;
+  ka.pr = d.pr;
   switch (d.epi) {
     case EPI_GELU_BF16:
-      if (d.N % 256 == 0) return run<256, 4, EPI_GELU_BF16>(d, ka, num_sms, st);
-      if (d.N % 64 == 0) return run<64, 8, EPI_GELU_BF16>(d, ka, num_sms, st);
+      if (d.N % 256 == 0) return run<256, 4, EPI_GELU_BF16>(d, d2, ka, num_sms, st);
+      if (d.N % 64 == 0) return run<64, 8, EPI_GELU_BF16>(d, d2, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_BIAS_BF16:
-      if (d.N % 256 == 0) return run<256, 4, EPI_BIAS_BF16>(d, ka, num_sms, st);
-      if (d.N % 64 == 0) return run<64, 8, EPI_BIAS_BF16>(d, ka, num_sms, st);
+      if (d.N % 256 == 0) return run<256, 4, EPI_BIAS_BF16>(d, d2, ka, num_sms, st);
+      if (d.N % 64 == 0) return run<64, 8, EPI_BIAS_BF16>(d, d2, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_ROPE_F32:
-      if (d.N == 64) return run<64, 8, EPI_ROPE_F32>(d, ka, num_sms, st);
-      if (d.N == 128) return run<128, 6, EPI_ROPE_F32>(d, ka, num_sms, st);
-      if (d.N == 256) return run<256, 4, EPI_ROPE_F32>(d, ka, num_sms, st);
+      if (d.N == 64) return run<64, 8, EPI_ROPE_F32>(d, d2, ka, num_sms, st);
+      if (d.N == 128) return run<128, 6, EPI_ROPE_F32>(d, d2, ka, num_sms, st);
+      if (d.N == 256) return run<256, 4, EPI_ROPE_F32>(d, d2, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_GELU_SPLIT:
       if (d.N % 256 == 0) {
         switch (d.tile_n) {
-          case 64: return run<64, 8, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
-          case 128: return run<128, 8, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
-          case 192: return run<192, 6, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
-          default: return run<256, 6, EPI_GELU_SPLIT, true>(d, ka, num_sms, st);
+          case 64: return run<64, 8, EPI_GELU_SPLIT, true>(d, d2, ka, num_sms, st);
+          case 128: return run<128, 8, EPI_GELU_SPLIT, true>(d, d2, ka, num_sms, st);
+          case 192: return run<192, 6, EPI_GELU_SPLIT, true>(d, d2, ka, num_sms, st);
+          default: return run<256, 6, EPI_GELU_SPLIT, true>(d, d2, ka, num_sms, st);
         }
       }
-      if (d.N % 64 == 0) return run<64, 8, EPI_GELU_SPLIT>(d, ka, num_sms, st);
+      if (d.N % 64 == 0) return run<64, 8, EPI_GELU_SPLIT>(d, d2, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_BIAS_SPLIT:
-      if (d.N % 256 == 0) return run<256, 6, EPI_BIAS_SPLIT, true>(d, ka, num_sms, st);
-      if (d.N % 64 == 0) return run<64, 8, EPI_BIAS_SPLIT>(d, ka, num_sms, st);
+      if (d.N % 256 == 0) return run<256, 6, EPI_BIAS_SPLIT, true>(d, d2, ka, num_sms, st);
+      if (d.N % 64 == 0) return run<64, 8, EPI_BIAS_SPLIT>(d, d2, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_ROPE_SPLIT3:   // dp = 128: 2-SM pairs share the B tile (each CTA loads 64 of its rows)
-      if (d.N == 64) return run<64, 8, EPI_ROPE_SPLIT3>(d, ka, num_sms, st);
-      if (d.N == 128) return run<128, 8, EPI_ROPE_SPLIT3, true>(d, ka, num_sms, st);
+      if (d.N == 64) return run<64, 8, EPI_ROPE_SPLIT3>(d, d2, ka, num_sms, st);
+      if (d.N == 128) return run<128, 8, EPI_ROPE_SPLIT3, true>(d, d2, ka, num_sms, st);
       return cudaErrorInvalidValue;
     case EPI_SM_STATS:
-      return run<256, 4, EPI_SM_STATS>(d, ka, num_sms, st);
+      return run<256, 4, EPI_SM_STATS>(d, d2, ka, num_sms, st);
     case EPI_SM_MEAN:
-      return run<256, 4, EPI_SM_MEAN>(d, ka, num_sms, st);
+      return run<256, 4, EPI_SM_MEAN>(d, d2, ka, num_sms, st);
     case EPI_PROJECT:
       if (d.N > kProjMaxBasis || d.batch < 1) return cudaErrorInvalidValue;
-      if (d.N <= 96) return run<96, 6, EPI_PROJECT>(d, ka, num_sms, st);
-      return run<128, 5, EPI_PROJECT>(d, ka, num_sms, st);
+      if (d.N <= 96) return run<96, 6, EPI_PROJECT>(d, d2, ka, num_sms, st);
+      return run<128, 5, EPI_PROJECT>(d, d2, ka, num_sms, st);
     case EPI_F32:   // the distillation's contractions
-      if (d.M <= kBM && d.N <= 128) return run<128, 6, EPI_F32>(d, ka, num_sms, st);
-      return run<256, 6, EPI_F32, true>(d, ka, num_sms, st);
+      if (d.M <= kBM && d.N <= 128) return run<128, 6, EPI_F32>(d, d2, ka, num_sms, st);
+      return run<256, 6, EPI_F32, true>(d, d2, ka, num_sms, st);
     default:
       return cudaErrorInvalidValue;
   }
 }
+
+}  // namespace
 
 }  // namespace mapk

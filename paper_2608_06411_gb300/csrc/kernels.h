@@ -101,12 +101,18 @@ struct GemmDesc {
   GemmProducts pr{};
   // EPI_GELU_SPLIT, N % 256 == 0: columns of a tile, 64, 128, 192 or 256 (0)
   int tile_n = 0;
+  // EPI_GELU_SPLIT, EPI_ROPE_SPLIT3: the rows are segments of seg_len rows, of which the first
+  // seg_valid[s] (device) hold data; tiles without such rows are skipped (nullptr: all rows)
+  const int* seg_valid = nullptr; int seg_len = 0;
 };
 
-// tile_n of the first layers of the visual and question branches (m_vis and m_text rows, N columns).
-void predictor_tile_widths(int m_vis, int m_text, int N, int K, int num_sms, int* w_vis, int* w_text);
+// tile_n of the first layer of both branches (m_vis and m_text rows, N columns).
+int predictor_tile_width(long long m_vis, long long m_text, int N, int K, int num_sms);
 // Returns cudaSuccess, or an error for an unsupported shape (cudaErrorInvalidValue).
 cudaError_t launch_gemm(const GemmDesc& d, int num_sms, cudaStream_t st);
+// Both in one launch: two row groups that share N, K, the epilogue and its table (EPI_GELU_SPLIT,
+// EPI_ROPE_SPLIT3).
+cudaError_t launch_gemm_groups(const GemmDesc& d, const GemmDesc& d2, int num_sms, cudaStream_t st);
 
 // Folds a projection after a linear layer into one matrix: W = Wp W2 ([dp, Dh] = [dp, Dh] x
 // [Dh, Dh]) and bias = Wp b2, accumulated in fp64 from the bf16 inputs.  W is stored as the

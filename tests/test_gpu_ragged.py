@@ -120,3 +120,31 @@ def test_ragged_qwen_config_sampled(K):
     out = ctx.gather(dev_bits(vis), torch.from_numpy(keep).to(DEV))
     torch.cuda.synchronize()
     np.testing.assert_array_equal(out.cpu().numpy().view(np.uint16), O.gather(vis, keep))
+
+
+@pytest.mark.parametrize("N,nv", [(100, [100, 1, 37, 99, 2]), (300, [300, 129, 1, 256, 257, 44]),
+                                  (512, [1, 2, 512, 255]), (640, [640] * 3 + [33] * 5)])
+def test_ragged_scores_equal_each_image_alone(N, nv):
+    """Row tiles without a valid row are skipped: tiles inside one image, across two or more (N below a
+    tile's 256 rows), the last tile of the batch, images of one token.  Every image's scores are those
+    of its valid tokens alone (the same sums; only empty slabs of the softmax statistics are added),
+    and the padding's are zero, with unrelated values and NaN bit patterns in the padded rows."""
+    dims = W.PredictorDims(D=512, Dh=512, dp=128)
+    wts = W.make_weights(dims, seed=5, bias_std=0.1)
+    ctx = mb.Context({k: dev_bits(v) for k, v in wts.items()}, dims.D, dims.Dh, dims.dp)
+    wl, B = W.WORKLOADS["c1"], len(nv)
+    nv = np.array(nv, np.int32)
+    lens = np.arange(2, 2 + 9 * B, 9).astype(np.int32)
+    vis = np.stack([W.make_image(wl, b, N=N, D=dims.D) for b in range(B)])
+    for b in range(B):
+        vis[b, nv[b]:] = 0x7FC0 if b % 2 else 0x4580
+    text = np.concatenate([W.make_text(wl, b, int(lens[b]), D=dims.D) for b in range(B)])
+    got = ctx.score_ragged(dev_bits(text), dev_bits(vis), lens, nv)
+    o = 0
+    for b in range(B):
+        n, m = int(nv[b]), int(lens[b])
+        alone = ctx.score(dev_bits(text[o:o + m]), dev_bits(vis[b:b + 1, :n]), lens[b:b + 1])
+        o += m
+        torch.testing.assert_close(got[b, :n], alone[0], rtol=2e-6, atol=0)
+        assert not got[b, n:].any()
+    ctx.check()
