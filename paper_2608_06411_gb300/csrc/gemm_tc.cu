@@ -246,7 +246,8 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
   float* Lsm = xpose + S::XPOSE / 4;
   float* rinv_sm = Lsm + S::LSM / 4;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // uniform in the warp, and known to be
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
     // tempty: one arrive per epilogue warp (of both CTAs with CG2, on the leader's barrier)
@@ -328,9 +329,11 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
   int last_par[STAGES];
 #pragma unroll
   for (int s = 0; s < STAGES; ++s) last_par[s] = -1;
+  bool drains = false;                            // this thread issued the loads
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---------------------------------------------------------------- TMA producer
+      drains = true;
       uint32_t stage = 0, phase = 0;
       bool ok = true;
       for (int t = unit0; t < total && ok; t += units_step) {
@@ -418,12 +421,13 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && crank == 0) {
+    if (crank == 0 && elect_one()) {
       // ---------------------------------------------------------------- MMA issuer (CG2: leader)
       uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
       bool issued = false, ok = true;
-      // products: descriptors without their address (shared memory addresses are below 2^18), and
+      // descriptors without their address (shared memory addresses are below 2^18); products: also
       // their step per 16 K: 32 bytes along a K-major row, 16 rows of 128 bytes of an MN-major box
+      const uint64_t kdesc0 = desc_sw128(0);
       const bool amn = PRODUCTS && a.pr.a_mn, bmn = PRODUCTS && a.pr.b_mn;
       const uint64_t adesc0 = amn ? desc_sw128_mn(0) : desc_sw128(0), bdesc0 = bmn ? desc_sw128_mn(0) : desc_sw128(0);
       const uint32_t astep = (amn ? 2048 : 32) >> 4, bstep = (bmn ? 2048 : 32) >> 4;
@@ -451,20 +455,19 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
             if constexpr (CG2) umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
             else umma_commit(&empty[stage]);
           } else if constexpr (CG2) {
+            const uint64_t da = kdesc0 + (a0 >> 4), db = kdesc0 + (b0 >> 4);
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k)
-              umma_bf16_cg2(d_tmem, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), IDESC, (kb != kb0 || k != 0));
+            for (int k = 0; k < kBK / 16; ++k) umma_bf16_cg2(d_tmem, da + 2 * k, db + 2 * k, IDESC, (kb != kb0 || k != 0));
             umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
           } else {
+            const uint64_t da = kdesc0 + (a0 >> 4), db = kdesc0 + (b0 >> 4);
 #pragma unroll
-            for (int k = 0; k < kBK / 16; ++k)
-              umma_bf16(d_tmem, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), IDESC, (kb != kb0 || k != 0));
+            for (int k = 0; k < kBK / 16; ++k) umma_bf16(d_tmem, da + 2 * k, db + 2 * k, IDESC, (kb != kb0 || k != 0));
             if constexpr (S::PROJ) {   // A A^T: its diagonal is ||row||^2
               const uint32_t n_tmem = tmem_base + 2 * BN + acc * kBM;
 #pragma unroll
               for (int k = 0; k < kBK / 16; ++k)
-                umma_bf16(n_tmem, desc_sw128(a0 + k * 32), desc_sw128(a0 + k * 32), idesc_bf16(kBM, kBM),
-                          (kb != kb0 || k != 0));
+                umma_bf16(n_tmem, da + 2 * k, da + 2 * k, idesc_bf16(kBM, kBM), (kb != kb0 || k != 0));
             }
             umma_commit(&empty[stage]);
           }
@@ -970,7 +973,7 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
   // may still be in flight that no MMA waited for: let them land before the CTA exits.  With
   // 2-SM pairs both CTAs' loads complete on the leader's barriers, which the leader drains.
   __syncthreads();
-  if (*abort_flag && warp == 0 && lane == 0 && crank == 0) {
+  if (*abort_flag && drains && crank == 0) {
     for (int s = 0; s < STAGES; ++s)
       if (last_par[s] >= 0) mbar_wait(&full[s], static_cast<uint32_t>(last_par[s]), a.status, nullptr);
   }

@@ -42,6 +42,17 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
+// One lane of a converged warp, the same for every call.  Code that issues tcgen05.mma or TMA copies
+// runs under it: the compiler then knows that one thread is active and keeps descriptors and
+// coordinates in uniform registers.  Under `lane == 0` four MMAs and their commit took 557 cycles to
+// issue, more than the 512 a 128 x 256 x 64 step takes to run; under elect.sync, with the descriptors'
+// constant part computed once, 386 (128 x 128) and 514 (128 x 256, the tensor core's time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 // ------------------------------------------------------------------ mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));

@@ -9,7 +9,7 @@
 // whatever the batch).  Per CTA:
 //   all threads   cp.async rows (16 bytes a thread, 128 bytes of a row per 8 threads) into a ring
 //                 of 128-byte-swizzled K-major stages of 64 columns;
-//   thread 0      tcgen05.mma (M = 128, K = 16) per stage into TMEM: columns 0-127 the rows 0-127,
+//   one thread    tcgen05.mma (M = 128, K = 16) per stage into TMEM: columns 0-127 the rows 0-127,
 //                 the next ones the rows 128-255;
 //   all threads   TMEM -> shared memory (the ring's space), cluster barrier, an eighth of the rows
 //                 summed over the ranks and written.
@@ -64,6 +64,7 @@ __device__ __forceinline__ void multiply(const SelState& s, int b, const int (&t
   constexpr int STAGES = BASIS ? 4 : 6, LAG = STAGES - 2;
   constexpr uint32_t STAGE = kActBytes + (BASIS ? kBasBytes : 0);
   const int tid = threadIdx.x, r0 = tid >> 3, c = tid & 7;
+  const bool warp0 = __shfl_sync(0xffffffffu, tid >> 5, 0) == 0;
   const uint16_t* V = static_cast<const uint16_t*>(s.uptr ? s.uptr[1] : s.V) + static_cast<long long>(b) * s.N * s.D + 8 * c;
   const int n = kb1 - kb0;
   volatile int* abort_flag = &sh.abort;
@@ -94,19 +95,20 @@ __device__ __forceinline__ void multiply(const SelState& s, int b, const int (&t
       cp_async_wait_group<LAG>();                    // this thread's copies of K block it - LAG
       fence_proxy_async_smem();                      // visible to the tensor core's reads
       __syncthreads();
-      if (tid == 0 && !*abort_flag) {
+      if (warp0 && elect_one() && !*abort_flag) {
         tc_fence_after();
         const int j = it - LAG, st = j % STAGES;
         const uint32_t a0 = ring + st * STAGE, a1 = a0 + kTileRows * kRowBytes, bb = a0 + kActBytes;
+        const uint64_t d0 = desc_sw128(0) + (a0 >> 4), d1 = desc_sw128(0) + (a1 >> 4), db = desc_sw128(0) + (bb >> 4);
 #pragma unroll
         for (int k = 0; k < kKb / 16; ++k) {
           const uint32_t on = j != 0 || k != 0;
           if (BASIS) {
-            umma_bf16(tmem, desc_sw128(a0 + k * 32), desc_sw128(bb + k * 32), idesc_bf16(128, 128), on);
-            if (two) umma_bf16(tmem + 128, desc_sw128(a1 + k * 32), desc_sw128(bb + k * 32), idesc_bf16(128, 128), on);
+            umma_bf16(tmem, d0 + 2 * k, db + 2 * k, idesc_bf16(128, 128), on);
+            if (two) umma_bf16(tmem + 128, d1 + 2 * k, db + 2 * k, idesc_bf16(128, 128), on);
           } else {
-            umma_bf16(tmem, desc_sw128(a0 + k * 32), desc_sw128(a0 + k * 32), idesc_bf16(128, 128), on);
-            if (two) umma_bf16(tmem + 128, desc_sw128(a1 + k * 32), desc_sw128(a0 + k * 32), idesc_bf16(128, 256), on);
+            umma_bf16(tmem, d0 + 2 * k, d0 + 2 * k, idesc_bf16(128, 128), on);
+            if (two) umma_bf16(tmem + 128, d1 + 2 * k, d0 + 2 * k, idesc_bf16(128, 256), on);
           }
         }
         umma_commit(&sh.empty[st]);
@@ -159,7 +161,7 @@ __global__ void __launch_bounds__(kThreads, 1) sel_gram_kernel(SelState s, int r
   if (unit > 0) multiply<true>(s, b, ta, tb, two, ring, sh, tmem, kb0, kb1, wait_ns);
   else multiply<false>(s, b, ta, tb, two, ring, sh, tmem, kb0, kb1, wait_ns);
   if (kb1 > kb0) {                                   // every MMA has read its stage and written TMEM
-    if (tid == 0) umma_commit(&sh.done);
+    if (warp == 0 && elect_one()) umma_commit(&sh.done);   // by the thread that issued them
     mbar_wait(&sh.done, 0, s.status, nullptr);
     tc_fence_after();
   }
