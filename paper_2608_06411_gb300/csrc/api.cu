@@ -22,6 +22,7 @@ constexpr int kMaxKDiverse = 768;   // k limit when the diversity term is on (th
                                     // stages slot rows and 32 basis rows of k floats in shared memory)
 constexpr int kProjMaxBasis = 128;  // basis vectors one projection pass takes
 constexpr int kMaxK = 4096;
+constexpr int kCombineInTile = 32;  // most 32-row slabs whose softmax statistics every tile combines itself
 constexpr int kMaxN = 16384;
 
 struct DevBuf {
@@ -350,9 +351,17 @@ int score_impl(map_ctx* c, const void* text, const void* vis, const int32_t* len
     d.epi = mapk::EPI_SM_STATS; d.stats = part; d.stat_ld = ld;
     d.C = part; d.ldc = 4; d.c_batch_stride = 0;
     MAP_TRY(gemm(c, d, st));
-    ++c->counters.launches;
-    CU_TRY(mapk::launch_stats_combine(part, B, nparts, ld, d_len, fin, st));
-    d.epi = mapk::EPI_SM_MEAN; d.stats = fin;
+    d.epi = mapk::EPI_SM_MEAN;
+    if (nparts <= kCombineInTile && static_cast<long long>(B) * m_tiles * n_tiles <= c->num_sms) {
+      // one tile a CTA and few slabs: each tile combines its columns' partial statistics itself while
+      // its MMAs run, a launch less (N = 576: 165 -> 159 us per call, with the selection's merged
+      // set-up launches); with 92 slabs (N = 2880) it took longer than the launch
+      d.stats = part; d.stat_parts = nparts;
+    } else {
+      ++c->counters.launches;
+      CU_TRY(mapk::launch_stats_combine(part, B, nparts, ld, d_len, fin, st));
+      d.stats = fin;
+    }
     d.C = mean_out; d.ldc = 4; d.c_batch_stride = static_cast<long long>(N) * n_tiles;
     MAP_TRY(gemm(c, d, st));
     if (n_tiles > 1) {
@@ -494,7 +503,7 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
       pd.A = vis; pd.a_rows_total = BN; pd.a_row_stride = N;
       pd.B = s.Vg; pd.b_rows_total = static_cast<long long>(B) * R; pd.b_row_stride = R; pd.b_base = S;
       pd.M = N; pd.N = kProjMaxBasis; pd.K = g.D; pd.batch = B; pd.n_limit = s.proj_lim;
-      pd.blist = s.blist;                         // images to project (built by proj_prep)
+      pd.blist = s.blist;                         // images to project (built by the gather)
       pd.m_limit = s.nvalid;
       pd.C = nullptr; pd.ldc = 0; pd.c_batch_stride = 0;
       pd.epi = mapk::EPI_PROJECT; pd.status = c->status;
@@ -503,13 +512,10 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
       pd.proj.lambda = g.lambda; pd.proj.tau = g.tau;
       pd.proj.r2 = s.r2; pd.proj.U = s.U; pd.proj.sqn = static_cast<float*>(c->sqn.p); pd.proj.cstep = s.cstep;
       auto project_all = [&](bool first) -> int {
-        c->counters.launches += 3;
-        CU_TRY(mapk::launch_sel_proj_prep(s, first, st));
-        CU_TRY(mapk::launch_sel_gather(s, st));
+        ++c->counters.launches;
+        CU_TRY(mapk::launch_sel_gather(s, first, st));
         take_list(pd);
-        MAP_TRY(gemm(c, pd, st));
-        CU_TRY(mapk::launch_sel_proj_done(s, st));
-        return MAP_OK;
+        return gemm(c, pd, st);
       };
       pd.N = K0c <= 96 ? 96 : kProjMaxBasis;   // basis columns the R0 projection needs
       MAP_TRY(project_all(true));

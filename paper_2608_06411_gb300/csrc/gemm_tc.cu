@@ -54,7 +54,7 @@ struct KArgs {
   const float2* rope; int rope_half; int rope_ld;
   int* status;
   const int* b_off;
-  float2* stats; int stat_ld;
+  float2* stats; int stat_ld; int stat_parts;
   const int* col_count;
   int b_base;
   ProjArgs proj;
@@ -85,9 +85,10 @@ struct Smem {
   static constexpr uint32_t B_BYTES = (CG2 ? BN / 2 : BN) * kBK * 2;   // CG2: this CTA's half
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr uint32_t TILES = STAGES * STAGE_BYTES;
-  static constexpr uint32_t BARS = (2 * STAGES + 5 + (PROJ ? 1 : 0)) * 8;
-  // per-warp 32x32 transposes (EPI_SM_STATS) or 32 column normalisers (EPI_SM_MEAN)
-  static constexpr uint32_t XPOSE = EPI == EPI_SM_STATS ? 4 * 32 * 33 * 4 : (EPI == EPI_SM_MEAN ? 4 * 32 * 4 : 0);
+  static constexpr bool EGSYNC = PROJ || EPI == EPI_SM_MEAN;   // epilogue warps' group barrier
+  static constexpr uint32_t BARS = (2 * STAGES + 5 + (EGSYNC ? 1 : 0)) * 8;
+  // per-warp 32x32 transposes (EPI_SM_STATS) or the tile's column normalisers (EPI_SM_MEAN)
+  static constexpr uint32_t XPOSE = EPI == EPI_SM_STATS ? 4 * 32 * 33 * 4 : (EPI == EPI_SM_MEAN ? BN * 4 : 0);
   // bf16 outputs written by TMA box stores from per-warp staging: hi/lo split epilogues use two
   // buffers of (hi, lo) 32x32 boxes, EPI_ROPE_SPLIT3 (BN = 128) one buffer of (hi, lo) x 2 halves
   static constexpr bool TSTORE_ROPE = EPI == EPI_ROPE_SPLIT3 && BN == 128;
@@ -239,9 +240,9 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
   uint64_t* tfull = empty + STAGES;
   uint64_t* tempty = tfull + 2;
   uint64_t* drain = tempty + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1 + (S::PROJ ? 1 : 0));
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1 + (S::EGSYNC ? 1 : 0));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  uint64_t* egsync = drain + 1;                  // EPI_PROJECT: epilogue warps' group barrier
+  uint64_t* egsync = drain + 1;                  // EGSYNC: epilogue warps' group barrier
   float* xpose = reinterpret_cast<float*>(smem + S::TILES + S::STG + S::BARS + 16);
   float* Lsm = xpose + S::XPOSE / 4;
   float* rinv_sm = Lsm + S::LSM / 4;
@@ -253,7 +254,7 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
     // tempty: one arrive per epilogue warp (of both CTAs with CG2, on the leader's barrier)
     for (int i = 0; i < 2; ++i) { mbar_init(&tfull[i], 1); mbar_init(&tempty[i], CG2 ? 8 : 4); }
     mbar_init(drain, 1);
-    if constexpr (S::PROJ) {
+    if constexpr (S::EGSYNC) {
       mbar_init(egsync, 128);
     }
     *abort_flag = 0;
@@ -529,6 +530,50 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
           staged_b = c.b;
         }
       }
+      if constexpr (EPI == EPI_SM_MEAN) {
+        // the tile's column normalisers c = max + ln(sum), +inf past the image's columns (exp(-inf) =
+        // 0): read, or, when stat_parts is given, combined here from the slabs' partial (max, sum) while the
+        // MMAs run, in stats_combine_kernel's order (eight interleaved sums, then their sum)
+        mbar_arrive(egsync);                       // the previous tile's are no longer read
+        if (!mbar_wait(egsync, eg_phase, a.status, abort_flag, a.wait_ns)) { eg_ok = false; break; }
+        eg_phase ^= 1;
+        const int ncols = min(a.n_limit ? min(a.N, __ldg(a.n_limit + c.b)) : a.N,
+                              a.col_count ? __ldg(a.col_count + c.b) : a.N);
+        for (int j = threadIdx.x - 64; j < BN; j += 128) {
+          const int col = c.n_blk * BN + j;
+          float v = INFINITY;
+          if (col < ncols) {
+            if (a.stat_parts > 0) {
+              const float2* p = a.stats + static_cast<long long>(c.b) * a.stat_parts * a.stat_ld + col;
+              float m = -INFINITY;
+#pragma unroll 8
+              for (int i = 0; i < a.stat_parts; ++i) m = fmaxf(m, p[static_cast<long long>(i) * a.stat_ld].x);
+              float s8[8];
+#pragma unroll
+              for (int y = 0; y < 8; ++y) s8[y] = 0.f;
+              for (int i0 = 0; i0 < a.stat_parts; i0 += 8) {
+                float2 w[8];
+#pragma unroll
+                for (int y = 0; y < 8; ++y)
+                  w[y] = i0 + y < a.stat_parts ? p[static_cast<long long>(i0 + y) * a.stat_ld] : make_float2(0.f, 0.f);
+#pragma unroll
+                for (int y = 0; y < 8; ++y)
+                  if (w[y].y > 0.f) s8[y] += w[y].y * expf(w[y].x - m);
+              }
+              float s = s8[0];
+#pragma unroll
+              for (int y = 1; y < 8; ++y) s += s8[y];
+              v = m + logf(s);
+            } else {
+              v = __ldg(a.stats + static_cast<long long>(c.b) * a.stat_ld + col).x;
+            }
+          }
+          xpose[j] = v;
+        }
+        mbar_arrive(egsync);
+        if (!mbar_wait(egsync, eg_phase, a.status, abort_flag, a.wait_ns)) { eg_ok = false; break; }
+        eg_phase ^= 1;
+      }
       const int row = c.m_blk * kBM + r_in_tile;
       const RowGroup& q = a.grp[GROUPED ? c.grp : 0];
       const bool row_ok = row < (a.m_limit ? min(q.M, __ldg(a.m_limit + c.b)) : q.M);
@@ -737,22 +782,15 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
           if (cbase + lane < ncol) part[cbase + lane] = make_float2(m, sum);
         }
       } else if constexpr (EPI == EPI_SM_MEAN) {
-        // p_hat[row] = (1/M_b) sum_col exp(l - c_col), c_col = max_col + ln(sum_col): each chunk's
-        // 32 column normalisers are loaded once (lane j: column j) into this warp's shared row
-        // and read back as broadcasts
+        // p_hat[row] = (1/M_b) sum_col exp(l - c_col), the c_col read as broadcasts
         const int ncol = a.col_count ? min(lim, __ldg(a.col_count + c.b)) : lim;
-        const float2* fin = a.stats + static_cast<long long>(c.b) * a.stat_ld;
-        float* cn = xpose + (warp - 2) * 32;
         float acc_p = 0.f;
 #pragma unroll 1
         for (int ch = 0; ch < BN / 32; ++ch) {
           uint32_t r[32];
           tmem_ld32(tbase + ch * 32, r);
-          const int cbase = col0 + ch * 32;
-          if (cbase >= ncol) continue;                    // uniform in the warp
-          __syncwarp();                                   // the previous chunk's reads are done
-          cn[lane] = cbase + lane < ncol ? __ldg(fin + cbase + lane).x : INFINITY;   // exp(-inf) = 0
-          __syncwarp();
+          if (col0 + ch * 32 >= ncol) continue;           // uniform in the warp
+          const float* cn = xpose + ch * 32;
 #pragma unroll
           for (int j = 0; j < 32; ++j) acc_p += __expf(__uint_as_float(r[j]) - cn[j]);
         }
@@ -1192,7 +1230,7 @@ cudaError_t launch_checked(const GemmDesc& d, const GemmDesc* d2, int num_sms, c
   ka.rope = d.rope; ka.rope_half = d.rope_half; ka.rope_ld = d.rope_ld;
   ka.status = d.status;
   ka.b_off = d.b_off;
-  ka.stats = d.stats; ka.stat_ld = d.stat_ld; ka.col_count = d.col_count;
+  ka.stats = d.stats; ka.stat_ld = d.stat_ld; ka.stat_parts = d.stat_parts; ka.col_count = d.col_count;
   ka.b_base = d.b_base; ka.proj = d.proj;
   ka.a_kwrap = d.a_kwrap; ka.split3 = d.split3;
   ka.blist = d.blist; ka.bcount = d.blist ? d.bcount : nullptr;

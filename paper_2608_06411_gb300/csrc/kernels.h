@@ -72,8 +72,9 @@ struct GemmDesc {
   const int* b_off = nullptr;
   // EPI_SM_STATS: partial (max, sum) per 32-row slab [batch][m_tiles * 4][stat_ld] (float2)
   // EPI_SM_MEAN:  final (max + ln sum, 1/sum) per column [batch][stat_ld]; output C = scores
-  //               [batch][M] when one column tile covers all columns
-  float2* stats = nullptr; int stat_ld = 0;
+  //               [batch][M] when one column tile covers all columns; with stat_parts > 0, stats is the
+  //               partial array of that many slabs instead, combined by every tile for its columns
+  float2* stats = nullptr; int stat_ld = 0; int stat_parts = 0;
   const int* col_count = nullptr;       // per-batch number of valid columns (M_b)
   // B rows at b * b_row_stride + b_base
   int b_base = 0;

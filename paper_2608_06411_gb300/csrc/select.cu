@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(1024) sel_init_kernel(SelState s) {
   }
   if (threadIdx.x == 0) {
     s.npicks[b] = 0; s.nbasis[b] = 0; s.done[b] = 0; s.gbase[b] = 0;
+    if (s.proj_lim) s.proj_lim[b] = 0;
     cnt = 0;
   }
   __syncthreads();
@@ -293,18 +294,31 @@ __global__ void __launch_bounds__(1024) sel_choose_kernel(SelState s) {
   if (threadIdx.x == 0) {
     s.mode[b] = mode;
     s.theta[b] = theta;
+    // a projection since the last choose: later Gram blocks start past the coordinates it gave
+    if (s.proj_lim && s.proj_lim[b] > 0) {
+      s.gbase[b] = min(s.nbasis[b], kReprojMax);
+      s.proj_lim[b] = 0;
+    }
   }
 }
 
-// Copies the basis rows of the images to project into Vg: row S + beta <- basis token beta.
-// kGatherCtas CTAs per image, each walking every kGatherCtas-th row; other images exit.
+// Sets up a projection: which images to project (first: all; otherwise those still selecting whose
+// basis has grown and has at most kReprojMax vectors), their list for the projection GEMM, and the
+// rows of their basis in Vg: row S + beta <- basis token beta.  kGatherCtas CTAs per image, each
+// walking every kGatherCtas-th row.  proj_lim is read back by the next choose.
 constexpr int kGatherCtas = 64;
 constexpr int kGatherThreads = 128;
 
-__global__ void __launch_bounds__(kGatherThreads) sel_gather_kernel(SelState s) {
+__global__ void __launch_bounds__(kGatherThreads) sel_gather_kernel(SelState s, int first) {
   pdl_enter();
   const int b = blockIdx.y;
-  if (s.proj_lim[b] == 0) return;
+  const bool go = first || (!s.done[b] && s.nbasis[b] > s.gbase[b] && s.nbasis[b] <= kReprojMax);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (b == 0) s.bcount[s.bc_par ^ 1] = 0;
+    s.proj_lim[b] = go ? kReprojMax : 0;
+    if (go) s.blist[atomicAdd(s.bcount + s.bc_par, 1)] = b;
+  }
+  if (!go) return;
   const int nb = min(s.nbasis[b], kReprojMax);
   const int vec = s.D / 8;
   for (int r = blockIdx.x; r < nb; r += kGatherCtas) {
@@ -622,8 +636,9 @@ __global__ void __launch_bounds__(kCholThreads, 1) sel_chol_kernel(SelState s) {
       const float floor2 = s.tau * dg[c0 + lane];
       float mydiag = 0.f;
       bool myext = false;
+      const int cols = min(32, K0 - c0);               // the last panel's other columns are empty
 #pragma unroll 1
-      for (int t0 = 0; t0 < 32; t0 += 8) {
+      for (int t0 = 0; t0 < cols; t0 += 8) {
         float ev[8];
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
@@ -1058,33 +1073,6 @@ __global__ void __launch_bounds__(kActiveSlots, 1) sel_greedy_kernel(SelState s)
   }
 }
 
-// ------------------------------------------------------------------ projection set-up
-// Which images to project: all (first), or those still selecting whose basis has grown and has at
-// most kReprojMax vectors; their list for the projection.
-__global__ void sel_proj_prep_kernel(SelState s, int first) {
-  pdl_enter();
-  const int b = blockIdx.x;
-  const int nb = s.nbasis[b];
-  const bool go = first || (!s.done[b] && nb > s.gbase[b] && nb <= kReprojMax);
-  if (s.blist && b == 0 && threadIdx.x == 0) s.bcount[s.bc_par ^ 1] = 0;
-  if (!go) {
-    if (threadIdx.x == 0) s.proj_lim[b] = 0;
-    return;
-  }
-  if (threadIdx.x == 0) {
-    if (s.blist) s.blist[atomicAdd(s.bcount + s.bc_par, 1)] = b;
-    s.proj_lim[b] = kReprojMax;
-  }
-}
-
-__global__ void sel_proj_done_kernel(SelState s) {
-  pdl_enter();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < s.B && s.proj_lim[b] > 0) {
-    s.gbase[b] = min(s.nbasis[b], kReprojMax);         // coordinates the projection gave
-  }
-}
-
 // ------------------------------------------------------------------ outputs
 // keep = picks sorted ascending; pick_order = picks.
 __global__ void sel_finalize_kernel(const int32_t* picks, int K, int32_t* keep, int32_t* order) {
@@ -1218,16 +1206,8 @@ cudaError_t launch_sel_copy_r0(const int32_t* r0, int B, int K, int32_t* picks, 
   return launch_k(sel_copy_r0_kernel, dim3(B), dim3(256), 0, st, r0, K, picks);
 }
 
-cudaError_t launch_sel_proj_prep(const SelState& s, bool first, cudaStream_t st) {
-  return launch_k(sel_proj_prep_kernel, dim3(s.B), dim3(32), 0, st, s, first ? 1 : 0);
-}
-
-cudaError_t launch_sel_gather(const SelState& s, cudaStream_t st) {
-  return launch_k(sel_gather_kernel, dim3(kGatherCtas, s.B), dim3(kGatherThreads), 0, st, s);
-}
-
-cudaError_t launch_sel_proj_done(const SelState& s, cudaStream_t st) {
-  return launch_k(sel_proj_done_kernel, dim3((s.B + 127) / 128), dim3(128), 0, st, s);
+cudaError_t launch_sel_gather(const SelState& s, bool first, cudaStream_t st) {
+  return launch_k(sel_gather_kernel, dim3(kGatherCtas, s.B), dim3(kGatherThreads), 0, st, s, first ? 1 : 0);
 }
 
 cudaError_t launch_sel_identity(int B, int N, int32_t* keep, int32_t* order, cudaStream_t st) {
@@ -1269,7 +1249,7 @@ std::vector<long long> loop_key(const SelState& s, long long wait_ns, int cap_it
                                 const long long* iters_total) {
   return {s.B, s.N, s.D, s.K, s.K0, s.S, s.R, s.KP, fbits(s.lambda), fbits(s.tau), pbits(s.sqn), pbits(s.U),
           pbits(s.r2), pbits(s.cstep), pbits(s.state), pbits(s.Ec), pbits(s.picks), pbits(s.r0), pbits(s.basis_tok),
-          pbits(s.rnorm), pbits(s.npicks), pbits(s.nbasis), pbits(s.done), pbits(s.mode), pbits(s.gbase),
+          pbits(s.rnorm), pbits(s.npicks), pbits(s.nbasis), pbits(s.done), pbits(s.mode), pbits(s.gbase), pbits(s.proj_lim),
           pbits(s.theta), pbits(s.aslot), pbits(s.G), pbits(s.done_count), pbits(s.status), pbits(s.nvalid),
           pbits(s.uptr), wait_ns, cap_iters, pbits(iters), pbits(iters_total)};
 }

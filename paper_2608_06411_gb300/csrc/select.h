@@ -34,9 +34,9 @@ struct SelState {
   void* Vg;                       // [B, R, D] bf16 rows of the basis to project on, at S + beta
   float* G;                       // [B, S, R] Gram block: A x A at and below the diagonal, A x basis from S on
   int32_t* done_count;            // images finished
-  int32_t* proj_lim;              // [B] basis columns the projection GEMM computes (0: image skipped)
-  // Images the next projection GEMM processes: blist[0 .. bcount[bc_par]).  Its preparation appends
-  // through bcount[bc_par] and zeroes bcount[bc_par ^ 1] for the next one, so no separate reset
+  int32_t* proj_lim;              // [B] basis columns the projection GEMM computes (0: image skipped); nullptr: none
+  // Images the next projection GEMM processes: blist[0 .. bcount[bc_par]).  The gather before it
+  // appends through bcount[bc_par] and zeroes bcount[bc_par ^ 1] for the next one, so no separate reset
   // precedes it; the host flips bc_par after each projection.
   int32_t* blist; int32_t* bcount; int bc_par;
   int* status;
@@ -71,13 +71,10 @@ cudaError_t launch_sel_copy_r0(const int32_t* r0, int B, int K, int32_t* picks, 
 cudaError_t launch_sel_identity(int B, int N, int32_t* keep, int32_t* order, cudaStream_t st);
 // Ahead of a projection of every candidate on the basis (its first kReprojMax vectors): first =
 // the R0 basis of every image; otherwise (after a greedy round) the basis of each image still
-// selecting whose basis has grown and has at most kReprojMax vectors, other images are skipped
-// (proj_lim 0).  The gather copies the basis rows into Vg (rows S + beta).
+// selecting whose basis has grown and has at most kReprojMax vectors, other images are skipped.
+// Copies the basis rows into Vg (rows S + beta).  The next choose moves gbase past the projected vectors.
 constexpr int kReprojMax = 128;
-cudaError_t launch_sel_proj_prep(const SelState& s, bool first, cudaStream_t st);
-cudaError_t launch_sel_gather(const SelState& s, cudaStream_t st);
-// After a projection: the projected images' later Gram blocks start past their basis.
-cudaError_t launch_sel_proj_done(const SelState& s, cudaStream_t st);
+cudaError_t launch_sel_gather(const SelState& s, bool first, cudaStream_t st);
 
 // ------------------------------------------------------------------ device-side round loop
 // The selection rounds after the first ones run as a CUDA graph: a kernel node that tests

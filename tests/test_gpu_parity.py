@@ -424,11 +424,12 @@ def test_retention_sweep_config(K, lam, k0_frac):
                      label=f"c2 N=2880 k={K} lambda={lam} K0={O.resolve_k0(K, k0_frac)}")
 
 
-@pytest.mark.parametrize("N,B", [(100, 9), (576, 12), (1731, 5)])
+@pytest.mark.parametrize("N,B", [(100, 9), (576, 12), (1731, 5), (576, 40)])
 def test_scores_of_a_batch_equal_its_images_alone(N, B):
     """The first layer's tiles are narrower when there are few rows (64, 128, 192 or 256 columns, by
-    the number of tiles), which must not change a bit of any sum: an image scored alone gets the
-    scores it gets in a batch."""
+    the number of tiles), and with few tiles and slabs Eq. 3's second pass combines the softmax statistics
+    itself; neither may change a bit of any sum: an image scored alone gets the scores it gets in a
+    batch."""
     dims = W.PredictorDims(D=1024, Dh=1024, dp=128)
     wl = W.WORKLOADS["c0"]
     wts = W.make_weights(dims, seed=21, bias_std=0.1)
