@@ -364,15 +364,17 @@ __host__ __device__ inline int coord_pitch(int KP) { return ((KP + 7) / 8) * 8 +
 // without the division's chain in every step), while the other warps copy the next chunk's L rows,
 // triangle, Gram entries and basis norms into shared memory (cp.async), so that no chunk waits for
 // a global load.  Writes Ec, r2 and cstep = nb.
-// 200 vectors 49 us -> 20 us, 600 vectors (19 chunks) about 180 -> 103 us with 32 slots and four
-// warps a CTA before; 8 slots a CTA were slower in a batch (16 images: the L rows are copied
-// twice as often).
+// k = 640 of 2880, 2 images, a round at 560 vectors: 90 us with the triangle's 32 steps unrolled and
+// branching per slot, 82 us like this.  32 slots and four warps a CTA took about twice that; 8 slots a
+// CTA were slower in a batch (the L rows are copied twice as often), and a second buffer of L rows did
+// not help.
 constexpr int kUpdWarps = 8;
 
 __global__ void __launch_bounds__(32 * kUpdWarps) sel_update_kernel(SelState s) {
   pdl_enter();
   extern __shared__ __align__(16) float shu[];           // [kUpdSlots][P] slot rows, then [32][P] L rows
-  __shared__ float Lt[2][kChunk][kChunk + 1];            // a chunk's triangle L[i][b0 + q], q < i
+  // a chunk's triangle by columns, LT[q][i] = L[b0 + i][b0 + q], q < i; zeros past column 31
+  __shared__ __align__(16) float LT[2][kChunk][kChunk + 24];
   __shared__ float gsm[2][kUpdSlots][kChunk + 1];        // its Gram entries G[slot][b0 + i]
   __shared__ float rn[2][kChunk];                        // its basis norms
   __shared__ float part[kUpdWarps][kUpdSlots][kChunk + 1];
@@ -407,7 +409,7 @@ __global__ void __launch_bounds__(32 * kUpdWarps) sel_update_kernel(SelState s) 
     }
     for (int e = t0; e < nch * kChunk; e += stride) {   // the triangle: row i, columns c .. c + i - 1
       const int i = e / kChunk, q = e - i * kChunk;
-      if (q < i) cp_async4(&Lt[buf][i][q], s.Ec + (base + __ldg(btok_g + c + i)) * KP + c + q);
+      if (q < i) cp_async4(&LT[buf][q][i], s.Ec + (base + __ldg(btok_g + c + i)) * KP + c + q);
     }
     for (int e = t0; e < kUpdSlots * nch; e += stride) {   // Gram entries of the slots that need them
       const int sl = e / nch, i = e - sl * nch;
@@ -423,6 +425,7 @@ __global__ void __launch_bounds__(32 * kUpdWarps) sel_update_kernel(SelState s) 
     float* me = shu + r * P;
     for (int q = 4 * lane; q < c0; q += 128) cp_async16(me + q, g + q);
   }
+  for (int i = threadIdx.x; i < 2 * kChunk * 24; i += 32 * kUpdWarps) LT[i / (24 * kChunk)][i / 24 % kChunk][kChunk + i % 24] = 0.f;
   const int first = (cmin / kChunk) * kChunk;
   stage(first, 0, threadIdx.x, blockDim.x);
   const int mtok = lane < kUpdSlots ? tok_s[lane] : -1, mc0 = lane < kUpdSlots ? c0_s[lane] : nb;   // warp 0: this lane's slot
@@ -476,30 +479,44 @@ __global__ void __launch_bounds__(32 * kUpdWarps) sel_update_kernel(SelState s) 
     if (warp != 0) {
       if (b0 + kChunk < nb) stage(b0 + kChunk, buf ^ 1, threadIdx.x - 32, blockDim.x - 32);
     } else {
-      const float my_rn = lane < nch ? rn[buf][lane] : 1.f, my_inv = 1.0f / my_rn;
-      float* me = shu + lane * P;
+      // eight basis vectors per pass, then the row shifts down by eight: the code stays small, and
+      // without branches (a slot without a token, a cached coordinate, a vector past nb are selects)
+      const float my_rn = lane < nch ? rn[buf][lane] : 1.f, my_inv = lane < nch ? 1.0f / my_rn : 0.f;
+      const bool act = mtok >= 0;
+      float* me = shu + (lane & (kUpdSlots - 1)) * P + b0;
       float av[kChunk];
 #pragma unroll
-      for (int i = 0; i < kChunk; ++i) av[i] = mtok >= 0 && i < nch && b0 + i >= mc0 ? part[0][lane][i] : 0.f;
+      for (int i = 0; i < kChunk; ++i) av[i] = part[0][lane & (kUpdSlots - 1)][i];
+#pragma unroll 1
+      for (int t0 = 0; t0 < nch; t0 += 8) {
+        float old[8], ev[8];
 #pragma unroll
-      for (int i = 0; i < kChunk; ++i) {
-        const float ri = __shfl_sync(0xffffffffu, my_inv, i), rr = __shfl_sync(0xffffffffu, my_rn, i);
-        if (i < nch) {                               // uniform
-          const int beta = b0 + i;
-          float ei = 0.f;
-          if (mtok >= 0) {
-            if (beta >= mc0) {
-              ei = av[i] * ri;
-              ei = fmaf(fmaf(-ei, rr, av[i]), ri, ei);
-              me[beta] = ei;
-              r2 = fmaf(-ei, ei, r2);
-            } else {
-              ei = me[beta];
-            }
+        for (int u = 0; u < 8; ++u) old[u] = t0 + u < nch ? me[t0 + u] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float ri = __shfl_sync(0xffffffffu, my_inv, t0 + u), rr = __shfl_sync(0xffffffffu, my_rn, t0 + u);
+          const bool fresh = b0 + t0 + u >= mc0 && t0 + u < nch;   // past nb: e = 0
+          float e = av[u] * ri;
+          e = fmaf(fmaf(-e, rr, av[u]), ri, e);
+          e = fresh ? e : old[u];
+          r2 = fresh ? fmaf(-e, e, r2) : r2;
+          ev[u] = e;
+#pragma unroll
+          for (int j = (u + 1) & ~3; j < kChunk; j += 4) {
+            const float4 l = *reinterpret_cast<const float4*>(&LT[buf][t0 + u][t0 + j]);
+            if (j > u) av[j] = fmaf(-e, l.x, av[j]);
+            if (j + 1 > u) av[j + 1] = fmaf(-e, l.y, av[j + 1]);
+            if (j + 2 > u) av[j + 2] = fmaf(-e, l.z, av[j + 2]);
+            if (j + 3 > u) av[j + 3] = fmaf(-e, l.w, av[j + 3]);
           }
-#pragma unroll
-          for (int j = i + 1; j < kChunk; ++j) av[j] = fmaf(-Lt[buf][j][i], ei, av[j]);
         }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (act && t0 + u < nch) me[t0 + u] = ev[u];
+#pragma unroll
+        for (int j = 0; j < 24; ++j) av[j] = av[j + 8];
+#pragma unroll
+        for (int j = 24; j < 32; ++j) av[j] = 0.f;
       }
     }
     __syncthreads();                                 // this chunk's coordinates are written
