@@ -939,7 +939,7 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
     long long T; const void* X; int i1, ip; cudaStream_t st;
     const int32_t* pos; int pos_mod;
     const void* xa;                                  // the features, 16-byte aligned
-    float *z1, *raw, *pre, *part, *ws;
+    float *g1, *raw, *pre, *part, *ws;               // g1: GELU'(z1)
     uint16_t *h1, *h2, *dpre, *dh2, *dh1;
     long long ws_floats;
   };
@@ -975,7 +975,7 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
       used += (static_cast<size_t>(n) * sizeof(T) + 255) / 256 * 256;
     };
     for (Branch& x : br) {
-      take(x.z1, x.T * Dh); take(x.raw, x.T * Dh); take(x.pre, x.T * dp);
+      take(x.g1, x.T * Dh); take(x.raw, x.T * Dh); take(x.pre, x.T * dp);
       take(x.part, (x.T + 63) / 64 * Dh); take(x.ws, x.ws_floats);
       take(x.h1, x.T * 3 * Dh); take(x.h2, x.T * 3 * Dh); take(x.dh2, x.T * 3 * Dh); take(x.dh1, x.T * 3 * Dh);
       take(x.dpre, x.T * 3 * dp);
@@ -1013,7 +1013,7 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
       CU_TRY(cudaMemcpyAsync(const_cast<void*>(x.xa), x.X, static_cast<size_t>(x.T) * D * 2, cudaMemcpyDeviceToDevice, x.st));
     MAP_TRY(mm(x.T, iDh, D, exact(x.xa, x.T, iD, 0), exact(c->w[x.i1], Dh, iD, 0), TcBatch{}, slices(x.T, iDh, D, 1),
                false, x.raw, Dh, x.ws, x.st, &r));
-    CU_TRY(mapk::launch_act_split(true, r, c->w[x.i1 + 1], x.T, iDh, x.z1, x.h1, x.st));
+    CU_TRY(mapk::launch_act_split(true, r, c->w[x.i1 + 1], x.T, iDh, x.g1, x.h1, x.st));
     MAP_TRY(mm(x.T, iDh, Dh, split(x.h1, x.T, iDh, 0), exact(c->w[x.i1 + 2], Dh, iDh, 0), TcBatch{},
                slices(x.T, iDh, Dh, 3), false, x.raw, Dh, x.ws, x.st, &r));
     CU_TRY(mapk::launch_act_split(false, r, c->w[x.i1 + 3], x.T, iDh, nullptr, x.h2, x.st));
@@ -1038,7 +1038,7 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
                true, gout[x.i1 + 2], Dh, x.ws, x.st, nullptr));                                      // dW2
     MAP_TRY(mm(x.T, iDh, Dh, split(x.dh2, x.T, iDh, 0), exact(c->w[x.i1 + 2], Dh, iDh, 1), TcBatch{},
                slices(x.T, iDh, Dh, 3), false, x.raw, Dh, x.ws, x.st, &r));                          // dh1
-    CU_TRY(mapk::launch_back_split(r, x.z1, x.T, iDh, x.dh1, x.part, gout[x.i1 + 1], x.st));
+    CU_TRY(mapk::launch_back_split(r, x.g1, x.T, iDh, x.dh1, x.part, gout[x.i1 + 1], x.st));
     MAP_TRY(mm(Dh, iD, x.T, split(x.dh1, x.T, iDh, 1), exact(x.xa, x.T, iD, 1), TcBatch{}, slices(Dh, iD, x.T, 3), true,
                gout[x.i1], D, x.ws, x.st, nullptr));                                                 // dW1
     launches += 5;

@@ -75,12 +75,12 @@ __device__ __forceinline__ float2 load_result2(const TcResult& in, long long r, 
   return x;
 }
 
-__device__ __forceinline__ float gelu_f(float x) { return 0.5f * x * (1.0f + erff(x * 0.70710678118654752f)); }
-// d/dx [x Phi(x)] = Phi(x) + x phi(x)
-__device__ __forceinline__ float gelu_grad_f(float x) {
+// x Phi(x) and its derivative Phi(x) + x phi(x)
+__device__ __forceinline__ float gelu_and_grad(float x, float& grad) {
   const float Phi = 0.5f * (1.0f + erff(x * 0.70710678118654752f));
   const float phi = 0.39894228040143268f * expf(-0.5f * x * x);
-  return Phi + x * phi;
+  grad = Phi + x * phi;
+  return x * Phi;
 }
 
 // Elementwise steps and the staging of their result in one pass: a warp reads 128 columns of a row
@@ -89,10 +89,11 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
 constexpr int kColRows = 64;                        // rows of a block, and of a partial column sum
 constexpr int kActWarps = 8;
 
-// x = GELU(z) with z = in + bias kept in fp32 for the backward pass (GELU), or x = in + bias.
+// x = GELU(in + bias), its derivative kept in fp32 for the backward pass (GELU; the error function is
+// evaluated once for both), or x = in + bias.
 template <bool GELU>
 __global__ void __launch_bounds__(32 * kActWarps) act_split_kernel(TcResult in, const __nv_bfloat16* __restrict__ bias,
-                                                                   long long rows, int cols, float* __restrict__ z,
+                                                                   long long rows, int cols, float* __restrict__ grad,
                                                                    uint16_t* __restrict__ dst) {
   pdl_enter();
   const int c = blockIdx.x * 128 + 4 * (threadIdx.x & 31), w = threadIdx.x >> 5;
@@ -107,17 +108,18 @@ __global__ void __launch_bounds__(32 * kActWarps) act_split_kernel(TcResult in, 
     const float4 v = load_result4(in, r, c);
     float x[4] = {v.x + b[0], v.y + b[1], v.z + b[2], v.w + b[3]};
     if (GELU) {
-      *reinterpret_cast<float4*>(z + r * cols + c) = make_float4(x[0], x[1], x[2], x[3]);
+      float g[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) x[u] = gelu_f(x[u]);
+      for (int u = 0; u < 4; ++u) x[u] = gelu_and_grad(x[u], g[u]);
+      *reinterpret_cast<float4*>(grad + r * cols + c) = make_float4(g[0], g[1], g[2], g[3]);
     }
     store_split4(dst + r * 3 * cols + c, cols, x);
   }
 }
 
-// x = in * GELU'(z) (BACK) or in; part[block row][c] = the block's column sums of x.
+// x = in * grad (BACK) or in; part[block row][c] = the block's column sums of x.
 template <bool BACK>
-__global__ void __launch_bounds__(32 * kActWarps) back_split_kernel(TcResult in, const float* __restrict__ z,
+__global__ void __launch_bounds__(32 * kActWarps) back_split_kernel(TcResult in, const float* __restrict__ grad,
                                                                     long long rows, int cols,
                                                                     uint16_t* __restrict__ dst,
                                                                     float* __restrict__ part) {
@@ -133,11 +135,11 @@ __global__ void __launch_bounds__(32 * kActWarps) back_split_kernel(TcResult in,
     const float4 v = load_result4(in, r, c);
     float x[4] = {v.x, v.y, v.z, v.w};
     if (BACK) {
-      const float4 g = *reinterpret_cast<const float4*>(z + r * cols + c);
-      x[0] *= gelu_grad_f(g.x);
-      x[1] *= gelu_grad_f(g.y);
-      x[2] *= gelu_grad_f(g.z);
-      x[3] *= gelu_grad_f(g.w);
+      const float4 g = *reinterpret_cast<const float4*>(grad + r * cols + c);
+      x[0] *= g.x;
+      x[1] *= g.y;
+      x[2] *= g.z;
+      x[3] *= g.w;
     }
     s.x += x[0]; s.y += x[1]; s.z += x[2]; s.w += x[3];
     store_split4(dst + r * 3 * cols + c, cols, x);
@@ -461,23 +463,23 @@ dim3 act_grid(long long rows, int cols) {
 }
 }  // namespace
 
-cudaError_t launch_act_split(bool gelu, const TcResult& in, const void* bias, long long rows, int cols, float* z,
+cudaError_t launch_act_split(bool gelu, const TcResult& in, const void* bias, long long rows, int cols, float* grad,
                              void* dst, cudaStream_t st) {
   if (cols % 128 != 0) return cudaErrorInvalidValue;
   const __nv_bfloat16* b = static_cast<const __nv_bfloat16*>(bias);
   uint16_t* d = static_cast<uint16_t*>(dst);
-  if (gelu) return launch_k(act_split_kernel<true>, act_grid(rows, cols), dim3(32 * kActWarps), 0, st, in, b, rows, cols, z, d);
-  return launch_k(act_split_kernel<false>, act_grid(rows, cols), dim3(32 * kActWarps), 0, st, in, b, rows, cols, z, d);
+  if (gelu) return launch_k(act_split_kernel<true>, act_grid(rows, cols), dim3(32 * kActWarps), 0, st, in, b, rows, cols, grad, d);
+  return launch_k(act_split_kernel<false>, act_grid(rows, cols), dim3(32 * kActWarps), 0, st, in, b, rows, cols, grad, d);
 }
 
-cudaError_t launch_back_split(const TcResult& in, const float* z, long long rows, int cols, void* dst, float* part,
+cudaError_t launch_back_split(const TcResult& in, const float* grad, long long rows, int cols, void* dst, float* part,
                               float* colsum, cudaStream_t st) {
   if (cols % 128 != 0) return cudaErrorInvalidValue;
   uint16_t* d = static_cast<uint16_t*>(dst);
   const dim3 grid = act_grid(rows, cols);
   const cudaError_t e =
-      z ? launch_k(back_split_kernel<true>, grid, dim3(32 * kActWarps), 0, st, in, z, rows, cols, d, part)
-        : launch_k(back_split_kernel<false>, grid, dim3(32 * kActWarps), 0, st, in, z, rows, cols, d, part);
+      grad ? launch_k(back_split_kernel<true>, grid, dim3(32 * kActWarps), 0, st, in, grad, rows, cols, d, part)
+           : launch_k(back_split_kernel<false>, grid, dim3(32 * kActWarps), 0, st, in, grad, rows, cols, d, part);
   if (e != cudaSuccess) return e;
   return launch_k(colsum_final_kernel, dim3((cols + 31) / 32), dim3(256), 0, st, static_cast<const float*>(part),
                   static_cast<int>(grid.y), cols, colsum);

@@ -193,12 +193,12 @@ cudaError_t launch_tc_matmul(int M, int N, int K, const TcOperand& A, const TcOp
 // padded row of every question row, and the image of every padded row (-1: padding).
 cudaError_t launch_distill_meta(const int32_t* len, const int32_t* off, int B, int32_t* poff, int32_t* prow,
                                 int32_t* img, cudaStream_t st);
-// x = GELU(in + bias) (gelu: in + bias goes to z) or in + bias, as three bf16 terms [rows, 3 cols].
-cudaError_t launch_act_split(bool gelu, const TcResult& in, const void* bias, long long rows, int cols, float* z,
+// x = GELU(in + bias) (gelu: GELU'(in + bias) goes to grad) or in + bias, as three bf16 terms [rows, 3 cols].
+cudaError_t launch_act_split(bool gelu, const TcResult& in, const void* bias, long long rows, int cols, float* grad,
                              void* dst, cudaStream_t st);
-// x = in * GELU'(z) (z given) or in, as three bf16 terms, and its column sums (part: kColRows-row
+// x = in * grad (if given) or in, as three bf16 terms, and its column sums (part: kColRows-row
 // partial sums, ceil(rows / 64) * cols floats).
-cudaError_t launch_back_split(const TcResult& in, const float* z, long long rows, int cols, void* dst, float* part,
+cudaError_t launch_back_split(const TcResult& in, const float* grad, long long rows, int cols, void* dst, float* part,
                               float* colsum, cudaStream_t st);
 // RoPE (or its transpose) of in [rows, d] times scale, as three bf16 terms at row in_map / out_map
 // (nullptr: the row itself).  Position pos[r] or r % pos_mod.
