@@ -366,7 +366,7 @@ int score_impl(map_ctx* c, const void* text, const void* vis, const int32_t* len
     MAP_TRY(gemm(c, d, st));
     if (n_tiles > 1) {
       ++c->counters.launches;
-      CU_TRY(mapk::launch_sum_tiles(mean_out, B, N, n_tiles, scores, st));
+      CU_TRY(mapk::launch_sum_tiles(mean_out, B, N, n_tiles, 256, d_len, scores, st));
     }
   }
   return MAP_OK;

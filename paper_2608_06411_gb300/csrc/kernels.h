@@ -138,8 +138,10 @@ cudaError_t launch_flags_to_host(const int32_t* a, const int* b, int32_t* a_host
 // Squared row norms of bf16 rows: out[r] = sum_d x[r, d]^2 (fp32).
 cudaError_t launch_row_sqnorm(const void* x, long long rows, int D, float* out, cudaStream_t st);
 
-// scores[b, n] = sum_t part[b, t, n] over n_tiles column-tile partial means.
-cudaError_t launch_sum_tiles(const float* part, int B, int N, int n_tiles, float* scores, cudaStream_t st);
+// scores[b, n] = sum_t part[b, t, n] over the column tiles (of `cols` question tokens, n_tiles slots an
+// image) that hold image b's lens[b] tokens; the other slots are never written.
+cudaError_t launch_sum_tiles(const float* part, int B, int N, int n_tiles, int cols, const int* lens, float* scores,
+                             cudaStream_t st);
 
 // Combines the per-slab softmax statistics into (max + ln sum, 1/sum) per question token:
 // part [B][nparts][ld] -> fin [B][ld], columns < lens[b].

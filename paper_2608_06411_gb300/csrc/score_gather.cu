@@ -88,14 +88,16 @@ __global__ void __launch_bounds__(32 * kCombY) stats_combine_kernel(const float2
   }
 }
 
-__global__ void sum_tiles_kernel(const float* __restrict__ part, int N, int n_tiles, long long total,
-                                 float* __restrict__ scores) {
+// Column tiles (of `cols` question tokens) past an image's question are not computed, and not added.
+__global__ void sum_tiles_kernel(const float* __restrict__ part, int N, int n_tiles, int cols,
+                                 const int* __restrict__ lens, long long total, float* __restrict__ scores) {
   pdl_enter();
   const long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (i >= total) return;
   const long long b = i / N, n = i - b * N;
+  const int own = min(n_tiles, (lens[b] + cols - 1) / cols);
   float s = 0.f;
-  for (int t = 0; t < n_tiles; ++t) s += part[(b * n_tiles + t) * N + n];
+  for (int t = 0; t < own; ++t) s += part[(b * n_tiles + t) * N + n];
   scores[i] = s;
 }
 
@@ -311,10 +313,11 @@ cudaError_t launch_gather(const void* V, const int32_t* idx, int B, int N, int k
                   static_cast<const uint4*>(V), idx, N, k, D / 8, static_cast<uint4*>(out), status);
 }
 
-cudaError_t launch_sum_tiles(const float* part, int B, int N, int n_tiles, float* scores, cudaStream_t st) {
+cudaError_t launch_sum_tiles(const float* part, int B, int N, int n_tiles, int cols, const int* lens, float* scores,
+                             cudaStream_t st) {
   const long long total = static_cast<long long>(B) * N;
   return launch_k(sum_tiles_kernel, dim3(static_cast<unsigned>((total + 255) / 256)), dim3(256), 0, st, part, N,
-                  n_tiles, total, scores);
+                  n_tiles, cols, lens, total, scores);
 }
 
 }  // namespace mapk
