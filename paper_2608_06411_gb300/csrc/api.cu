@@ -517,9 +517,11 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
         take_list(pd);
         return gemm(c, pd, st);
       };
-      pd.N = K0c <= 96 ? 96 : kProjMaxBasis;   // basis columns the R0 projection needs
+      // basis columns a projection on n vectors computes
+      auto proj_cols = [](int n) { return n <= 32 ? 32 : (n <= 96 ? 96 : kProjMaxBasis); };
+      pd.N = proj_cols(K0c);
       MAP_TRY(project_all(true));
-      pd.N = kProjMaxBasis;
+      pd.N = proj_cols(K);
       // one round (greedy, or the rest of R0 when K0 > K0c), then the images still selecting are
       // projected again on their whole basis (when it has at most kReprojMax vectors): exact
       // values for every candidate make the next active set the true top S

@@ -1327,6 +1327,7 @@ cudaError_t launch_checked(const GemmDesc& d, const GemmDesc* d2, int num_sms, c
       return run<256, 4, EPI_SM_MEAN>(d, d2, ka, num_sms, st);
     case EPI_PROJECT:
       if (d.N > kProjMaxBasis || d.batch < 1) return cudaErrorInvalidValue;
+      if (d.N <= 32) return run<32, 8, EPI_PROJECT>(d, d2, ka, num_sms, st);
       if (d.N <= 96) return run<96, 6, EPI_PROJECT>(d, d2, ka, num_sms, st);
       return run<128, 5, EPI_PROJECT>(d, d2, ka, num_sms, st);
     case EPI_F32:   // the distillation's contractions
