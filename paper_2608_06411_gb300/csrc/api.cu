@@ -522,15 +522,17 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
       pd.N = proj_cols(K0c);
       MAP_TRY(project_all(true));
       pd.N = proj_cols(K);
-      // one round (greedy, or the rest of R0 when K0 > K0c), then the images still selecting are
-      // projected again on their whole basis (when it has at most kReprojMax vectors): exact
-      // values for every candidate make the next active set the true top S
-      c->counters.launches += 5;
+      // One round (greedy, or the rest of R0 when K0 > K0c).  After a projection on the whole of R0's
+      // basis every coordinate is current; then the images still selecting are projected again on
+      // their whole basis (when it has at most kReprojMax vectors): exact values for every candidate
+      // make the next active set the true top S.
+      const bool whole = K0c <= mapk::kReprojMax;
+      c->counters.launches += whole ? 4 : 5;
       CU_TRY(mapk::launch_sel_choose(s, st));
       CU_TRY(mapk::launch_sel_gram(s, S, std::max(0, K0c - mapk::kReprojMax), c->wait_ns, st));
-      CU_TRY(mapk::launch_sel_greedy(s, st));
+      CU_TRY(mapk::launch_sel_greedy(s, !whole, st));
       ++c->counters.select_rounds;
-      MAP_TRY(project_all(false));
+      if (whole) MAP_TRY(project_all(false));
     }
     // The remaining rounds run as a device-side loop (a CUDA graph whose WHILE node repeats a
     // round while an image still selects): the host never waits for them.

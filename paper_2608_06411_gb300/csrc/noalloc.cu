@@ -176,7 +176,7 @@ extern "C" int map_select_noalloc(map_ctx* ctx, const float* scores, const void*
         *v.launches += 5;
         if ((rc = rc_of(mapk::launch_sel_choose(s, st))) != MAP_OK) return rc;
         if ((rc = rc_of(mapk::launch_sel_gram(s, S, K, 0, st))) != MAP_OK) return rc;
-        if ((rc = rc_of(mapk::launch_sel_greedy(s, st))) != MAP_OK) return rc;
+        if ((rc = rc_of(mapk::launch_sel_greedy(s, true, st))) != MAP_OK) return rc;
       }
       rounds += burst;
       *v.rounds += burst;

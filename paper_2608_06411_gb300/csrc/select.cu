@@ -1190,13 +1190,16 @@ cudaError_t launch_sel_choose(const SelState& s, cudaStream_t st) {
   return launch_k(sel_choose_kernel, dim3(s.B), dim3(1024), sm, st, s);
 }
 
-cudaError_t launch_sel_greedy(const SelState& s, cudaStream_t st) {
+cudaError_t launch_sel_greedy(const SelState& s, bool update, cudaStream_t st) {
   if (s.S != kActiveSlots) return cudaErrorInvalidValue;
-  const size_t um = sel_update_smem(s.KP);
-  cudaError_t e = cudaFuncSetAttribute(sel_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(um));
-  if (e != cudaSuccess) return e;
-  e = launch_k(sel_update_kernel, dim3((s.S + kUpdSlots - 1) / kUpdSlots, s.B), dim3(32 * kUpdWarps), um, st, s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if (update) {
+    const size_t um = sel_update_smem(s.KP);
+    e = cudaFuncSetAttribute(sel_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(um));
+    if (e != cudaSuccess) return e;
+    e = launch_k(sel_update_kernel, dim3((s.S + kUpdSlots - 1) / kUpdSlots, s.B), dim3(32 * kUpdWarps), um, st, s);
+    if (e != cudaSuccess) return e;
+  }
   const int T = s.S / kRgTile;
   e = launch_k(sel_resgram_kernel, dim3(T * (T + 1) / 2, s.B), dim3(kRgThreads), 0, st, s);
   if (e != cudaSuccess) return e;
@@ -1308,7 +1311,7 @@ cudaError_t build_loop(SelLoopCache* c, const SelState& s, long long wait_ns, in
   SelState r = s;
   if ((e = launch_sel_choose(r, c->cap)) == cudaSuccess &&
       (e = launch_sel_gram(r, r.S, r.K, wait_ns, c->cap)) == cudaSuccess)
-    e = launch_sel_greedy(r, c->cap);
+    e = launch_sel_greedy(r, true, c->cap);
   if (e == cudaSuccess) e = launch_k(sel_loop_cond_kernel, dim3(1), dim3(32), 0, c->cap, r, h, iters, cap_iters, iters_total);
   pdl_disabled() = false;
   cudaGraph_t captured = nullptr;

@@ -61,9 +61,10 @@ cudaError_t launch_sel_choose(const SelState& s, cudaStream_t st);
 // G of the active rows (the first `rows` slots) against themselves (tiles at and below the diagonal)
 // and against up to `basis` basis tokens from gbase on; wait_ns as in GemmDesc.
 cudaError_t launch_sel_gram(const SelState& s, int rows, int basis, long long wait_ns, cudaStream_t st);
-// sel_update_kernel (coordinates of the active tokens up to the current basis), the residual
-// Gram matrix of the active set on that basis, then the picks.
-cudaError_t launch_sel_greedy(const SelState& s, cudaStream_t st);
+// sel_update_kernel (coordinates of the active tokens up to the current basis; not needed, update =
+// false, right after a projection on the whole basis), the residual Gram matrix of the active set on
+// that basis, then the picks.
+cudaError_t launch_sel_greedy(const SelState& s, bool update, cudaStream_t st);
 // The K0 forced R0 picks from the Gram block G[R0, R0] of a forced round (K0 <= kCholMax, <= S).
 cudaError_t launch_sel_chol(const SelState& s, cudaStream_t st);
 cudaError_t launch_sel_finalize(const int32_t* picks, int B, int K, int32_t* keep, int32_t* order, cudaStream_t st);
