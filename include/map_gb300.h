@@ -316,7 +316,9 @@ int map_get_counters(map_ctx *ctx, map_counters *out);
 #define MAP_K_GATHER      6
 #define MAP_K_NUM         7
 
-/* enable != 0 records a CUDA event pair around every launch of the kernels above. */
+/* enable != 0 records a CUDA event pair around every launch of the kernels above.  Where a call
+ * otherwise runs two of them in one launch (the two modalities' layers, the kept indices' order and
+ * the compaction), it launches them separately while timing is on; the results are the same. */
 int map_set_timing(map_ctx *ctx, int enable);
 /* Synchronises the device; returns the summed event time (ms) and count of kernel `id`
  * since timing was enabled, and resets them. */

@@ -380,8 +380,10 @@ T* carve(char*& p, size_t n) {
 }
 
 // nv as for score_impl: tokens at or past nv[b] are never retained (K <= every nv[b]).
+// gather_out: where to compact the kept rows as well (nullptr: not); *gathered tells whether that was
+// done.
 int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t* nv, int B, int N, int K,
-                int32_t* keep, int32_t* order, cudaStream_t st) {
+                int32_t* keep, int32_t* order, cudaStream_t st, void* gather_out = nullptr, bool* gathered = nullptr) {
   if (!c || !scores || !vis) return MAP_EINVAL;
   if (B < 1 || N < 1 || K < 0 || K > N) return MAP_EINVAL;
   if (nv)
@@ -545,6 +547,12 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
     CU_TRY(mapk::launch_sel_copy_r0(s.r0, B, K, s.picks, st));
   }
   ++c->counters.launches;
+  if (gather_out && !order && !c->timing && K <= mapk::kFinalizeGatherMax && 2 * K <= g.D && B <= 65535 &&
+      aligned16(vis) && aligned16(gather_out)) {
+    CU_TRY(mapk::launch_sel_finalize_gather(s.picks, B, K, vis, N, g.D, keep, gather_out, c->status, st));
+    *gathered = true;
+    return MAP_OK;
+  }
   CU_TRY(mapk::launch_sel_finalize(s.picks, B, K, keep, order, st));
   return MAP_OK;
 }
@@ -823,8 +831,9 @@ int prune_impl(map_ctx* ctx, const void* text_feats, const void* vis_feats, cons
     void* oc = static_cast<char*>(o) + static_cast<size_t>(b0) * k * D * 2;
     const int32_t* nvc = nv ? nv + b0 : nullptr;
     int rc = score_impl(c, tc, vc, lens + b0, nvc, Bc, N, spc, nullptr, nullptr, st);
-    if (rc == MAP_OK) rc = select_impl(c, spc, vc, nvc, Bc, N, k, kpc, nullptr, st);
-    if (rc == MAP_OK) rc = gather_impl(c, vc, kpc, Bc, N, k, oc, st);
+    bool gathered = false;
+    if (rc == MAP_OK) rc = select_impl(c, spc, vc, nvc, Bc, N, k, kpc, nullptr, st, oc, &gathered);
+    if (rc == MAP_OK && !gathered) rc = gather_impl(c, vc, kpc, Bc, N, k, oc, st);
     if (rc != MAP_OK) return finish(rc);
     if (host_io) {
       cudaEvent_t ed = ev();

@@ -68,6 +68,11 @@ cudaError_t launch_sel_greedy(const SelState& s, bool update, cudaStream_t st);
 // The K0 forced R0 picks from the Gram block G[R0, R0] of a forced round (K0 <= kCholMax, <= S).
 cudaError_t launch_sel_chol(const SelState& s, cudaStream_t st);
 cudaError_t launch_sel_finalize(const int32_t* picks, int B, int K, int32_t* keep, int32_t* order, cudaStream_t st);
+// The same without pick_order, and out[b, j] = V[b, keep[b, j]] (B <= 65535).  Taken while the picks that
+// every CTA reads are fewer bytes than the row it copies (K <= D / 2) and at most kFinalizeGatherMax.
+constexpr int kFinalizeGatherMax = 1024;
+cudaError_t launch_sel_finalize_gather(const int32_t* picks, int B, int K, const void* V, int N, int D, int32_t* keep,
+                                       void* out, int* status, cudaStream_t st);
 cudaError_t launch_sel_copy_r0(const int32_t* r0, int B, int K, int32_t* picks, cudaStream_t st);
 cudaError_t launch_sel_identity(int B, int N, int32_t* keep, int32_t* order, cudaStream_t st);
 // Ahead of a projection of every candidate on the basis (its first kReprojMax vectors): first =

@@ -462,3 +462,25 @@ def test_select_gram_blocks_and_r0_factor_edges(D, K, k0_frac):
     keep, order = run_select(ctx, p32, vis, K)
     assert_selection(p32, vis, K, O.resolve_k0(K, k0_frac), keep, order,
                      label=f"N=900 D={D} k={K} K0={O.resolve_k0(K, k0_frac)}")
+
+
+@pytest.mark.parametrize("D,K,lam", [(64, 1, 1.0), (64, 32, 1.0), (64, 33, 1.0), (512, 129, 1.0), (4160, 33, 1.0),
+                                     (4160, 1024, 0.0), (4160, 1025, 0.0)])
+def test_prune_of_device_buffers_equals_its_stages(D, K, lam):
+    """Up to 1024 and D / 2 kept tokens map_prune orders the picks and copies their rows in one launch (128
+    threads a pick, four 16-byte loads each before a loop: rows of 64 and 4160 elements); beyond, in two."""
+    dims = W.PredictorDims(D=D, Dh=256, dp=64)
+    ctx, _ = make_ctx(dims, lam=lam)
+    wl = W.WORKLOADS["c1"]
+    B, N = 2, 1100
+    lens = np.array([5, 9], np.int32)
+    vis = dev_bits(np.stack([W.make_image(wl, b, N=N, D=D) for b in range(B)]))
+    text = dev_bits(np.concatenate([W.make_text(wl, b, int(lens[b]), D=D) for b in range(B)]))
+    out = torch.full((B, K, D), -1, dtype=torch.int16, device=DEV)
+    keep = torch.full((B, K), -1, dtype=torch.int32, device=DEV)
+    ctx.prune(text, vis, lens, K, out, keep)
+    want, _ = ctx.select(ctx.score(text, vis, lens), vis, K)
+    torch.cuda.synchronize()
+    ctx.check()
+    assert torch.equal(keep, want)
+    assert torch.equal(out, torch.gather(vis, 1, want.long()[:, :, None].expand(-1, -1, D)))
