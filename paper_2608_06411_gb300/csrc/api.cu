@@ -913,7 +913,7 @@ int map_distill_grad(map_ctx* ctx, const void* text_feats, const void* vis_feats
   const long long D = g.D, Dh = g.Dh, dp = g.dp, Tv = static_cast<long long>(B) * N, Tt = total_m;
   CU_TRY(cudaSetDevice(c->device));
   MAP_TRY(ensure_rope(c, g.rope_on ? N + max_m + 1 : 1));
-  // the staged rows are 64 to a block of the elementwise kernels' grids
+  // the most rows a training step takes (the elementwise kernels' grids, 64 rows a block, hold twice that)
   if ((std::max(Tv, Tt) + 31) / 32 > 65535) return MAP_EUNSUPPORTED;
   // question offsets and positions N + m (as for map_score)
   MAP_TRY(ensure(c->qoff, static_cast<size_t>(3 * B + 1) * 4));
