@@ -888,7 +888,8 @@ __global__ void __launch_bounds__(kRgThreads) sel_resgram_kernel(SelState s) {
 // coordinates in registers, moved there eight at a time, and in a shared row that the others
 // read by 16-byte broadcasts when it wins; the residual it publishes becomes the winner's 1 / r
 // beside the dot product.  The picks take one block barrier each: the winning slot is carried in
-// the low bits of the key.  At most kRoundPicks picks per launch (the next round continues):
+// the low bits of the key, and after the barrier a step writes no row and no residual that it reads of
+// another slot (only the remaining candidates write theirs).  At most kRoundPicks picks per launch (the next round continues):
 // the triangle leaves room for 88 coordinates a slot.  Bound by the chain of dependent
 // instructions of a pick (two reductions of keys, the barrier, the dot product: about 930 cycles,
 // 0.45 us; two slots a thread were slower, 1860 cycles, as were a branch per eight coordinates,
@@ -1039,10 +1040,14 @@ __global__ void __launch_bounds__(kActiveSlots, 1) sel_greedy_kernel(SelState s)
           }
       }
       const float e = (gji - ((sum2(a0) + sum2(a1)) + (sum2(a2) + sum2(a3)))) * rinv;
-      me[nr] = e;
       r2 = fmaf(-e, e, r2);
       const bool pos = r2 > floor2;                  // floor2 >= 0: the basis can be extended
-      pub[slot] = pos ? r2 : -1.f;
+      // Candidates only: the other warps may still read the winner's residual and row in this step (one
+      // barrier a pick), and its new residual, about zero, would read as degenerate.
+      if (alive) {
+        me[nr] = e;
+        pub[slot] = pos ? r2 : -1.f;
+      }
       if (lam1) val = pos ? fmaxf((pv * pv) * r2, 0.f) : 0.f;
       else val = sel_value(pv, r2, sq, s.lambda, s.tau);
       vkey = __float_as_uint(val);

@@ -484,3 +484,34 @@ def test_prune_of_device_buffers_equals_its_stages(D, K, lam):
     ctx.check()
     assert torch.equal(keep, want)
     assert torch.equal(out, torch.gather(vis, 1, want.long()[:, :, None].expand(-1, -1, D)))
+
+
+@pytest.mark.parametrize("case,repeats", [("one image, k = 160", 300), ("k = 640", 100), ("ragged", 200)])
+def test_selections_repeat_bit_for_bit(case, repeats):
+    """The same selection again and again gives the same pick order: nothing in it may depend on
+    which warp or block runs first."""
+    K = {"one image, k = 160": 160, "k = 640": 640, "ragged": 128}[case]
+    nv = None
+    if case == "ragged":
+        wl = W.RAGGED_WORKLOADS["c5"]
+        vis, _, _, nv = W.make_ragged_batch(wl, threads=8)
+    else:
+        wl = W.WORKLOADS["c1"]
+        vis = np.stack([W.make_image(wl, b) for b in range(1 if K == 160 else 2)])
+    B, N, D = vis.shape
+    ctx, _ = make_ctx(W.PredictorDims(D=D, Dh=256, dp=64))
+    rng = np.random.default_rng(K)
+    p32 = np.zeros((B, N), np.float32)
+    for b in range(B):
+        n = N if nv is None else int(nv[b])
+        p32[b, :n] = rng.dirichlet(np.full(n, 0.3))
+    p, v = torch.from_numpy(p32).to(DEV), dev_bits(vis)
+
+    def once():
+        return ctx.select(p, v, K) if nv is None else ctx.select_ragged(p, v, nv, K)
+
+    keep, order = once()
+    others = [once() for _ in range(repeats)]
+    torch.cuda.synchronize()
+    ctx.check()
+    assert all(torch.equal(o, order) and torch.equal(k, keep) for k, o in others)

@@ -148,3 +148,26 @@ def test_ragged_scores_equal_each_image_alone(N, nv):
         torch.testing.assert_close(got[b, :n], alone[0], rtol=2e-6, atol=0)
         assert not got[b, n:].any()
     ctx.check()
+
+
+@pytest.mark.parametrize("seed", [1, 2, 3, 4])
+def test_ragged_selection_matches_the_oracle_on_every_image(seed):
+    """16 variable-resolution images of up to 1280 tokens, 128 kept, scores shaped like Eq. 3's (means of
+    softmaxes over each image's own tokens): the picks of all of them against the oracle replay."""
+    wl = W.RaggedWorkload("seeded", 100 + seed, 16, 1280, 512, 512, 64, 0.3, 16, 128, 128)
+    vis, _, _, nv = W.make_ragged_batch(wl, threads=8)
+    ctx, _ = make_ctx(W.PredictorDims(D=512, Dh=256, dp=64))
+    rng = np.random.default_rng(seed)
+    p32 = np.zeros(vis.shape[:2], np.float32)
+    for b, n in enumerate(nv):
+        z = O.bf16_bits_to_f64(vis[b, :n]) @ rng.standard_normal((512, 48)) * (2.0 / np.sqrt(1.09 * 512))
+        z = np.exp(z - z.max(axis=0))
+        p32[b, :n] = (z / z.sum(axis=0)).mean(axis=1)
+    keep, order = ctx.select_ragged(torch.from_numpy(p32).to(DEV), dev_bits(vis), nv, 128)
+    torch.cuda.synchronize()
+    ctx.check()
+    keep, order = keep.cpu().numpy(), order.cpu().numpy()
+    for b, n in enumerate(nv):
+        rep = P.check_selection(p32[b, :n].astype(np.float64), O.bf16_bits_to_f64(vis[b, :n]), 128, O.resolve_k0(128),
+                                order[b], keep[b])
+        assert rep["ok"], f"image {b}: {rep['reason']}"
