@@ -19,7 +19,13 @@
 //               release the accumulator so the
 //               MMA warp can start the tile after next while this one drains.
 //   EPI_PROJECT: the MMA thread also accumulates A A^T (N = 128) of every stage into a second
-//               TMEM accumulator, whose diagonal is ||row||^2.
+//               TMEM accumulator, whose diagonal is ||row||^2.  K is taken in kGramSlices slices,
+//               an accumulator each (two, alternating).  Warps 6-9 add them in slice order, the Gram
+//               kernel's, in registers and hand a tile's sums to the epilogue warps in a third TMEM
+//               region, so that the substitution of one tile runs beside the products of the next.
+//               (With the additions in the epilogue warps themselves the MMAs waited for the
+//               substitution: calls on 64 images of 2880 tokens took 6 % longer than with one
+//               accumulation over K, this way 0.7 %, on one image 2 %.)
 // All waits are bounded (ptx.cuh); a timeout sets ST_TIMEOUT and every role drains and exits.
 #include <algorithm>
 #include <cstdio>
@@ -87,7 +93,9 @@ struct Smem {
   static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr uint32_t TILES = STAGES * STAGE_BYTES;
   static constexpr bool EGSYNC = PROJ || EPI == EPI_SM_MEAN;   // epilogue warps' group barrier
-  static constexpr uint32_t BARS = (2 * STAGES + 5 + (EGSYNC ? 1 : 0)) * 8;
+  // PROJ: also dempty, sfull and sempty, and one unused: L, which follows, is read 16 bytes at a time
+  static constexpr uint32_t XBARS = (EGSYNC ? 1 : 0) + (PROJ ? 4 : 0);
+  static constexpr uint32_t BARS = (2 * STAGES + 5 + XBARS) * 8;
   // per-warp 32x32 transposes (EPI_SM_STATS) or the tile's column normalisers (EPI_SM_MEAN)
   static constexpr uint32_t XPOSE = EPI == EPI_SM_STATS ? 4 * 32 * 33 * 4 : (EPI == EPI_SM_MEAN ? BN * 4 : 0);
   // bf16 outputs written by TMA box stores from per-warp staging: hi/lo split epilogues use two
@@ -98,11 +106,12 @@ struct Smem {
   static constexpr bool TSTORE_F32 = EPI == EPI_F32;
   static constexpr uint32_t STG = TSTORE || TSTORE_F32 ? 4 * 4 * 32 * 32 * 2 : 0;
   static constexpr uint32_t LSM = PROJ ? BN * BN * 4 : 0;       // L rows of the basis (pitch BN)
-  static constexpr uint32_t PEXTRA = PROJ ? BN * 4 : 0;          // 1/r of the basis
+  static constexpr uint32_t PEXTRA = PROJ ? (BN + kBM) * 4 : 0;  // 1/r of the basis, ||row||^2 of the tile
   static constexpr uint32_t TOTAL = 1024 + TILES + STG + BARS + 16 + XPOSE + LSM + PEXTRA;
-  static constexpr uint32_t TMEM_COLS =                           // a power of two; PROJ: + A A^T
-      PROJ ? (2 * BN + 2 * kBM <= 256 ? 256u : 512u) : (2 * BN > 256 ? 512u : 2 * BN);
-  static constexpr int THREADS = 192;
+  static constexpr uint32_t TMEM_COLS =                           // a power of two; PROJ: + the sums, A A^T
+      PROJ ? (3 * BN + kBM <= 256 ? 256u : 512u) : (2 * BN > 256 ? 512u : 2 * BN);
+  static constexpr int THREADS = PROJ ? 320 : 192;
+  static_assert(!PROJ || (TILES + STG + BARS + 16 + XPOSE) % 16 == 0, "float4 reads of L");
 };
 
 // Selection value, squared: p^2 * rho^(2 lambda) orders candidates like p * rho^lambda (both are
@@ -243,12 +252,16 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
   uint64_t* tfull = empty + STAGES;
   uint64_t* tempty = tfull + 2;
   uint64_t* drain = tempty + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1 + (S::EGSYNC ? 1 : 0));
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1 + S::XBARS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint64_t* egsync = drain + 1;                  // EGSYNC: epilogue warps' group barrier
+  uint64_t* dempty = drain + 2;                  // PROJ: A A^T has been read; the tile's sums are written; read
+  uint64_t* sfull = drain + 3;
+  uint64_t* sempty = drain + 4;
   float* xpose = reinterpret_cast<float*>(smem + S::TILES + S::STG + S::BARS + 16);
   float* Lsm = xpose + S::XPOSE / 4;
   float* rinv_sm = Lsm + S::LSM / 4;
+  float* sq_sm = rinv_sm + BN;                   // PROJ
 
   // uniform in the warp, and known to be
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -259,6 +272,11 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
     mbar_init(drain, 1);
     if constexpr (S::EGSYNC) {
       mbar_init(egsync, 128);
+    }
+    if constexpr (S::PROJ) {                       // an arrive per warp
+      mbar_init(dempty, 4);
+      mbar_init(sfull, 4);
+      mbar_init(sempty, 4);
     }
     *abort_flag = 0;
     fence_mbar_init();
@@ -299,6 +317,7 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
     else return tile_coord<PAIR, EPI == EPI_PROJECT>(a, t, nbatch, m_units, n_tiles, BN, crank);
   };
   constexpr bool PRODUCTS = EPI == EPI_F32;       // the epilogue of the segmented products
+  constexpr int SLICES = S::PROJ ? kGramSlices : 1;   // accumulators per tile, one after the other
   // K blocks of one product of image c.b
   auto product_kblocks = [&](const TileCoord& c) {
     return a.pr.k_count ? (__ldg(a.pr.k_count + c.b) + kBK - 1) / kBK : a.pr.kblocks;
@@ -428,6 +447,7 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
     if (crank == 0 && elect_one()) {
       // ---------------------------------------------------------------- MMA issuer (CG2: leader)
       uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
+      [[maybe_unused]] uint32_t d_phase = 0;
       bool issued = false, ok = true;
       // descriptors without their address (shared memory addresses are below 2^18); products: also
       // their step per 16 K: 32 bytes along a K-major row, 16 rows of 128 bytes of an MN-major box
@@ -439,50 +459,63 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
       for (int t = unit0; t < total && ok; t += units_step) {
         TileCoord c = coord(t);
         if (c.skip) continue;
-        if (!mbar_wait(&tempty[acc], acc_phase ^ 1, a.status, abort_flag, a.wait_ns)) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * BN;
-        int kb0, kb1;
-        kb_range(c, kb0, kb1);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(&full[stage], phase, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t a0 = smem_u32(sA + stage * S::A_BYTES);
-          const uint32_t b0 = smem_u32(sB + stage * S::B_BYTES);
-          if (PRODUCTS && a.pr.n > 0) {
-#pragma unroll
-            for (int k = 0; k < kBK / 16; ++k) {
-              const uint64_t da = adesc0 + (a0 >> 4) + k * astep, db = bdesc0 + (b0 >> 4) + k * bstep;
-              if constexpr (CG2) umma_bf16_cg2(d_tmem, da, db, pid, (kb != kb0 || k != 0));
-              else umma_bf16(d_tmem, da, db, pid, (kb != kb0 || k != 0));
-            }
-            if constexpr (CG2) umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
-            else umma_commit(&empty[stage]);
-          } else if constexpr (CG2) {
-            const uint64_t da = kdesc0 + (a0 >> 4), db = kdesc0 + (b0 >> 4);
-#pragma unroll
-            for (int k = 0; k < kBK / 16; ++k) umma_bf16_cg2(d_tmem, da + 2 * k, db + 2 * k, IDESC, (kb != kb0 || k != 0));
-            umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
-          } else {
-            const uint64_t da = kdesc0 + (a0 >> 4), db = kdesc0 + (b0 >> 4);
-#pragma unroll
-            for (int k = 0; k < kBK / 16; ++k) umma_bf16(d_tmem, da + 2 * k, db + 2 * k, IDESC, (kb != kb0 || k != 0));
-            if constexpr (S::PROJ) {   // A A^T: its diagonal is ||row||^2
-              const uint32_t n_tmem = tmem_base + 2 * BN + acc * kBM;
-#pragma unroll
-              for (int k = 0; k < kBK / 16; ++k)
-                umma_bf16(n_tmem, da + 2 * k, da + 2 * k, idesc_bf16(kBM, kBM), (kb != kb0 || k != 0));
-            }
-            umma_commit(&empty[stage]);
+        for (int sl = 0; sl < SLICES; ++sl) {
+          int kb0, kb1;
+          kb_range(c, kb0, kb1);
+          if constexpr (S::PROJ) {
+            kb0 = sl * (a.K / kBK) / kGramSlices;
+            kb1 = (sl + 1) * (a.K / kBK) / kGramSlices;
+            if (kb0 == kb1) continue;                // fewer K blocks than slices
           }
-          issued = true;
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
+          if (!mbar_wait(&tempty[acc], acc_phase ^ 1, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t d_tmem = tmem_base + acc * BN;
+          for (int kb = kb0; kb < kb1; ++kb) {
+            if (!mbar_wait(&full[stage], phase, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t a0 = smem_u32(sA + stage * S::A_BYTES);
+            const uint32_t b0 = smem_u32(sB + stage * S::B_BYTES);
+            if (PRODUCTS && a.pr.n > 0) {
+#pragma unroll
+              for (int k = 0; k < kBK / 16; ++k) {
+                const uint64_t da = adesc0 + (a0 >> 4) + k * astep, db = bdesc0 + (b0 >> 4) + k * bstep;
+                if constexpr (CG2) umma_bf16_cg2(d_tmem, da, db, pid, (kb != kb0 || k != 0));
+                else umma_bf16(d_tmem, da, db, pid, (kb != kb0 || k != 0));
+              }
+              if constexpr (CG2) umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
+              else umma_commit(&empty[stage]);
+            } else if constexpr (CG2) {
+              const uint64_t da = kdesc0 + (a0 >> 4), db = kdesc0 + (b0 >> 4);
+#pragma unroll
+              for (int k = 0; k < kBK / 16; ++k) umma_bf16_cg2(d_tmem, da + 2 * k, db + 2 * k, IDESC, (kb != kb0 || k != 0));
+              umma_commit_cg2_mc(&empty[stage], static_cast<uint16_t>(3));
+            } else {
+              const uint64_t da = kdesc0 + (a0 >> 4), db = kdesc0 + (b0 >> 4);
+#pragma unroll
+              for (int k = 0; k < kBK / 16; ++k) umma_bf16(d_tmem, da + 2 * k, db + 2 * k, IDESC, (kb != kb0 || k != 0));
+              issued = true;
+              if constexpr (S::PROJ) {   // A A^T: its diagonal is ||row||^2
+                if (kb == kb0) {         // the previous slice's has been read
+                  if (!mbar_wait(dempty, d_phase ^ 1, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
+                  tc_fence_after();
+                  d_phase ^= 1;
+                }
+                const uint32_t n_tmem = tmem_base + 3 * BN;
+#pragma unroll
+                for (int k = 0; k < kBK / 16; ++k)
+                  umma_bf16(n_tmem, da + 2 * k, da + 2 * k, idesc_bf16(kBM, kBM), (kb != kb0 || k != 0));
+              }
+              umma_commit(&empty[stage]);
+            }
+            issued = true;
+            if (++stage == STAGES) { stage = 0; phase ^= 1; }
+          }
+          if (!ok) break;
+          if constexpr (CG2) umma_commit_cg2_mc(&tfull[acc], static_cast<uint16_t>(3));
+          else umma_commit(&tfull[acc]);
+          acc ^= 1;
+          if (acc == 0) acc_phase ^= 1;
         }
-        if (!ok) break;
-        if constexpr (CG2) umma_commit_cg2_mc(&tfull[acc], static_cast<uint16_t>(3));
-        else umma_commit(&tfull[acc]);
-        acc ^= 1;
-        if (acc == 0) acc_phase ^= 1;
       }
       if (issued) {   // every MMA of this CTA has completed before TMEM is released
         if constexpr (CG2) umma_commit_cg2(drain);
@@ -595,9 +628,11 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
         rt = a.rope + pos;
         load_rope(0);
       }
-      if (!mbar_wait(&tfull[acc], acc_phase, a.status, abort_flag, a.wait_ns)) break;
+      // EPI_PROJECT: the tile's sums, in their own region
+      if (!mbar_wait(S::PROJ ? sfull : &tfull[acc], acc_phase, a.status, abort_flag, a.wait_ns)) break;
       tc_fence_after();
-      const uint32_t tbase = tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + acc * BN;
+      const uint32_t tbase =
+          tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + (S::PROJ ? 2 * BN : acc * BN);
       const long long crow = static_cast<long long>(c.b) * a.c_batch_stride + static_cast<long long>(row) * a.ldc;
 
       if constexpr (EPI == EPI_ROPE_F32) {
@@ -811,13 +846,7 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
         const long long tok = static_cast<long long>(c.b) * a.M + row;
         const bool alive = row_ok && __ldg(pj.state + tok) == 0;
         float* erow = pj.Ec + tok * pj.KP;
-        float sq = 0.f;
-        {
-          uint32_t dg[32];
-          tmem_ld32(tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16) + 2 * BN + acc * kBM + lane_grp * 32, dg);
-#pragma unroll
-          for (int j = 0; j < 32; ++j) sq = j == lane ? __uint_as_float(dg[j]) : sq;
-        }
+        const float sq = sq_sm[r_in_tile];
         float r2 = sq;
 #pragma unroll 1
         for (int b0 = 0; b0 < nb0; b0 += 32) {
@@ -1022,14 +1051,81 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
       __syncwarp();
       if (lane == 0) {
         if constexpr (CG2) mbar_arrive_cluster(mapa_u32(&tempty[acc], 0));
-        else mbar_arrive(&tempty[acc]);
+        else mbar_arrive(S::PROJ ? sempty : &tempty[acc]);
       }
-      acc ^= 1;
-      if (acc == 0) acc_phase ^= 1;
+      if constexpr (S::PROJ) {
+        acc_phase ^= 1;
+      } else {
+        acc ^= 1;
+        if (acc == 0) acc_phase ^= 1;
+      }
     }
     if constexpr (S::TSTORE || S::TSTORE_F32) {
       if (lane == 0) bulk_wait_group_all();              // every box store has completed
       __syncwarp();
+    }
+  } else if constexpr (S::PROJ) {
+    // ------------------------------------------------------------------ K slices' sums
+    const int lane_grp = warp & 3;
+    const uint32_t lanes = tmem_base + (static_cast<uint32_t>(lane_grp * 32) << 16);
+    const int slices = min(SLICES, a.K / kBK);     // those with K blocks
+    uint32_t acc = 0, acc_phase = 0, s_phase = 0;
+    bool ok = true;
+    for (int t = unit0; t < total && ok; t += units_step) {
+      TileCoord c = coord(t);
+      if (c.skip) continue;
+      const int nb0 = min(BN, __ldg(a.proj.nbasis + c.b));
+      float sum[BN], sq = 0.f;
+#pragma unroll
+      for (int j = 0; j < BN; ++j) sum[j] = 0.f;
+#pragma unroll 1
+      for (int sl = 0; sl < slices; ++sl) {
+        if (!mbar_wait(&tfull[acc], acc_phase, a.status, abort_flag, a.wait_ns)) { ok = false; break; }
+        tc_fence_after();
+        float d = 0.f;                             // this row's diagonal element of A A^T
+#pragma unroll
+        for (int h = 0; h < 32; h += 16) {
+          uint32_t r[16];
+          tmem_ld16(lanes + 3 * BN + lane_grp * 32 + h, r);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) d = h + j == lane ? __uint_as_float(r[j]) : d;
+        }
+        sq += d;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(dempty);
+#pragma unroll
+        for (int ch = 0; ch < BN / 32; ++ch) {
+          if (ch * 32 >= nb0) break;               // uniform
+#pragma unroll
+          for (int h = 0; h < 32; h += 16) {       // 16 at a time: 128 sums leave room for no more
+            uint32_t r[16];
+            tmem_ld16(lanes + acc * BN + ch * 32 + h, r);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) sum[ch * 32 + h + j] += __uint_as_float(r[j]);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[acc]);
+        acc ^= 1;
+        if (acc == 0) acc_phase ^= 1;
+      }
+      if (!ok || !mbar_wait(sempty, s_phase ^ 1, a.status, abort_flag, a.wait_ns)) break;
+      tc_fence_after();
+#pragma unroll
+      for (int ch = 0; ch < BN / 32; ++ch) {
+        if (ch * 32 >= nb0) break;                 // uniform
+        uint32_t r[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(sum[ch * 32 + j]);
+        tmem_st32(lanes + 2 * BN + ch * 32, r);
+      }
+      sq_sm[lane_grp * 32 + lane] = sq;
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sfull);
+      s_phase ^= 1;
     }
   }
   // Every role of this CTA has left its loop.  If one gave up (a bounded wait ran out), loads

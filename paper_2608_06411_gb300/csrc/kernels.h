@@ -5,6 +5,14 @@
 
 namespace mapk {
 
+// Products of two tokens' features (selection) are fp32 sums of this many K slices, slice s the 64-column
+// blocks s KB / kGramSlices ..., added in slice order: in the Gram kernel, where a CTA of the cluster takes a slice,
+// and in EPI_PROJECT alike.  What is subtracted from or divided by each other (a Gram entry and the norms
+// it meets) must be the same sum: the tensor cores lose up to an ulp a 16-term step, so two orders differ
+// by about 5e-6 of ||v||^2 at 4096 columns and more than tau = 1e-5 beyond 8192, where an exact copy of a
+// retained token then counted as independent.
+constexpr int kGramSlices = 8;
+
 // *_SPLIT epilogues store an fp32 activation x as two bf16 halves, hi = bf16(x) at
 // column c and lo = bf16(x - hi) at column N + c of a [rows, 2N] buffer, so that the next
 // layer can consume ~16 significant bits through a bf16 GEMM: [hi | lo] @ [W | W]^T.
@@ -16,7 +24,7 @@ namespace mapk {
 // visual tokens, columns = question tokens): per-column max / sum of exp over each
 // 32-row slab, then per-row mean over columns of exp(l - max) / sum.
 // EPI_PROJECT: rows = visual tokens, columns = the R0 basis tokens' rows (Gram entries
-// <v_n, v_r>); the epilogue solves for the tokens' Cholesky coordinates against the R0
+// <v_n, v_r>, sums of K slices); the epilogue solves for the tokens' Cholesky coordinates against the R0
 // basis (L staged in shared memory); ||v_n||^2 is the diagonal of an A A^T product that the
 // MMA thread accumulates from the same shared-memory tiles.  It writes the exact residual,
 // value and coordinate cache of every candidate token (see select.cu).

@@ -24,7 +24,7 @@
 namespace mapk {
 namespace {
 
-constexpr int kRanks = 8;                            // CTAs of a cluster
+constexpr int kRanks = kGramSlices;                  // CTAs of a cluster, a K slice each
 constexpr int kThreads = 256;
 constexpr int kTileRows = 128;
 constexpr int kKb = 64;                              // columns of a stage

@@ -515,3 +515,22 @@ def test_selections_repeat_bit_for_bit(case, repeats):
     torch.cuda.synchronize()
     ctx.check()
     assert all(torch.equal(o, order) and torch.equal(k, keep) for k, o in others)
+
+
+@pytest.mark.parametrize("D", [1024, 4096, 8192, 12288])
+@pytest.mark.parametrize("distinct,K0", [(40, 40), (100, 100), (40, 10), (40, 0), (200, 200)])
+def test_exact_copies_of_retained_tokens_have_no_value(D, distinct, K0):
+    """Once every distinct token is retained, all that is left are exact copies: each has no residual
+    (below tau = 1e-5 of its norm), so they follow in index order, whatever their scores.  The norms, the
+    projection's products and the Gram blocks must be the same sums for that: two orders of summing the products
+    differ by more than tau.  Copies of factored R0 tokens, of later picks and of both."""
+    ctx, _ = make_ctx(W.PredictorDims(D=D, Dh=256, dp=64), k0_abs=K0)
+    N, K = 600, 2 * distinct
+    rng = np.random.default_rng(D + distinct + K0)
+    base = rng.standard_normal((distinct, D)).astype(np.float32)
+    vis = W.f32_to_bf16_bits(base[np.concatenate([np.arange(distinct), rng.integers(0, distinct, N - distinct)])])[None]
+    p32 = np.empty((1, N), np.float32)
+    p32[0, :distinct] = rng.uniform(0.5, 1.0, distinct)
+    p32[0, distinct:] = rng.uniform(0.3, 0.45, N - distinct)
+    _, order = run_select(ctx, p32, vis, K)
+    np.testing.assert_array_equal(order[0, distinct:], np.arange(distinct, K))
