@@ -938,6 +938,7 @@ gemm_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ KArgs 
             // N: written row by row from the lanes, a store instruction touches 32 rows, and a tile
             // took 6.8 us where this takes 2.5 us (the step of
             // 4 samples of 2880 tokens: 736 -> 699 us, 2 of 576: 245 -> 224 us)
+            // (a tile stores an even number of chunks, so the two buffers alternate across tiles too)
             uint8_t* sb = stg + (ew * 2 + (ch & 1)) * 4096;
             if (lane == 0) bulk_wait_group_read<1>();    // this buffer's previous store has read it
             __syncwarp();
@@ -1170,13 +1171,6 @@ bool make_map(CUtensorMap* m, const void* base, long long rows, int K, int box_r
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
-}
-
-// EPI_F32 results that box stores can write: every batch entry's (or K slice's) rows and columns end at
-// M and N, at a fixed distance from the next one's.
-bool f32_box_store(const GemmDesc& d) {
-  return d.epi == EPI_F32 && (d.batch == 1 || d.ksplit == 1) && !d.n_limit && !d.m_limit && !d.blist &&
-         (!d.pr.a_off || d.pr.a_mn);
 }
 
 // Tensor maps of one row group.

@@ -115,6 +115,15 @@ struct GemmDesc {
   const int* seg_valid = nullptr; int seg_len = 0;
 };
 
+// EPI_F32 results that box stores can write: every batch entry's (or K slice's) rows and columns end at
+// M and N, at a fixed distance from the next one's.  N % 64 == 0: a warp's two staging buffers take the
+// 32-column chunks of a tile in turn, from the first one in every tile, and a chunk waits for all stores but the
+// last; after a tile of an odd number of chunks that last one might still read the buffer.
+inline bool f32_box_store(const GemmDesc& d) {
+  return d.epi == EPI_F32 && d.N % 64 == 0 && (d.batch == 1 || d.ksplit == 1) && !d.n_limit && !d.m_limit &&
+         !d.blist && (!d.pr.a_off || d.pr.a_mn);
+}
+
 // tile_n of the first layer of both branches (m_vis and m_text rows, N columns).
 int predictor_tile_width(long long m_vis, long long m_text, int N, int K, int num_sms);
 // Returns cudaSuccess, or an error for an unsupported shape (cudaErrorInvalidValue).
