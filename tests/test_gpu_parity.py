@@ -534,3 +534,27 @@ def test_exact_copies_of_retained_tokens_have_no_value(D, distinct, K0):
     p32[0, distinct:] = rng.uniform(0.3, 0.45, N - distinct)
     _, order = run_select(ctx, p32, vis, K)
     np.testing.assert_array_equal(order[0, distinct:], np.arange(distinct, K))
+
+
+def test_scores_of_short_questions_ignore_what_an_earlier_batch_left():
+    """A batch with questions above and below 256 tokens, after one on the same context in which every
+    image fills all column tiles: the tiles that a short question does not reach still hold the earlier
+    batch's sums and must not be added."""
+    dims = W.PredictorDims(D=256, Dh=256, dp=64)
+    ctx, _ = make_ctx(dims, seed=21, bias_std=0.1)
+    wl, B, N = W.WORKLOADS["c0"], 4, 200
+    vis = dev_bits(np.stack([W.make_image(wl, b, N=N, D=dims.D) for b in range(B)]))
+
+    def score(lens, first=0, count=B):
+        text = np.concatenate([W.make_text(wl, first + i, m, D=dims.D) for i, m in enumerate(lens)])
+        return ctx.score(dev_bits(text), vis[first:first + count], np.array(lens, np.int32)).clone()
+
+    full = score([600, 520, 540, 770])                    # three column tiles of 256 questions
+    lens = [17, 600, 256, 257]
+    mixed = score(lens)
+    alone = [score([m], b, 1)[0] for b, m in enumerate(lens)]
+    torch.cuda.synchronize()
+    ctx.check()
+    assert float(full.min()) > 0.0
+    for b in range(B):
+        assert torch.equal(mixed[b], alone[b]), b
