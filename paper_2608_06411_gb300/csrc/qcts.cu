@@ -46,6 +46,7 @@ struct QctsMeta {
   int32_t order[kMaxSamples];    // samples of this launch, most rows first
   long long row0[kMaxSamples];   // first row (of N elements) of each sample's question block
 };
+static_assert(sizeof(QctsMeta) + 7 * sizeof(void*) <= 32764, "a kernel's parameters: at most 32764 bytes");
 
 __device__ __forceinline__ float low_bf16(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float high_bf16(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
@@ -333,7 +334,7 @@ extern "C" int map_qcts(const void* attn, const int32_t* lens, const void* attn_
 
   // samples per launch: the parameter table, and at most 65535 rows of the finish grid
   const int per_launch = std::max(1, std::min(kMaxSamples, 65535 / L));
-  std::unique_ptr<QctsMeta> mp(new (std::nothrow) QctsMeta);   // ~12 KB, copied into the launch parameters
+  std::unique_ptr<QctsMeta> mp(new (std::nothrow) QctsMeta);   // 16 KB, copied into the launch parameters
   if (!mp) return MAP_ENOMEM;
   QctsMeta& m = *mp;
   long long row = 0;
