@@ -35,6 +35,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "newton.cuh"
 #include "ptx.cuh"
 #include "select.h"
 
@@ -65,13 +66,6 @@ __device__ __forceinline__ float sel_value(float p, float r2, float sq, float la
   if (!(r2 > tau * sq) || !(r2 > 0.f)) return 0.f;
   const float v = lam == 1.f ? (p * p) * r2 : (p * p) * powf(r2, lam);
   return v > 0.f ? v : 0.f;
-}
-
-// 1 / sqrt(x), x > 0: the hardware estimate (2 ulp) and one Newton step (below 1 ulp, like the
-// quotient of a rounded root), without the branches of an IEEE root and division.
-__device__ __forceinline__ float inv_sqrt(float x) {
-  const float y = rsqrtf(x), t = x * y;
-  return x < INFINITY ? fmaf(0.5f * y, fmaf(-t, y, 1.0f), y) : 0.f;
 }
 
 // Two fp32 fused multiply-adds in one instruction (the halves of a 64-bit register pair).
@@ -367,8 +361,8 @@ __host__ __device__ inline int coord_pitch(int KP) { return ((KP + 7) / 8) * 8 +
 // 16-column block with 4 slots x 4 rows per thread, then each thread adds the eight partial
 // products of two entries.  Warp 0 solves the chunk's 32 x 32 triangle right-looking (lane = slot:
 // each new coordinate is subtracted from the later ones at once), dividing by the basis norm as a
-// product with its reciprocal and one correction step (the quotient to the last bit or nearly so,
-// without the division's chain in every step), while the other warps copy the next chunk's L rows,
+// product with its reciprocal and one correction step (newton.cuh: without the division's chain in every
+// step), while the other warps copy the next chunk's L rows,
 // triangle, Gram entries and basis norms into shared memory (cp.async), so that no chunk waits for
 // a global load.  Writes Ec, r2 and cstep = nb.
 // k = 640 of 2880, 2 images, a round at 560 vectors: 90 us with the triangle's 32 steps unrolled and
@@ -503,9 +497,7 @@ __global__ void __launch_bounds__(32 * kUpdWarps) sel_update_kernel(SelState s) 
         for (int u = 0; u < 8; ++u) {
           const float ri = __shfl_sync(0xffffffffu, my_inv, t0 + u), rr = __shfl_sync(0xffffffffu, my_rn, t0 + u);
           const bool fresh = b0 + t0 + u >= mc0 && t0 + u < nch;   // past nb: e = 0
-          float e = av[u] * ri;
-          e = fmaf(fmaf(-e, rr, av[u]), ri, e);
-          e = fresh ? e : old[u];
+          const float e = fresh ? quotient(av[u], rr, ri) : old[u];
           r2 = fresh ? fmaf(-e, e, r2) : r2;
           ev[u] = e;
 #pragma unroll
