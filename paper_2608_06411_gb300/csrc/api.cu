@@ -22,7 +22,7 @@ constexpr int kMaxKDiverse = 768;   // k limit when the diversity term is on (th
                                     // stages slot rows and 32 basis rows of k floats in shared memory)
 constexpr int kProjMaxBasis = 128;  // basis vectors one projection pass takes
 constexpr int kMaxK = 4096;
-constexpr int kCombineInTile = 32;  // most 32-row slabs whose softmax statistics every tile combines itself
+constexpr int kCombineInTile = 28;  // most softmax statistics a thread combines in Eq. 3's second pass itself
 constexpr int kMaxN = 16384;
 
 struct DevBuf {
@@ -352,10 +352,14 @@ int score_impl(map_ctx* c, const void* text, const void* vis, const int32_t* len
     d.C = part; d.ldc = 4; d.c_batch_stride = 0;
     MAP_TRY(gemm(c, d, st));
     d.epi = mapk::EPI_SM_MEAN;
-    if (nparts <= kCombineInTile && static_cast<long long>(B) * m_tiles * n_tiles <= c->num_sms) {
-      // one tile a CTA and few slabs: each tile combines its columns' partial statistics itself while
-      // its MMAs run, a launch less (N = 576: 165 -> 159 us per call, with the selection's merged
-      // set-up launches); with 92 slabs (N = 2880) it took longer than the launch
+    // One tile a CTA and few statistics: each tile combines its columns' slabs itself while its MMAs run, a
+    // launch less.  128 threads take up to 256 columns, so a thread reads the slabs of one column or two, in
+    // sequence.  Calls with a launch of its own against in the tile (D = 4096): 20 slabs (N = 576), up to 128
+    // question tokens, 155.3 -> 153.7 us, 16 images 249.0 -> 246.7; 24 slabs 154.7 -> 152.2; 32 slabs 157.0 ->
+    // 156.9 with 16 tokens, 158.8 -> 159.2 with 128; 36 slabs 160.4 -> 161.6.  Two columns: 8 slabs 158.5 -> 156.9,
+    // 20 slabs 157.3 -> 158.2, 32 slabs 162.4 -> 166.3.
+    const int per_thread = nparts * (max_m > 128 ? 2 : 1);
+    if (per_thread <= kCombineInTile && static_cast<long long>(B) * m_tiles * n_tiles <= c->num_sms) {
       d.stats = part; d.stat_parts = nparts;
     } else {
       ++c->counters.launches;
