@@ -120,7 +120,7 @@ int map_score(map_ctx *ctx, const void *text_feats, const void *vis_feats,
  * selects; built on the first call of a shape and workspace, then cached in the context), so
  * the host never waits for it.  A device-side failure (a bounded wait that ran out, or the
  * loop's iteration cap, set at the most rounds the selection can take:
- * k * (ceil(N / 256) + 1) + ceil(k / 128) + 64) is reported by map_status.
+ * k * (ceil(N / 256) + 1) + ceil(k / 88) + 64) is reported by map_status.
  */
 int map_select(map_ctx *ctx, const float *scores, const void *vis_feats, int B, int N,
                int k, int32_t *keep_idx, int32_t *pick_order, void *stream);
@@ -172,7 +172,8 @@ int map_assemble(map_ctx *ctx, const void *vis_feats, const int32_t *keep_idx,
  * + 8 B + small per-image counters, plus, when the diversity term is on (lambda > 0 and
  * K0 < k), 4 B*N*ceil4(k) + 2 B*R*D + 4 B*256*R with R = ceil16(256 + k).  A request
  * that does not fit returns MAP_EUNSUPPORTED and does nothing.  One LLaVA-NeXT image
- * (N = 2880, k = 160, D = 4096) needs about 6 MB.
+ * (N = 2880, k = 160, D = 4096) counts as about 6 MB.  (2 B*R*D of it is reserved and no longer
+ * written: the same requests fit as before.)
  * Unlike map_select, whose later rounds run as a device-side loop, it waits on the host
  * for bursts of selection rounds (it synchronises `stream`); a device-side error is
  * returned and also recorded for map_status.  It skips map_select's tensor-core
@@ -270,8 +271,10 @@ int map_assemble_ragged(map_ctx *ctx, const void *vis_feats, const int32_t *keep
  *   grads      float32 device outputs, each with its weight's shape (wT1 [Dh, D], bT1 [Dh],
  *              wT2 [Dh, Dh], bT2 [Dh], wQ [dp, Dh], and the same for V / K); overwritten.
  * fp32 arithmetic throughout (bf16 inputs decoded exactly); deterministic.  Workspace (about
- * 4 (B N + sum(lens)) (D + 5 Dh + 4 dp) + 4 sum(lens) N bytes) is owned by the context.
- * B N <= 2^24 and sum(lens) <= 2^24 (MAP_EUNSUPPORTED beyond).
+ * (B N + sum(lens)) (32 Dh + 20 dp) + 10 P N bytes, P the question tokens with each image's rounded up
+ * to 64, plus the K slices of contractions with few output tiles and a copy of features that are
+ * not 16-byte aligned) is owned by the context.
+ * B N <= 2097120 and sum(lens) <= 2097120 (MAP_EUNSUPPORTED beyond).
  */
 typedef struct {
     float *wT1, *bT1, *wT2, *bT2, *wQ;

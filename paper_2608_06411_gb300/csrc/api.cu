@@ -523,7 +523,9 @@ int select_impl(map_ctx* c, const float* scores, const void* vis, const int32_t*
         take_list(pd);
         return gemm(c, pd, st);
       };
-      // basis columns a projection on n vectors computes
+      // Basis columns a projection on n vectors computes: 32 for the smallest R0 (one image of 576 tokens,
+      // k = 32: 1.014 times faster than with 96).  64 for 33 to 64 vectors is not built; measured in a copy it took
+      // 184 -> 181 us for one image of 576 tokens and k = 96, 212 -> 210 us of 2880.
       auto proj_cols = [](int n) { return n <= 32 ? 32 : (n <= 96 ? 96 : kProjMaxBasis); };
       pd.N = proj_cols(K0c);
       MAP_TRY(project_all(true));

@@ -199,7 +199,7 @@ struct TcBatch {
   long long c_stride = 0;                            // C elements per entry (without a_off)
   long long c_rows = 0;                              // rows of C over the whole batch
 };
-// K slices launch_tc_matmul takes for an M x N output over K, and the floats its slices need.
+// K slices launch_tc_matmul takes for an M x N output over K.
 int tc_ksplit(int M, int N, int K, int products, int num_sms);
 int tc_products(bool a_split, bool b_split);
 // C[i, j] = sum_k A(i, k) B(j, k) on the tcgen05 GEMM, fp32 out, deterministic (fixed order).  With

@@ -148,8 +148,8 @@ extern "C" int map_select_noalloc(map_ctx* ctx, const float* scores, const void*
   s.aslot = cv.take<int32_t>(static_cast<size_t>(B) * S);
   if (K0 < K) {
     s.Ec = cv.take<float>(static_cast<size_t>(BN) * KP);
-    // no longer written (the Gram blocks read the features in place); still counted, so that the same
-    // calls fit the array as before
+    // no longer written (the Gram blocks read the features in place); still counted, because what fits
+    // is part of the interface (the formula in the header): callers plan with it
     cv.take<uint16_t>(static_cast<size_t>(B) * R * g.D);
     s.G = cv.take<float>(static_cast<size_t>(B) * S * R);
   }
