@@ -8,9 +8,8 @@ namespace mapk {
 // Products of two tokens' features (selection) are fp32 sums of this many K slices, slice s the 64-column
 // blocks s KB / kGramSlices ..., added in slice order: in the Gram kernel, where a CTA of the cluster takes a slice,
 // and in EPI_PROJECT alike.  What is subtracted from or divided by each other (a Gram entry and the norms
-// it meets) must be the same sum: the tensor cores lose up to an ulp a 16-term step, so two orders differ
-// by about 5e-6 of ||v||^2 at 4096 columns and more than tau = 1e-5 beyond 8192, where an exact copy of a
-// retained token then counted as independent.
+// it meets) must be the same sum: the tensor cores lose up to an ulp a 16-term step, and with two orders exact
+// copies of R0 tokens counted as independent (r^2 > tau ||v||^2) from 4096 columns on.
 constexpr int kGramSlices = 8;
 
 // *_SPLIT epilogues store an fp32 activation x as two bf16 halves, hi = bf16(x) at
